@@ -1,4 +1,4 @@
-// Shared host helpers and the generic list-ranking entry point.
+// Shared host helpers: memory, tuning parameters, status names.
 #include <atomic>
 #include <mutex>
 
@@ -135,21 +135,6 @@ extern "C" const char *etl_status_string(int32_t status) {
         case ETL_ETIMEOUT: return "ETL_ETIMEOUT";
         default: return "ETL_UNKNOWN";
     }
-}
-
-extern "C" etl_status etl_list_rank(const int32_t *succ, int64_t len, int32_t head, int32_t *rank, int32_t *status,
-                                    void *stream) {
-    if (!succ || !rank || len < 1 || len > int64_t(INT32_MAX) - 1 || head < 0 || head >= len) return ETL_EINVAL;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    Workspace ws(s);
-    int32_t *d_head = ws.get<int32_t>(1);
-    int32_t *st = status ? status : ws.get<int32_t>(1);
-    if (!ws.ok()) return ETL_ENOMEM;
-    etl_status rc = set_device_i32(d_head, head, s);
-    RankResult rr{};
-    if (!rc) rc = list_rank(succ, len, nullptr, d_head, false, len, st, ws, &rr);
-    if (!rc) rc = final_rank(rr, len, rank, s);
-    return rc;
 }
 
 extern "C" etl_status etl_tune_set(int32_t key, int32_t value) {

@@ -222,8 +222,9 @@ __global__ void k_arc_scatter(const int32_t *__restrict__ tuv, const int32_t *__
 
 // succ(twin(b)) := next(b) for every half-edge b at position i of B; half-edge
 // slots beyond the forest (and the virtual head, set later) are inert
+template <class S>
 __global__ void k_forest_succ(const int2 *__restrict__ B, const int32_t *__restrict__ d_len, int64_t cap,
-                              const int32_t *__restrict__ off, int32_t *__restrict__ succ) {
+                              const int32_t *__restrict__ off, typename S::T *__restrict__ succ) {
     pdl_prologue();
     const int64_t len = *d_len;
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < cap; i += int64_t(gridDim.x) * blockDim.x) {
@@ -233,9 +234,9 @@ __global__ void k_forest_succ(const int2 *__restrict__ B, const int32_t *__restr
             // entry of a group reads the group's start
             const int2 nx = i + 1 < len ? B[i + 1] : make_int2(-1, -1);
             const int32_t nb = nx.y == bx.y ? nx.x : B[off[bx.y]].x;
-            succ[bx.x ^ 1] = nb;
+            succ[bx.x ^ 1] = S::make(nb);
         } else {
-            succ[i] = ETL_END;
+            succ[i] = S::off_list();
         }
     }
 }
@@ -256,16 +257,18 @@ __global__ void k_root_list(int32_t n, const uint8_t *__restrict__ flag, const i
 
 // cut each component's cyclic tour in front of its root's first half-edge and
 // chain the components: virtual head -> comp 0 -> comp 1 -> ... -> end
+template <class S>
 __global__ void k_chain(int32_t n, const int32_t *__restrict__ rpos, const int32_t *__restrict__ roots,
                         const int2 *__restrict__ B, const int32_t *__restrict__ off, int32_t vhead,
-                        int32_t *__restrict__ succ) {
+                        typename S::T *__restrict__ succ) {
     pdl_prologue();
     const int32_t c = rpos[n];
-    if (blockIdx.x == 0 && threadIdx.x == 0) succ[vhead] = c > 0 ? B[off[roots[0]]].x : ETL_END;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        succ[vhead] = S::make(c > 0 ? B[off[roots[0]]].x : ETL_END);
     for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < c; k += int64_t(gridDim.x) * blockDim.x) {
         const int32_t r = roots[k];
         const int32_t tail = B[off[r + 1] - 1].x ^ 1;  // the half-edge whose successor was the head
-        succ[tail] = (k + 1 < c) ? B[off[roots[k + 1]]].x : ETL_END;
+        succ[tail] = S::make((k + 1 < c) ? B[off[roots[k + 1]]].x : ETL_END);
     }
 }
 
@@ -275,15 +278,13 @@ __global__ void k_forest_tin(RankResult rr, const int32_t *__restrict__ d_arcs, 
                              int32_t *__restrict__ etout) {
     pdl_prologue();
     const int64_t T = *d_arcs / 2;
-    const uint4 *pk = reinterpret_cast<const uint4 *>(rr.packed);
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < T; t += int64_t(gridDim.x) * blockDim.x) {
-        const uint4 q = pk[t];
-        if (q.x >= rr.rcap || q.z >= rr.rcap) {  // cannot happen for a forest built above; keep memory safe
+        const int32_t r0 = rank_at(rr, 2 * t), r1 = rank_at(rr, 2 * t + 1);
+        if (r0 < 0 || r1 < 0) {  // cannot happen for a forest built above; keep memory safe
             child[t] = 0;
             etin[t] = etout[t] = -1;
             continue;
         }
-        const int32_t r0 = rank_of(rr, make_uint2(q.x, q.y)), r1 = rank_of(rr, make_uint2(q.z, q.w));
         const int32_t c = r0 < r1 ? tuv[2 * t + 1] : tuv[2 * t];
         const int32_t a = min(r0, r1), b = max(r0, r1);
         tin[c] = a;
@@ -300,8 +301,8 @@ __global__ void k_root_tin(int32_t n, const int32_t *__restrict__ rpos, const in
     const int32_t c = rpos[n];
     for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < c; k += int64_t(gridDim.x) * blockDim.x) {
         const int32_t r = roots[k];
-        const uint2 p = rr.packed[B[off[r]].x];
-        tin[r] = p.x < rr.rcap ? rank_of(rr, p) - 1 : -1;
+        const int32_t p = rank_at(rr, B[off[r]].x);
+        tin[r] = p < 0 ? -1 : p - 1;
     }
 }
 
@@ -562,8 +563,9 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
     uint8_t *is_tree = ws.get<uint8_t>(m), *rflag = ws.get<uint8_t>(n);
     int32_t *tpos = ws.get<int32_t>(m + 1), *rpos = ws.get<int32_t>(int64_t(n) + 1), *roots = ws.get<int32_t>(n);
     int32_t *tuv = ws.get<int32_t>(A > 0 ? A : 1), *tedge = ws.get<int32_t>(n);
-    int32_t *n_arcs = ws.get<int32_t>(1), *vhead = ws.get<int32_t>(1), *giant = ws.get<int32_t>(1);
-    int32_t *succ = ws.get<int32_t>(N);
+    int32_t *n_arcs = ws.get<int32_t>(1), *giant = ws.get<int32_t>(1);
+    const bool wide = wide_slots(N);
+    void *succ = wide ? static_cast<void *>(ws.get<Slot8::T>(N)) : static_cast<void *>(ws.get<Slot4::T>(N));  // slots or successors
     int32_t *child = ws.get<int32_t>(n), *etin = ws.get<int32_t>(n), *etout = ws.get<int32_t>(n);
     uint8_t *tflag = ws.get<uint8_t>(n);
     int32_t *Lt = (hybrid || blocked) ? nullptr : ws.get<int32_t>(ld * levels);
@@ -628,7 +630,10 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
         PhaseTimer pt("br.forest_succ", s);
         launch(k_arc_scatter, gA, 256, 0, s, tuv, n_arcs, off, deg, B);
         note_launch();
-        launch(k_forest_succ, gA, 256, 0, s, B, n_arcs, N, off, succ);
+        if (wide)
+            launch(k_forest_succ<Slot8>, gA, 256, 0, s, B, n_arcs, N, off, static_cast<Slot8::T *>(succ));
+        else
+            launch(k_forest_succ<Slot4>, gA, 256, 0, s, B, n_arcs, N, off, static_cast<Slot4::T *>(succ));
         note_launch();
         launch(k_root_flags, gn, 256, 0, s, n, par, off, rflag);
         note_launch();
@@ -639,13 +644,15 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
         PhaseTimer pt("br.chain", s);
         launch(k_root_list, gn, 256, 0, s, n, rflag, rpos, roots);
         note_launch();
-        launch(k_chain, gn, 256, 0, s, n, rpos, roots, B, off, int32_t(A), succ);
+        if (wide)
+            launch(k_chain<Slot8>, gn, 256, 0, s, n, rpos, roots, B, off, int32_t(A), static_cast<Slot8::T *>(succ));
+        else
+            launch(k_chain<Slot4>, gn, 256, 0, s, n, rpos, roots, B, off, int32_t(A), static_cast<Slot4::T *>(succ));
         note_launch();
         rc = last_launch();
     }
-    if (!rc) rc = set_device_i32(vhead, int32_t(A), s);
     RankResult rr{};
-    if (!rc) rc = list_rank(succ, N, nullptr, vhead, false, -1, st, ws, &rr);
+    if (!rc) rc = list_rank(succ, N, nullptr, int32_t(A), false, -1, st, ws, &rr);
     if (!rc) {
         const int gt = grid_for(n, 256);
         PhaseTimer pt("br.lowhigh_prep", s);

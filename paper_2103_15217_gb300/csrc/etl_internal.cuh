@@ -192,23 +192,79 @@ etl_status radix_sort_pairs(const int32_t *keys_in, const int32_t *vals_in, cons
 
 // ----------------------------------------------------------------- list ranking
 
-// Result of ranking one list: element e lies in sublist sid = packed[e].x at
-// local offset (packed[e].y & 0xffff) with (packed[e].y >> 16) even-indexed
-// elements before it inside the sublist; R[sid] / O[sid] are the number of
-// elements / of even-indexed elements before that sublist's first element.
-// So rank(e) = R[sid] + lr and evens_before(e) = O[sid] + lo.
-struct RankResult {
-    const uint2 *packed;
-    const int32_t *R;
-    const int32_t *O;
-    int64_t rcap;  // entries of R / O; a packed sublist id >= rcap marks an element off the list
+// Records of ranked list elements: the sublist's id, the element's offset in it (lr) and, in 8-byte
+// records, the number of even-indexed elements before it in the sublist (lo; bit 15 of that field: a
+// contracted leaf). In the in-place form (rank.cu) the same word is the element's slot: its successor
+// before the ranking, its record afterwards. A slot can also be marked as not on the list: a walk that
+// comes across it by claiming it at random leaves it alone.
+struct Slot4 {  // successor < 2^30 or -1; kOff; record: top bit, sublist id << lb, lr (never -1)
+    using T = uint32_t;
+    static constexpr uint32_t kOff = 0x7ffffffeu;
+    __device__ static __forceinline__ T exch(T *p, T v) { return atomicExch(p, v); }
+    __device__ static __forceinline__ bool off(T v) { return v == kOff; }
+    __device__ static __forceinline__ bool raw(T v) { return (!(v >> 31) && v != kOff) || v == 0xffffffffu; }
+    __device__ static __forceinline__ T make(int32_t succ) { return uint32_t(succ); }
+    __device__ static __forceinline__ T off_list() { return kOff; }
+    __device__ static __forceinline__ int32_t next(T v) { return int32_t(v); }
+    __device__ static __forceinline__ T rec(int32_t sid, uint32_t lr, uint32_t, int lb) {
+        return 0x80000000u | (uint32_t(sid) << lb) | lr;
+    }
+    __device__ static __forceinline__ int32_t sid(T v, int lb) { return int32_t((v & 0x7fffffffu) >> lb); }
+    __device__ static __forceinline__ uint32_t lr(T v, int lb) { return v & ((1u << lb) - 1u); }
 };
+struct Slot8 {  // low word: successor / sublist id; high word: kRaw / kOff / lr | lo << 16
+    using T = unsigned long long;
+    static constexpr uint32_t kRaw = 0xffffffffu, kOff = 0xfffffffeu;
+    __device__ static __forceinline__ T pack(uint32_t lo, uint32_t hi) { return (T(hi) << 32) | lo; }
+    __device__ static __forceinline__ T exch(T *p, T v) { return atomicExch(p, v); }
+    __device__ static __forceinline__ bool off(T v) { return uint32_t(v >> 32) == kOff; }
+    __device__ static __forceinline__ bool raw(T v) { return uint32_t(v >> 32) == kRaw; }
+    __device__ static __forceinline__ T make(int32_t succ) { return pack(uint32_t(succ), kRaw); }
+    __device__ static __forceinline__ T off_list() { return pack(uint32_t(ETL_END), kOff); }
+    __device__ static __forceinline__ int32_t next(T v) { return int32_t(uint32_t(v)); }
+    __device__ static __forceinline__ T rec(int32_t sid, uint32_t lr, uint32_t lo, int) {
+        return pack(uint32_t(sid), lr | (lo << 16));
+    }
+    __device__ static __forceinline__ int32_t sid(T v, int) { return int32_t(uint32_t(v)); }
+    __device__ static __forceinline__ uint32_t lr(T v, int) { return uint32_t(v >> 32) & 0xffffu; }
+    __device__ static __forceinline__ uint32_t lo(T v) { return uint32_t(v >> 48) & 0x7fffu; }
+    __device__ static __forceinline__ bool leaf(T v) { return (v >> 63) && !raw(v) && !off(v); }
+};
+inline bool wide_slots(int64_t len) { return len > (int64_t(1) << 30); }
+
+// Result of ranking one list: element e's record names its sublist; T[sid].x / T[sid].y are the number
+// of elements / of even-indexed elements before that sublist's first element. So rank(e) =
+// T[sid].x + lr and evens_before(e) = T[sid].y + lo.
+struct RankResult {
+    const void *recs;  // Slot8 records if wide, else Slot4
+    bool wide;
+    int lb;
+    const int4 *T;
+    int64_t rcap;  // entries of T
+};
+
+// rank of element e of a list ranked without dual; -1 if its record shows that it is not on the list
+__device__ __forceinline__ int32_t rank_at(const RankResult &r, int64_t e) {
+    int32_t sid, lr;
+    if (r.wide) {
+        const Slot8::T v = static_cast<const Slot8::T *>(r.recs)[e];
+        if (Slot8::raw(v) || Slot8::off(v)) return -1;
+        sid = Slot8::sid(v, 0);
+        lr = int32_t(Slot8::lr(v, 0));
+    } else {
+        const Slot4::T v = static_cast<const Slot4::T *>(r.recs)[e];
+        if (Slot4::raw(v) || Slot4::off(v)) return -1;
+        sid = Slot4::sid(v, r.lb);
+        lr = int32_t(Slot4::lr(v, r.lb));
+    }
+    return (sid >= 0 && sid < r.rcap) ? __ldg(&r.T[sid].x) + lr : -1;
+}
 
 struct RankParams {
     int k0_log2 = 5;     // level-0 splitter density: one in 2^k0_log2 elements
     int k_log2 = 3;      // density at the upper levels (1 in 8: 1-4% faster than 1 in 16 on trees of 2^15 .. 2^22)
     int block = 128;     // threads per block of the walk kernels
-    int blocks_per_sm = 4;  // 512 walkers per SM: more of them measured slower (DRAM contention)
+    int blocks_per_sm = 8;  // 1024 walkers per SM on lists larger than L2
 };
 RankParams &rank_params();
 
@@ -232,20 +288,15 @@ struct RmqParams {
 };
 RmqParams &rmq_params();
 
-// succ[0..n_cap) with elements >= *d_len (if d_len) inert; head = *d_head.
-// dual: also count even-indexed elements (the opening brackets of a tour).
-etl_status list_rank(const int32_t *succ, int64_t n_cap, const int32_t *d_len, const int32_t *d_head, bool dual,
-                     int64_t expect_len, int32_t *status, Workspace &ws, RankResult *out);
-
-// rank[e] for e in [0, len) (plain output of the generic list-ranking entry point)
-etl_status final_rank(const RankResult &r, int64_t len, int32_t *rank, cudaStream_t s);
-// *p = v on the stream (a kernel, so no host buffer has to outlive the call)
-etl_status set_device_i32(int32_t *p, int32_t v, cudaStream_t s);
-
-__device__ __forceinline__ int32_t rank_of(const RankResult &r, uint2 p) { return r.R[p.x] + int32_t(p.y & 0xffffu); }
-__device__ __forceinline__ int32_t evens_before(const RankResult &r, uint2 p) {
-    return r.O[p.x] + int32_t(p.y >> 16);
-}
+// Ranks a list of len elements, from *d_head, or from `head` if d_head is null. list: if
+// rank_in_place(len, dual), len slots (Slot8 if dual or wide_slots(len), else Slot4), which the records
+// replace; otherwise len int32 successors, and the records get an array of their own. An element that
+// is on no list holds off_list() in a slot, Slot4::kOff as a successor; a contracted leaf's second
+// element off_list() in a slot, -1 as a successor. dual: also counts even-indexed elements (the opening
+// brackets of a tour). expect_len: the total weight the list must have (-1: not checked).
+bool rank_in_place(int64_t len, bool dual);
+etl_status list_rank(void *list, int64_t len, const int32_t *d_head, int32_t head, bool dual, int64_t expect_len,
+                     int32_t *status, Workspace &ws, RankResult *out);
 
 // ----------------------------------------------------------------- sparse tables
 

@@ -139,19 +139,25 @@ __global__ void k_tour_succ(const int2 *__restrict__ kv, const int32_t *__restri
     }
 }
 
-// succ[2v] = so[v], succ[2v + 1] = sc[v], one 8-byte store per node. A leaf v's brackets are
-// adjacent in the tour: 2v jumps straight to the successor of 2v+1 with weight 2 (top bit set), and
-// 2v+1 leaves the list. Roots are never contracted.
+// The tour's list (rank.cu): element 2v is followed by so[v], element 2v + 1 by sc[v]; one store per
+// node. A leaf v's brackets are adjacent in the tour: 2v jumps straight to the successor of 2v+1 with
+// weight 2 (top bit set), and 2v+1 is off the list. Roots are never contracted.
+template <bool SLOTS>
 __global__ void k_tour_assemble(const int32_t *__restrict__ coff, const int32_t *__restrict__ par,
                                 const int32_t *__restrict__ so, const int32_t *__restrict__ sc, int32_t n,
-                                int32_t *__restrict__ succ) {
+                                void *__restrict__ list) {
     pdl_prologue();
-    int2 *pair = reinterpret_cast<int2 *>(succ);
     for (int64_t t = gtid(); t < n; t += gstride()) {
         const bool leaf = __ldcs(coff + t) == __ldcs(coff + t + 1) && __ldcs(par + t) >= 0;  // no children, no root
         const int32_t a = __ldcs(so + t), c = __ldcs(sc + t);
         // a malformed close successor (c < 0) stays uncontracted: the validity checks see it
-        pair[t] = (leaf && c >= 0) ? make_int2(int32_t(uint32_t(c) | 0x80000000u), ETL_END) : make_int2(a, c);
+        const bool one = leaf && c >= 0;
+        const int32_t x = one ? int32_t(uint32_t(c) | 0x80000000u) : a;
+        if (SLOTS)
+            static_cast<ulonglong2 *>(list)[t] =
+                make_ulonglong2(Slot8::make(x), one ? Slot8::off_list() : Slot8::make(c));
+        else
+            static_cast<int2 *>(list)[t] = make_int2(x, one ? ETL_END : c);
     }
 }
 
@@ -171,28 +177,25 @@ __global__ void k_link_roots(const int32_t *__restrict__ root_cnt, const int32_t
     }
 }
 
-__global__ void k_node_stats(RankResult rr, const int32_t *__restrict__ succ, int32_t n, int32_t *__restrict__ pre,
-                             int32_t *__restrict__ depth, int32_t *__restrict__ size, int32_t *__restrict__ order,
-                             int32_t *__restrict__ status) {
+__global__ void k_node_stats(RankResult rr, int32_t n, int32_t *__restrict__ pre, int32_t *__restrict__ depth,
+                             int32_t *__restrict__ size, int32_t *__restrict__ order, int32_t *__restrict__ status) {
     pdl_prologue();
-    const uint4 *pk = reinterpret_cast<const uint4 *>(rr.packed);  // brackets 2v and 2v+1 side by side
+    const ulonglong2 *recs = static_cast<const ulonglong2 *>(rr.recs);  // brackets 2v and 2v+1 side by side
     for (int64_t t = gtid(); t < n; t += gstride()) {
-        const bool leaf = __ldcs(succ + 2 * t) < ETL_END;  // contracted: the closing bracket is ranked right after
-        uint4 q;
-        if (leaf) {
-            const uint2 a = __ldcs(rr.packed + 2 * t);
-            q = make_uint4(a.x, a.y, a.x, 0u);
-        } else {
-            q = __ldcs(pk + t);
-        }
-        if (q.x >= rr.rcap || q.z >= rr.rcap) {  // not on the list from the root: malformed input
+        const ulonglong2 q = __ldcs(recs + t);
+        // contracted: the closing bracket is ranked right after
+        const bool leaf = Slot8::leaf(q.x) || Slot8::off(q.y);
+        const int32_t sa = Slot8::sid(q.x, 0), sb = leaf ? sa : Slot8::sid(q.y, 0);
+        if (Slot8::raw(q.x) || Slot8::off(q.x) || (!leaf && Slot8::raw(q.y)) || sa < 0 || sa >= rr.rcap || sb < 0 ||
+            sb >= rr.rcap) {  // not on the list from the root: malformed input
             set_status(status, ETL_EBADTREE);
             pre[t] = depth[t] = size[t] = -1;
             continue;
         }
-        const uint2 in = make_uint2(q.x, q.y), out = make_uint2(q.z, q.w);
-        const int32_t r0 = rank_of(rr, in), r1 = leaf ? r0 + 1 : rank_of(rr, out);
-        const int32_t p = evens_before(rr, in);
+        const int2 A = __ldg(reinterpret_cast<const int2 *>(rr.T + sa));
+        const int32_t r0 = A.x + int32_t(Slot8::lr(q.x, 0));
+        const int32_t r1 = leaf ? r0 + 1 : __ldg(&rr.T[sb].x) + int32_t(Slot8::lr(q.y, 0));
+        const int32_t p = A.y + int32_t(Slot8::lo(q.x));
         __stcs(pre + t, p);
         __stcs(depth + t, 2 * p - r0);
         __stcs(size + t, (r1 - r0 + 1) >> 1);
@@ -433,7 +436,8 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         int32_t *cnt = ws.get<int32_t>(n);
         int32_t *coff = ws.get<int32_t>(int64_t(n) + 1);
         int32_t *misc = ws.get<int32_t>(4);  // [0] list head, [1] offsets invalid
-        int32_t *succ = ws.get<int32_t>(2 * int64_t(n));
+        const bool slots = rank_in_place(2 * int64_t(n), true);
+        void *list = slots ? static_cast<void *>(ws.get<ulonglong2>(n)) : ws.get<int2>(n);  // 2n list elements
         int32_t *sc = ws.get<int32_t>(n);  // successors of the closing brackets; those of the opening ones reuse cnt
         int32_t *root_cnt = ws.get<int32_t>(k), *root_of = ws.get<int32_t>(k);
         int32_t *inst_of = batch ? ws.get<int32_t>(n) : nullptr;
@@ -471,16 +475,16 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
             note_launch();
             launch(k_link_roots, grid_for(k, 256), 256, 0, s, root_cnt, root_of, k, n, sc, misc, h->status);
             note_launch();
-            launch(k_tour_assemble, grid_for(n, 256), 256, 0, s, coff, par, so, sc, n, succ);
+            launch(slots ? k_tour_assemble<true> : k_tour_assemble<false>, grid_for(n, 256), 256, 0, s, coff, par, so,
+                   sc, n, list);
             note_launch();
             st = last_launch();
         }
         RankResult rr{};
-        if (!st) st = list_rank(succ, 2 * int64_t(n), nullptr, misc, true, 2 * int64_t(n), h->status, ws, &rr);
+        if (!st) st = list_rank(list, 2 * int64_t(n), misc, 0, true, 2 * int64_t(n), h->status, ws, &rr);
         if (!st) {
             PhaseTimer pt("lca.node_stats", s);
-            launch(k_node_stats, grid_for(n, 256), 256, 0, s, rr, succ, n, h->pre, h->depth, h->size, h->order,
-                   h->status);
+            launch(k_node_stats, grid_for(n, 256), 256, 0, s, rr, n, h->pre, h->depth, h->size, h->order, h->status);
             note_launch();
             launch(k_check_instances, grid_for(k, 256), 256, 0, s, root_of, batch ? h->node_off : nullptr, k, n, h->pre,
                    h->size, h->status);

@@ -3,23 +3,40 @@
 // ranks. The paper uses the Wei-JaJa sparse-ruling-set method; this is a
 // GB300-oriented ruling-set ranker:
 //
-//  * Splitters ("rulers") are picked by a multiplicative hash of the element
-//    index: e is a splitter iff (e * M mod 2^b) < 2^b / K. The hashed value
-//    is also the splitter's sublist id, so no table maps elements to sublists
-//    and any structure in the labels (e.g. all opening brackets at even
-//    indices) does not line up with the splitter pattern.
-//  * The walk kernel is persistent: each lane walks one sublist, writing for
-//    every element its sublist id and local offsets, and as soon as a lane's
-//    walk ends it takes the next splitter from a warp-aggregated atomic
-//    counter, so lanes stay busy despite the geometric spread of sublist
-//    lengths. The hot loop is one dependent 4-byte load of succ[] per element,
-//    so throughput comes from the number of walks in flight.
-//  * A walk longer than kLcap elements opens a new sublist on the fly
-//    ("dynamic splitter"), which bounds every local offset and every walk.
+//  * Level 0 cuts the list into sublists, walks them and leaves a record
+//    (sublist id, local offset) per element. It has two forms:
+//    - k_walk0, for lists whose successors and records fit in L2: sublists
+//      start at splitters picked by a multiplicative hash of the element
+//      index, e is one iff (e * M mod 2^b) < S0; the hashed value is the
+//      sublist's id. A step is one dependent load, 0.25 us, and the walks are
+//      bound by the longest sublist, about len / S0 * ln S0 steps.
+//    - k_walk0_in_place, for longer ones, which are bound by memory: element
+//      and record share one slot, and a step is ONE atomic exchange, which
+//      stores the record and returns the successor. Reading the successor in
+//      one array and writing the record in another touches two sectors per
+//      element over three times the memory: 2^25 random elements take 1.65 ms
+//      that way (4 B read + 8 B write) and 0.49 ms as 4-byte exchanges (0.95
+//      ms as 8-byte ones), measured with independent accesses. An exchange
+//      takes 0.47 us, so the short lists keep the loads. (A load followed by
+//      a store to the same sector costs 1 us and more.)
+//  * The in-place form decides where sublists start as it runs. Every lane
+//    claims an element by exchanging it for the record (its sublist, offset 0)
+//    and walks on from there; a walk ends at the tail or where its exchange
+//    returns another walk's record, which it puts back and links to. A lane
+//    whose walk has ended claims its next candidate; if that was visited
+//    already, the record goes back and the claim is dropped. So long sublists
+//    are cut by the lanes that have run out of work: with 13 claims per lane
+//    the last walk ends after 2 to 2.5 len / lanes steps, and 2.5 to 3 sublists
+//    per lane have been opened. Candidates are the multiples of the golden
+//    ratio times len (any prefix of them is evenly spread, and no two of
+//    len / 3 fall on one element).
+//  * A walk whose offset no longer fits the record opens a new sublist and
+//    goes on in it ("dynamic" sublist).
 //  * The reduced list of sublists (weights = sublist length, and number of
-//    even-indexed elements) is ranked recursively the same way; when it has
-//    at most kPjCap elements one CTA finishes it with pointer jumping in
-//    shared memory, then the prefixes are pushed back down level by level.
+//    even-indexed elements) is cut and walked again until at most kTopCap
+//    entries are left, which one CTA ranks in shared memory: walks, then
+//    pointer jumping over at most kTopSub sublists. The prefixes are pushed
+//    back down level by level.
 //
 // The "dual" mode also counts even-indexed elements: in the bracket layout
 // of a rooted tree (2v = entering v, 2v+1 = leaving v) that count is the
@@ -28,7 +45,7 @@
 // set (and not -1) marks a contracted leaf: element 2v of a leaf v stands for
 // both of its brackets (weight 2), the low 31 bits are the successor of 2v+1,
 // and 2v+1 itself is off the list.
-#include <cstdio>
+#include <algorithm>
 #include <mutex>
 
 #include "etl_internal.cuh"
@@ -36,96 +53,219 @@
 namespace etl {
 namespace {
 
-constexpr int32_t kLcap = 4096;    // longest walk before a dynamic splitter is opened (< 2^16 - 2)
-constexpr int kPjCap = 8192;       // top level solved by one CTA in shared memory
-constexpr int kPjThreads = 1024;
-constexpr int kPjItems = kPjCap / kPjThreads;
+constexpr int32_t kLcap = 4096;  // longest sublist of 8-byte records (< 2^15)
+constexpr int kTopThreads = 1024;
+constexpr int kTopCap = 15360;   // entries one CTA ranks in shared memory (12 bytes each)
+constexpr int kTopSub = 2 * kTopThreads;
+constexpr int32_t kEndT = 0x7fffffff;  // "no successor" in a reduced list's entry
+constexpr int32_t kVisited = int32_t(0x80000000u);
 constexpr uint32_t kMul = 0x9E3779B1u;  // odd, so multiplication is a bijection mod 2^b
 
-struct Hash {
-    uint32_t M, Minv, mask, S0;
-    __device__ __forceinline__ bool split(uint32_t e) const { return ((e * M) & mask) < S0; }
-    __device__ __forceinline__ int32_t sid(uint32_t e) const { return int32_t((e * M) & mask); }
-    __device__ __forceinline__ uint32_t elem(uint32_t s) const { return (s * Minv) & mask; }
-};
-
-uint32_t inverse_mod_2_32(uint32_t a) {  // Newton iteration for a^-1 mod 2^32 (a odd)
+constexpr uint32_t inverse_mod_2_32(uint32_t a) {  // Newton iteration for a^-1 mod 2^32 (a odd)
     uint32_t x = a;
     for (int i = 0; i < 5; ++i) x *= 2u - a * x;
     return x;
 }
 
-Hash make_hash(int64_t cap, int k_log2) {
-    int b = ceil_log2(uint64_t(cap > 1 ? cap : 1));
-    if (b < k_log2) b = k_log2;
-    Hash h;
-    h.M = kMul;
-    h.Minv = inverse_mod_2_32(kMul);
-    h.mask = b >= 32 ? 0xffffffffu : ((1u << b) - 1u);
-    h.S0 = 1u << (b - k_log2);
-    return h;
+struct Hash {
+    uint32_t mask, S0;  // elements [0, mask], splitters hash below S0
+    __device__ __forceinline__ bool split(uint32_t e) const { return ((e * kMul) & mask) < S0; }
+    __device__ __forceinline__ int32_t sid(uint32_t e) const { return int32_t((e * kMul) & mask); }
+    __device__ __forceinline__ uint32_t elem(uint32_t s) const {
+        constexpr uint32_t kInv = inverse_mod_2_32(kMul);
+        return (s * kInv) & mask;
+    }
+};
+
+// candidate w >= 1 of a list of len elements: floor(frac(w * golden ratio) * len). The distance of any
+// two of the first W multiples is above 0.38 / W, so W <= len / 3 candidates are distinct elements.
+__device__ __forceinline__ int64_t candidate(uint32_t w, int64_t len) {
+    return int64_t(__umul64hi(uint64_t(w) * 0x9E3779B97F4A7C15ull, uint64_t(len)));
 }
 
+// A warp's supply of sublist ids: kFirst of its own, then kTake at a time from a counter. Only a
+// successful claim uses one up, so that the reduced list has few empty entries; once the ids have passed
+// `limit` the warp claims nothing any more (claims shorten the walks; the result does not need them).
+// (Ids 8 at a time, all from the counter: the walk of 2^25 elements 10% slower, each refill holds up the
+// warp for one contended atomic.)
+struct SidPool {
+    static constexpr int kFirst = 64, kTake = 32;
+    int32_t base, count;  // the same in every lane
+    bool closed = false;
+    __device__ __forceinline__ explicit SidPool(uint32_t warp) : base(int32_t(warp) * kFirst), count(kFirst) {}
+    // ids from the counter start at `start`
+    __device__ __forceinline__ void refill(int32_t *ctr, int32_t start, int32_t limit, bool need, int32_t &sid) {
+        const unsigned m = __ballot_sync(kFull, need);
+        if (!m) return;
+        const int cnt = __popc(m), i = __popc(m & lanemask_lt());
+        int32_t nb = 0;
+        const bool more = cnt > count;
+        if (more) {
+            if ((threadIdx.x & 31) == 0) nb = start + atomicAdd(ctr, kTake);
+            nb = __shfl_sync(kFull, nb, 0);
+            closed = nb + kTake > limit;
+        }
+        if (need) sid = i < count ? base + i : nb + (i - count);
+        if (more) {
+            base = nb + (cnt - count);
+            count += kTake - cnt;
+        } else {
+            base += cnt;
+            count -= cnt;
+        }
+    }
+    // ids taken and not used become empty sublists
+    __device__ __forceinline__ void give_back(int32_t sid, int4 *T, int32_t cap) const {
+        if (sid >= 0 && sid < cap) T[sid] = make_int4(0, 0, kEndT, 0);
+        for (int i = threadIdx.x & 31; i < count; i += kWarp)
+            if (base + i < cap) T[base + i] = make_int4(0, 0, kEndT, 0);
+    }
+};
+
+// *d_len entries (plus those of *d_add), at most cap
 __device__ __forceinline__ int64_t level_len(int64_t base, const int32_t *d_add, int64_t cap) {
-    int64_t l = base + (d_add ? int64_t(*d_add) : 0);
-    return l < cap ? l : cap;
+    return min(base + (d_add ? int64_t(*d_add) : 0), cap);
 }
 
-// ------------------------------------------------------------ level-0 walk
+// ------------------------------------------------------------ level-0 walk over a list in L2
 
-template <bool DUAL>
-__global__ void k_walk0(const int32_t *__restrict__ succ, int64_t len, const int32_t *__restrict__ d_head, Hash H,
-                        uint2 *__restrict__ packed, int32_t *__restrict__ rnext, int32_t *__restrict__ rw1,
-                        int32_t *__restrict__ rw2, int32_t *__restrict__ ctr, int32_t dyn_cap,
-                        int32_t *__restrict__ next_head, int32_t *__restrict__ status) {
+// Sublist ids: a splitter's hash, S0 for the head's own sublist, S0 + 1 + d for dynamic ones. A lane
+// takes the ids w, w + lanes, ... A record is written once the successor is known, so that it can say
+// whether the element is a contracted leaf.
+template <class S, bool DUAL>
+__global__ void k_walk0(const uint32_t *__restrict__ succ, int64_t len, const int32_t *__restrict__ d_head,
+                        int32_t head_value, Hash H, typename S::T *__restrict__ recs, int lb, uint32_t lcap,
+                        int4 *__restrict__ T, int32_t *__restrict__ dyn, int32_t cap, int32_t *__restrict__ next_head,
+                        int32_t *__restrict__ status) {
     pdl_prologue();
-    const int32_t head = *d_head;
+    const int32_t head = d_head ? *d_head : head_value;
     const bool head_split = H.split(uint32_t(head));
-    if (blockIdx.x == 0 && threadIdx.x == 0) *next_head = head_split ? H.sid(uint32_t(head)) : int32_t(H.S0);
-    const int64_t nwork = int64_t(H.S0) + 1;
-    const int lane = threadIdx.x & 31;
-    int32_t cur = 0, sid = 0;
+    const uint32_t nwork = H.S0 + 1, lanes = gridDim.x * blockDim.x;
+    uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w == 0) *next_head = head_split ? H.sid(uint32_t(head)) : int32_t(H.S0);
+    int32_t cur = -1, sid = 0;
     uint32_t lr = 0, lo = 0;
     int64_t steps = 0;
-    bool active = false, exhausted = false;
     while (true) {
-        unsigned idle = __ballot_sync(kFull, !active);
-        if (idle && !exhausted) {
-            const int leader = __ffs(idle) - 1;
-            int32_t base = 0;
-            if (lane == leader) base = atomicAdd(&ctr[0], __popc(idle));
-            base = __shfl_sync(kFull, base, leader);
-            if (int64_t(base) + __popc(idle) >= nwork) exhausted = true;
-            if (!active) {
-                const int64_t w = int64_t(base) + __popc(idle & lanemask_lt());
-                if (w < nwork) {
-                    int64_t e;
-                    if (w < H.S0) {
-                        e = H.elem(uint32_t(w));
-                    } else {
-                        e = head_split ? len : head;  // the head gets its own sublist unless it is a splitter
-                    }
-                    if (e >= len) {  // hole: no element behind this sublist id
-                        rnext[w] = ETL_END;
-                        rw1[w] = 0;
-                        rw2[w] = 0;
-                    } else {
-                        cur = int32_t(e);
-                        sid = int32_t(w);
-                        lr = lo = 0;
-                        steps = 0;
-                        active = true;
-                    }
+        if (cur < 0) {
+            if (w >= nwork) break;
+            const int64_t e = w < H.S0 ? int64_t(H.elem(w)) : head_split ? len : int64_t(head);
+            sid = int32_t(w);
+            w += lanes;
+            if (e < 0 || e >= len) {  // no element behind this id
+                T[sid] = make_int4(0, 0, kEndT, 0);
+                continue;
+            }
+            cur = int32_t(e);
+            lr = lo = 0;
+            steps = 0;
+        }
+        const uint32_t v = __ldg(succ + cur);
+        int32_t nxt = int32_t(v);
+        bool leaf = false;
+        if (DUAL && nxt < ETL_END) {  // contracted leaf: its closing bracket follows at once
+            nxt &= 0x7fffffff;
+            leaf = true;
+        }
+        recs[cur] = S::rec(sid, lr, leaf ? lo | 0x8000u : lo, lb);
+        const uint32_t l0 = lr;
+        lr += leaf ? 2 : 1;
+        if (DUAL) lo += (cur & 1) == 0 ? 1u : 0u;
+        int32_t link = kEndT;
+        if (nxt == ETL_END) {
+            cur = -1;
+        } else if (nxt < 0 || nxt >= len || ++steps > len) {
+            // a slot that is off the list may be a splitter; reaching one is an error
+            if (v != Slot4::kOff || l0) set_status(status, ETL_EBADTREE);
+            if (v == Slot4::kOff && !l0) lr = 0;
+            cur = -1;
+        } else if (H.split(uint32_t(nxt))) {
+            link = H.sid(uint32_t(nxt));
+            cur = -1;
+        } else {
+            cur = nxt;
+            if (lr >= lcap) {
+                const int32_t ns = int32_t(H.S0) + 1 + atomicAdd(dyn, 1);
+                if (ns >= cap) {
+                    set_status(status, ETL_ETIMEOUT);
+                    cur = -1;
+                } else {
+                    T[sid] = make_int4(int32_t(lr), int32_t(lo), ns, 0);
+                    sid = ns;
+                    lr = lo = 0;
                 }
             }
         }
-        if (__ballot_sync(kFull, active) == 0) {
-            if (exhausted) break;
+        if (cur < 0) T[sid] = make_int4(int32_t(lr), int32_t(lo), link, 0);
+    }
+}
+
+// ------------------------------------------------------------ level-0 walk in place
+
+struct Walk0 {
+    int64_t len;
+    const int32_t *d_head;  // the list's head, or null: `head`
+    int32_t head;
+    uint32_t nclaims;  // the head and nclaims - 1 candidates
+    int32_t start;     // sublist ids below it belong to the warps, the counter hands out those above
+    int32_t limit;     // ids after which no more claims are made
+    int32_t cap;       // sublists there is room for
+    int32_t lb;        // 4-byte records: bits of the local offset
+    int32_t lcap;      // a sublist of lcap elements is continued in a new one
+};
+
+// One lane = one walk at a time. The claims of a lane are fixed (its index, + lanes, + 2 lanes, ...),
+// so that no counter is shared by them.
+template <class S, bool DUAL>
+__global__ void k_walk0_in_place(typename S::T *__restrict__ slots, Walk0 W, int4 *__restrict__ T, int32_t *__restrict__ ctr,
+                        int32_t *__restrict__ next_head, int32_t *__restrict__ status) {
+    pdl_prologue();
+    const uint32_t lanes = gridDim.x * blockDim.x;
+    uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
+    const int32_t head = W.d_head ? *W.d_head : W.head;
+    SidPool pool(w >> 5);
+    int32_t cur = -1, sid = -1;
+    uint32_t lr = 0, lo = 0;
+    bool active = false, claim = false, is_head = false;
+    while (true) {
+        const bool want = !active && w < W.nclaims;
+        pool.refill(ctr, W.start, W.limit, want && sid < 0, sid);
+        if (want) {
+            is_head = w == 0;
+            const int64_t e = is_head ? int64_t(head) : candidate(w, W.len);
+            w += lanes;
+            if (sid < W.cap && e >= 0 && e < W.len) {  // both always hold; keep memory safe
+                cur = int32_t(e);
+                lr = lo = 0;
+                active = claim = true;
+            }
+        }
+        if (pool.closed) w = W.nclaims;
+        if (!__any_sync(kFull, active)) {
+            if (!__any_sync(kFull, w < W.nclaims)) break;
             continue;
         }
-        if (active) {
-            packed[cur] = make_uint2(uint32_t(sid), lr | (lo << 16));
-            int32_t nxt = __ldg(succ + cur);
+        if (!active) continue;
+        const typename S::T v = S::exch(slots + cur, S::rec(sid, lr, lo, W.lb));
+        int32_t link = kEndT;
+        bool done = false;
+        if (!S::raw(v)) {  // visited already, or off the list: put it back
+            S::exch(slots + cur, v);
+            if (claim) {
+                if (is_head) *next_head = S::off(v) ? 0 : S::sid(v, W.lb);
+                if (S::off(v) && is_head) set_status(status, ETL_EBADTREE);
+                active = false;
+            } else {  // link to the sublist that starts here
+                if (S::off(v) || S::lr(v, W.lb) != 0)
+                    set_status(status, ETL_EBADTREE);  // not the first of a sublist: a second predecessor
+                else
+                    link = S::sid(v, W.lb);
+                done = true;
+            }
+        } else {
+            if (claim && is_head) *next_head = sid;
+            claim = false;
+            int32_t nxt = S::next(v);
             lr += 1;
             if (DUAL) {
                 lo += (cur & 1) == 0 ? 1u : 0u;
@@ -134,228 +274,291 @@ __global__ void k_walk0(const int32_t *__restrict__ succ, int64_t len, const int
                     lr += 1;
                 }
             }
-            ++steps;
-            const bool bad = nxt >= len || nxt < ETL_END || steps > len;
-            if (nxt == ETL_END || bad || H.split(uint32_t(nxt))) {
-                if (bad) set_status(status, ETL_EBADTREE);
-                rnext[sid] = (nxt == ETL_END || bad) ? ETL_END : H.sid(uint32_t(nxt));
-                rw1[sid] = int32_t(lr);
-                rw2[sid] = int32_t(lo);
-                active = false;
-            } else if (lr >= uint32_t(kLcap)) {
-                const int32_t d = atomicAdd(&ctr[1], 1);
-                if (d >= dyn_cap) {
-                    set_status(status, ETL_ETIMEOUT);
-                    rnext[sid] = ETL_END;
-                    rw1[sid] = int32_t(lr);
-                    rw2[sid] = int32_t(lo);
-                    active = false;
-                } else {
-                    const int32_t ns = int32_t(H.S0) + 1 + d;
-                    rnext[sid] = ns;
-                    rw1[sid] = int32_t(lr);
-                    rw2[sid] = int32_t(lo);
-                    sid = ns;
-                    lr = lo = 0;
-                    cur = nxt;
-                }
+            if (nxt == ETL_END) {
+                done = true;
+            } else if (nxt < 0 || nxt >= W.len) {
+                set_status(status, ETL_EBADTREE);
+                done = true;
             } else {
                 cur = nxt;
-            }
-        }
-    }
-}
-
-// ------------------------------------------------------------ upper-level walk (explicit weights)
-
-__global__ void k_walk(const int32_t *__restrict__ succ, const int32_t *__restrict__ w1in,
-                       const int32_t *__restrict__ w2in, int64_t len_base, const int32_t *__restrict__ d_len_add,
-                       int64_t cap, const int32_t *__restrict__ d_head, Hash H, int4 *__restrict__ loc,
-                       int32_t *__restrict__ rnext, int32_t *__restrict__ rw1, int32_t *__restrict__ rw2,
-                       int32_t *__restrict__ ctr, int32_t dyn_cap, int32_t *__restrict__ next_head,
-                       int32_t *__restrict__ status) {
-    pdl_prologue();
-    const int64_t len = level_len(len_base, d_len_add, cap);
-    const int32_t head = *d_head;
-    const bool head_split = H.split(uint32_t(head));
-    if (blockIdx.x == 0 && threadIdx.x == 0) *next_head = head_split ? H.sid(uint32_t(head)) : int32_t(H.S0);
-    const int64_t nwork = int64_t(H.S0) + 1;
-    const int lane = threadIdx.x & 31;
-    int32_t cur = 0, sid = 0, a1 = 0, a2 = 0, lr = 0;
-    int64_t steps = 0;
-    bool active = false, exhausted = false;
-    while (true) {
-        unsigned idle = __ballot_sync(kFull, !active);
-        if (idle && !exhausted) {
-            const int leader = __ffs(idle) - 1;
-            int32_t base = 0;
-            if (lane == leader) base = atomicAdd(&ctr[0], __popc(idle));
-            base = __shfl_sync(kFull, base, leader);
-            if (int64_t(base) + __popc(idle) >= nwork) exhausted = true;
-            if (!active) {
-                const int64_t w = int64_t(base) + __popc(idle & lanemask_lt());
-                if (w < nwork) {
-                    int64_t e = (w < H.S0) ? int64_t(H.elem(uint32_t(w))) : (head_split ? len : head);
-                    if (e >= len) {
-                        rnext[w] = ETL_END;
-                        rw1[w] = 0;
-                        rw2[w] = 0;
+                if (lr >= uint32_t(W.lcap)) {
+                    const int32_t ns = W.start + atomicAdd(ctr, 1);
+                    if (ns >= W.cap) {
+                        set_status(status, ETL_ETIMEOUT);
+                        done = true;
                     } else {
-                        cur = int32_t(e);
-                        sid = int32_t(w);
-                        a1 = a2 = lr = 0;
-                        steps = 0;
-                        active = true;
+                        T[sid] = make_int4(int32_t(lr), int32_t(lo), ns, 0);
+                        sid = ns;
+                        lr = lo = 0;
                     }
                 }
             }
         }
-        if (__ballot_sync(kFull, active) == 0) {
-            if (exhausted) break;
-            continue;
+        if (done) {
+            T[sid] = make_int4(int32_t(lr), int32_t(lo), link, 0);
+            active = false;
+            sid = -1;
         }
-        if (active) {
-            loc[cur] = make_int4(sid, a1, a2, 0);
-            a1 += w1in[cur];
-            a2 += w2in[cur];
-            ++lr;
-            const int32_t nxt = succ[cur];
-            ++steps;
-            const bool bad = nxt >= len || nxt < ETL_END || steps > len;
-            if (nxt == ETL_END || bad || H.split(uint32_t(nxt))) {
-                if (bad) set_status(status, ETL_EBADTREE);
-                rnext[sid] = (nxt == ETL_END || bad) ? ETL_END : H.sid(uint32_t(nxt));
-                rw1[sid] = a1;
-                rw2[sid] = a2;
-                active = false;
-            } else if (lr >= kLcap) {
-                const int32_t d = atomicAdd(&ctr[1], 1);
-                if (d >= dyn_cap) {
-                    set_status(status, ETL_ETIMEOUT);
-                    rnext[sid] = ETL_END;
-                    rw1[sid] = a1;
-                    rw2[sid] = a2;
-                    active = false;
-                } else {
-                    const int32_t ns = int32_t(H.S0) + 1 + d;
-                    rnext[sid] = ns;
-                    rw1[sid] = a1;
-                    rw2[sid] = a2;
-                    sid = ns;
-                    a1 = a2 = lr = 0;
-                    cur = nxt;
-                }
-            } else {
-                cur = nxt;
+    }
+    pool.give_back(sid, T, W.cap);
+}
+
+// ------------------------------------------------------------ upper-level walk (explicit weights)
+
+// Entry of a reduced list: x, y = the sublist's weights, z = the id of the next sublist (kEndT: none).
+// The hash covers the entries there are (the device knows how many); one in 2^k_log2 is a splitter, and
+// never more than `most`. One 16-byte load per step, 0.25 us; an entry's place (sublist, offsets) goes to
+// loc. (Replacing the entry by it would put a load and a store on one sector.)
+__global__ void k_walk(const int4 *__restrict__ T, int64_t base, const int32_t *__restrict__ d_add, int64_t cap,
+                       const int32_t *__restrict__ d_head, int k_log2, uint32_t most, int4 *__restrict__ loc,
+                       int4 *__restrict__ up, int32_t *__restrict__ up_len, int32_t *__restrict__ next_head,
+                       int32_t *__restrict__ status) {
+    pdl_prologue();
+    const int64_t len = level_len(base, d_add, cap);
+    const int32_t head = *d_head;
+    Hash H;
+    const int b = len <= 1 ? 0 : 64 - __clzll(len - 1);
+    H.mask = (1u << b) - 1u;
+    H.S0 = min(((H.mask >> k_log2) + 1u), most);
+    const bool head_split = H.split(uint32_t(head));
+    const uint32_t nwork = H.S0 + 1, lanes = gridDim.x * blockDim.x;
+    uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w == 0) {
+        *next_head = head_split ? H.sid(uint32_t(head)) : int32_t(H.S0);
+        *up_len = int32_t(nwork);
+    }
+    int32_t cur = -1, sid = 0, a1 = 0, a2 = 0;
+    int64_t steps = 0;
+    while (true) {
+        if (cur < 0) {
+            if (w >= nwork) break;
+            const int64_t e = w < H.S0 ? int64_t(H.elem(w)) : head_split ? len : int64_t(head);
+            sid = int32_t(w);
+            w += lanes;
+            if (e < 0 || e >= len) {
+                up[sid] = make_int4(0, 0, kEndT, 0);
+                continue;
             }
+            cur = int32_t(e);
+            a1 = a2 = 0;
+            steps = 0;
         }
+        const int4 t = __ldg(T + cur);
+        loc[cur] = make_int4(a1, a2, sid, 0);
+        a1 += t.x;
+        a2 += t.y;
+        int32_t link = kEndT;
+        if (t.z == kEndT) {
+            cur = -1;
+        } else if (t.z < 0 || t.z >= len || ++steps > len) {
+            set_status(status, ETL_EBADTREE);
+            cur = -1;
+        } else if (H.split(uint32_t(t.z))) {
+            link = H.sid(uint32_t(t.z));
+            cur = -1;
+        } else {
+            cur = t.z;
+        }
+        if (cur < 0) up[sid] = make_int4(a1, a2, link, 0);
     }
 }
 
-// ------------------------------------------------------------ top level: pointer jumping in smem
+// ------------------------------------------------------------ top level: one CTA, shared memory
 
-// Q = predecessor pointer, V1/V2 = sums over the segment (Q, e], F = first
-// element of that segment. A round replaces Q by Q[Q] and adds the
-// predecessor segment; after ceil(log2 len) rounds every Q is -1 and V is the
-// inclusive prefix from the list head, F the head itself.
-__global__ void __launch_bounds__(kPjThreads)
-    k_pointer_jump(const int32_t *__restrict__ succ, const int32_t *__restrict__ w1, const int32_t *__restrict__ w2,
-                   int64_t len_base, const int32_t *__restrict__ d_len_add, int64_t cap,
-                   const int32_t *__restrict__ d_head, int64_t expect_total, int32_t *__restrict__ R,
-                   int32_t *__restrict__ O, int32_t *__restrict__ status) {
+// FROM_LIST: the list itself instead of a reduced list; each element on it becomes its own sublist in
+// the result. Shared memory holds the entries (three words each); at most kTopSub - 1 splitters and the
+// head cut them into sublists, and those are ranked by pointer jumping: Q = predecessor, V1 / V2 = sums
+// over the segment (Q, e], F = first sublist of that segment. A round replaces Q by Q[Q] and adds the
+// predecessor's segment; after ceil(log2 kTopSub) rounds every Q is -1 and V is the inclusive prefix
+// from the list head, F the head's sublist. One SM issues all of it, so the steps are kept to a few
+// instructions (claims as in the in-place walk, tried here, took twice the time).
+constexpr int kTopBatch = 5;  // entries per thread whose loads are in flight together
+
+template <class S, bool DUAL, bool FROM_LIST>
+__global__ void __launch_bounds__(kTopThreads)
+    k_top(const uint32_t *__restrict__ succ, typename S::T *__restrict__ recs, int lb, int4 *__restrict__ T,
+          int64_t base, const int32_t *__restrict__ d_add, int64_t cap, const int32_t *__restrict__ d_head,
+          int32_t head_value, int64_t expect_total, int32_t *__restrict__ status) {
     pdl_prologue();
     extern __shared__ int32_t sm[];
-    int32_t *Q = sm, *V1 = sm + kPjCap, *V2 = sm + 2 * kPjCap, *F = sm + 3 * kPjCap;
     __shared__ int found;
-    const int len = int(level_len(len_base, d_len_add, cap));
-    const int32_t head = *d_head;
+    int32_t *Q = sm, *V1 = sm + kTopSub, *V2 = sm + 2 * kTopSub, *F = sm + 3 * kTopSub, *SN = sm + 4 * kTopSub;
+    const int len = int(level_len(base, d_add, cap));
+    int32_t *nx = sm + 5 * kTopSub, *a1 = nx + len, *a2 = a1 + len;
+    const int32_t head = d_head ? *d_head : head_value;
+    Hash H;
+    const int b = len <= 1 ? 0 : 32 - __clz(len - 1);
+    H.mask = (1u << b) - 1u;
+    H.S0 = min((H.mask + 1u) >> 1, uint32_t(kTopSub - 1));
+    const bool head_split = H.split(uint32_t(head));
+    const int32_t head_sub = head_split ? H.sid(uint32_t(head)) : int32_t(H.S0);
     if (threadIdx.x == 0) found = 0;
-    for (int e = threadIdx.x; e < len; e += kPjThreads) Q[e] = -1;
+    for (int i = threadIdx.x; i < len; i += kTopBatch * kTopThreads) {
+        int4 t[kTopBatch];
+        uint32_t v[kTopBatch];
+#pragma unroll
+        for (int j = 0; j < kTopBatch; ++j) {
+            const int e = i + j * kTopThreads;
+            if (e < len) {
+                if (FROM_LIST)
+                    v[j] = succ[e];
+                else
+                    t[j] = T[e];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kTopBatch; ++j) {
+            const int e = i + j * kTopThreads;
+            if (e >= len) continue;
+            if (FROM_LIST) {
+                int32_t nxt = int32_t(v[j]), w1 = 1;
+                if (DUAL && nxt < ETL_END) {
+                    nxt &= 0x7fffffff;
+                    w1 = 2;
+                }
+                // anything that is no element ends the list (the total is checked)
+                nx[e] = (nxt < 0 || nxt >= len) ? kEndT : nxt;
+                a1[e] = w1;
+                a2[e] = (DUAL && (e & 1) == 0) ? 1 : 0;
+                if (nxt != ETL_END && nxt >= len && v[j] != Slot4::kOff) set_status(status, ETL_EBADTREE);
+                if (!DUAL && nxt < ETL_END) set_status(status, ETL_EBADTREE);
+                if (!DUAL && expect_total >= 0 && v[j] == Slot4::kOff) set_status(status, ETL_EBADTREE);
+            } else {
+                nx[e] = t[j].z;
+                a1[e] = t[j].x;
+                a2[e] = t[j].y;
+            }
+        }
+    }
     __syncthreads();
-    for (int e = threadIdx.x; e < len; e += kPjThreads) {
-        const int32_t s = succ[e];
-        if (s >= 0 && s < len) Q[s] = e;
-        V1[e] = w1[e];
-        V2[e] = w2[e];
-        F[e] = e;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int w = threadIdx.x + k * kTopThreads;
+        const int32_t e0 = w < int(H.S0) ? int32_t(H.elem(uint32_t(w))) : w == int(H.S0) && !head_split ? head : len;
+        int32_t e = e0, x1 = 0, x2 = 0, link = kEndT;
+        while (e >= 0 && e < len) {
+            const int32_t z = nx[e], y1 = a1[e], y2 = a2[e];
+            if (z < 0) {  // visited before: no list
+                set_status(status, ETL_EBADTREE);
+                break;
+            }
+            nx[e] = kVisited | w;
+            a1[e] = x1;
+            a2[e] = x2;
+            x1 += y1;
+            x2 += y2;
+            e = z;
+            if (z < len && H.split(uint32_t(z))) {
+                link = H.sid(uint32_t(z));
+                break;
+            }
+        }
+        Q[w] = -1;
+        V1[w] = x1;
+        V2[w] = x2;
+        F[w] = w;
+        SN[w] = link;
+    }
+    __syncthreads();
+    int32_t s1[2], s2[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int w = threadIdx.x + k * kTopThreads;
+        s1[k] = V1[w];
+        s2[k] = V2[w];
+        const int32_t s = SN[w];
+        if (s != kEndT) Q[s] = w;  // a link is a sublist id below kTopSub
     }
     __syncthreads();
     int rounds = 0;
     while (true) {
-        int32_t nq[kPjItems], n1[kPjItems], n2[kPjItems], nf[kPjItems];
+        int32_t nq[2], n1[2], n2[2], nf[2];
         int any = 0;
 #pragma unroll
-        for (int k = 0; k < kPjItems; ++k) {
-            const int e = threadIdx.x + k * kPjThreads;
-            if (e < len) {
-                const int32_t q = Q[e];
-                if (q >= 0) {
-                    nq[k] = Q[q];
-                    n1[k] = V1[e] + V1[q];
-                    n2[k] = V2[e] + V2[q];
-                    nf[k] = F[q];
-                    any = 1;
-                } else {
-                    nq[k] = -1;
-                    n1[k] = V1[e];
-                    n2[k] = V2[e];
-                    nf[k] = F[e];
-                }
+        for (int k = 0; k < 2; ++k) {
+            const int w = threadIdx.x + k * kTopThreads;
+            const int32_t q = Q[w];
+            if (q >= 0) {
+                nq[k] = Q[q];
+                n1[k] = V1[w] + V1[q];
+                n2[k] = V2[w] + V2[q];
+                nf[k] = F[q];
+                any = 1;
+            } else {
+                nq[k] = -1;
+                n1[k] = V1[w];
+                n2[k] = V2[w];
+                nf[k] = F[w];
             }
         }
         any = __syncthreads_or(any);
         if (!any) break;
-        if (++rounds > 40) {  // cannot happen on a valid list of <= 2^31 elements
+        if (++rounds > 40) {  // a cycle: cannot happen on a valid list
             if (threadIdx.x == 0) set_status(status, ETL_EBADTREE);
             break;
         }
 #pragma unroll
-        for (int k = 0; k < kPjItems; ++k) {
-            const int e = threadIdx.x + k * kPjThreads;
-            if (e < len) {
-                Q[e] = nq[k];
-                V1[e] = n1[k];
-                V2[e] = n2[k];
-                F[e] = nf[k];
-            }
+        for (int k = 0; k < 2; ++k) {
+            const int w = threadIdx.x + k * kTopThreads;
+            Q[w] = nq[k];
+            V1[w] = n1[k];
+            V2[w] = n2[k];
+            F[w] = nf[k];
         }
         __syncthreads();
     }
-    for (int e = threadIdx.x; e < len; e += kPjThreads) {
-        R[e] = V1[e] - w1[e];
-        O[e] = V2[e] - w2[e];
-        if (expect_total >= 0 && succ[e] == ETL_END && F[e] == head && int64_t(V1[e]) == expect_total) found = 1;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int w = threadIdx.x + k * kTopThreads;
+        if (expect_total >= 0 && SN[w] == kEndT && F[w] == head_sub && int64_t(V1[w]) == expect_total) found = 1;
+        V1[w] -= s1[k];  // exclusive
+        V2[w] -= s2[k];
     }
     __syncthreads();
     if (threadIdx.x == 0 && expect_total >= 0 && !found) set_status(status, ETL_EBADTREE);
-}
-
-__global__ void k_expand(const int4 *__restrict__ loc, int64_t len_base, const int32_t *__restrict__ d_len_add,
-                         int64_t cap, int64_t up_cap, const int32_t *__restrict__ Rup,
-                         const int32_t *__restrict__ Oup, int32_t *__restrict__ R, int32_t *__restrict__ O) {
-    pdl_prologue();
-    const int64_t len = level_len(len_base, d_len_add, cap);
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x) {
-        const int4 l = loc[e];
-        if (l.x >= 0 && l.x < up_cap) {  // elements off every list keep whatever was there
-            R[e] = Rup[l.x] + l.y;
-            O[e] = Oup[l.x] + l.z;
+    for (int e = threadIdx.x; e < len; e += kTopThreads) {
+        const int32_t z = nx[e];
+        if (z >= 0) continue;  // on no walk
+        const int32_t s = z & ~kVisited;
+        if (FROM_LIST) {
+            T[e] = make_int4(V1[s] + a1[e], V2[s] + a2[e], 0, 0);
+            const bool leaf = DUAL && int32_t(succ[e]) < ETL_END;
+            recs[e] = S::rec(e, 0, leaf ? 0x8000u : 0u, lb);
+        } else {
+            *reinterpret_cast<int2 *>(T + e) = make_int2(V1[s] + a1[e], V2[s] + a2[e]);
         }
     }
 }
 
-__global__ void k_set_i32(int32_t *p, int32_t v) {
+size_t top_smem(int64_t len) { return size_t(5 * kTopSub + 3 * len) * sizeof(int32_t); }
+
+// an entry's weights give way to the prefix over the whole list
+__global__ void k_expand(int4 *__restrict__ T, const int4 *__restrict__ loc, int64_t base,
+                         const int32_t *__restrict__ d_add, int64_t cap, const int4 *__restrict__ up, int64_t up_cap) {
     pdl_prologue();
-    *p = v;
+    const int64_t len = level_len(base, d_add, cap);
+    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x) {
+        const int4 l = __ldcs(loc + e);
+        if (l.z >= 0 && l.z < up_cap) {  // entries on no walk get whatever is there
+            const int2 u = __ldg(reinterpret_cast<const int2 *>(up + l.z));
+            *reinterpret_cast<int2 *>(T + e) = make_int2(u.x + l.x, u.y + l.y);
+        }
+    }
 }
 
-__global__ void k_final_rank(const uint2 *__restrict__ packed, int64_t len, const int32_t *__restrict__ R,
-                             int64_t rcap, int32_t *__restrict__ rank) {
+// succ -> slots of the in-place walk
+template <class S>
+__global__ void k_list_slots(const int32_t *succ, int64_t len, typename S::T *slots) {
     pdl_prologue();
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x) {
-        const uint2 p = packed[e];
-        rank[e] = p.x < rcap ? R[p.x] + int32_t(p.y & 0xffffu) : -1;
-    }
+    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x)
+        slots[e] = S::make(__ldcs(succ + e));
+}
+
+// rank and 4-byte records may be the same array
+__global__ void k_final_rank(RankResult rr, int64_t len, int32_t *rank) {
+    pdl_prologue();
+    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x)
+        rank[e] = rank_at(rr, e);
 }
 
 }  // namespace
@@ -365,153 +568,220 @@ RankParams &rank_params() {
     return p;
 }
 
-// Walks of a list whose successors and records (12 bytes per element) fit in about three quarters of
-// the 129 MB L2 run with every SM full of walkers; on longer lists P.blocks_per_sm blocks per SM: with
-// fewer random sectors in flight fewer are evicted before their reuse (measured on 2^25-element tours:
-// 19% less DRAM traffic, and faster, with 512 walkers per SM than with 2048).
-constexpr int64_t kWalkL2Bytes = int64_t(96) << 20;
+// Successors and records (8 bytes per element, 12 in dual mode) of up to 96 of the 129 MB L2 are kept in
+// separate arrays; longer lists are ranked in place.
+bool rank_in_place(int64_t len, bool dual) { return len * (dual ? 12 : 8) > (int64_t(96) << 20); }
 
-// Level-0 splitter density (log2 of elements per splitter). A list longer than 2^22 elements takes
-// the tuned value (P.k0_log2): its walks are bound by DRAM traffic, which sparser splitters reduce.
-// A shorter list sits in L2 and its walk is bound by the latency of its longest sublist (about
-// 2^k * ln(len / 2^k) dependent steps), so it takes denser splitters: one in 4 up to 2^15 elements,
-// one in 8 up to 2^20, one in 16 up to 2^22, or the tuned value if that is denser (measured on
-// random recursive trees of 2^11 .. 2^22 nodes and on forest tours of 2^12 .. 2^22-node graphs).
-int level0_density(int64_t len, const RankParams &P) {
-    if (len > (int64_t(1) << 22)) return P.k0_log2;
-    const int k = len > (int64_t(1) << 20) ? 4 : len > (int64_t(1) << 15) ? 3 : 2;
-    return k < P.k0_log2 ? k : P.k0_log2;
+namespace {
+
+int grid_of(int64_t lanes, int64_t per_sm, const RankParams &P) {
+    const int64_t most = int64_t(num_sms()) * (per_sm > 0 ? per_sm : 1);
+    return int(std::max<int64_t>(1, std::min(most, ceil_div(lanes, P.block))));
 }
 
-// ... and never more walkers than sublists: on a short list the surplus warps would only contend for
-// the work counter before finding nothing to walk
-int walk_grid(int64_t len, int64_t bytes_per_elem, int64_t sublists, const RankParams &P) {
-    const int per_sm = len * bytes_per_elem > kWalkL2Bytes ? P.blocks_per_sm : 2048 / P.block;
-    const int64_t grid = int64_t(num_sms()) * (per_sm > 0 ? per_sm : 1);
-    const int64_t need = ceil_div(sublists, P.block);
-    return int(need < grid ? (need > 0 ? need : 1) : grid);
+// splitters of a level of len entries, one in 2^k of the hashed range; if that is at most twice the
+// top's capacity, as many as the top takes (one level less, or shorter walks), but one in two at most
+uint32_t splitters(int64_t len, int k) {
+    const uint32_t range = uint32_t(uint64_t(1) << ceil_log2(uint64_t(len)));
+    const uint32_t s = std::max(1u, range >> k);
+    return s < 2u * kTopCap ? std::max(std::min(s, uint32_t(kTopCap - 1)), std::min(range >> 1, uint32_t(kTopCap - 1))) : s;
 }
 
-etl_status list_rank(const int32_t *succ, int64_t n_cap, const int32_t *d_len, const int32_t *d_head, bool dual,
-                     int64_t expect_len, int32_t *status, Workspace &ws, RankResult *out) {
-    (void)d_len;  // level 0 always spans the whole array; inert slots carry succ = -1
-    cudaStream_t s = ws.stream();
-    const RankParams &P = rank_params();
-    cudaFuncSetAttribute(k_pointer_jump, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kPjCap * 4);
-
-    // ---- level 0: implicit weights, packed 16-bit local offsets
-    const int64_t len0 = n_cap;
-    Hash H = make_hash(len0, level0_density(len0, P));
-    int32_t dyn_cap = int32_t(len0 / kLcap + 2);
-    int64_t cap1 = int64_t(H.S0) + 1 + dyn_cap;
-    uint2 *packed = ws.get<uint2>(len0);
-    int32_t *rnext = ws.get<int32_t>(cap1), *rw1 = ws.get<int32_t>(cap1), *rw2 = ws.get<int32_t>(cap1);
-    int32_t *ctr = ws.get<int32_t>(2);
-    int32_t *head1 = ws.get<int32_t>(1);
-    if (!ws.ok()) return ETL_ENOMEM;
-    memset_async(ctr, 0, 2 * sizeof(int32_t), s);
+// A: where scratch comes from (get<T>(count); a null pointer when there is none). list: len 4-byte
+// successors, recs: room for len records (or null: taken from alloc); in place: list = slots S::T
+template <class S, bool DUAL, class A>
+etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head, int32_t head, int64_t expect_len,
+                     int32_t *status, const RankParams &P, A &alloc, cudaStream_t s, RankResult *out) {
+    using R = typename S::T;
+    const bool in_place = rank_in_place(len, DUAL);
+    out->wide = sizeof(R) == 8;
+    out->lb = out->wide ? 16 : 12;
+    if (in_place) recs = list;
+    if (!recs) recs = alloc.template get<R>(len);
+    if (!recs) return ETL_ENOMEM;
+    out->recs = recs;
+    const uint32_t *succ = static_cast<const uint32_t *>(list);
+    cudaFuncSetAttribute(k_top<S, DUAL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap)));
+    cudaFuncSetAttribute(k_top<S, DUAL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap)));
     etl_status st;
-    {
+    if (len <= kTopCap) {
+        int4 *T = alloc.template get<int4>(len);
+        if (!T) return ETL_ENOMEM;
+        out->T = T;
+        out->rcap = len;
+        PhaseTimer pt("rank.top", s);
+        launch(k_top<S, DUAL, true>, 1, kTopThreads, top_smem(len), s, succ, static_cast<R *>(recs), out->lb, T, len,
+               nullptr, len, d_head, head, expect_len, status);
+        note_launch();
+        return last_launch();
+    }
+
+    struct Level {
+        int4 *T, *loc;
+        int64_t base, cap;  // entries: base + *d_add, at most cap
+        const int32_t *d_add, *d_head;
+    };
+    Level lv[32];
+    int nl = 0;
+    int32_t *words = alloc.template get<int32_t>(64);  // per level: [2 i] entry count, [2 i + 1] head
+    if (!words) return ETL_ENOMEM;
+    memset_async(words, 0, sizeof(int32_t), s);
+    if (in_place) {
+        Walk0 w{};
+        w.len = len;
+        w.d_head = d_head;
+        w.head = head;
+        const int64_t per_lane = int64_t(1) << (P.k0_log2 - 1);
+        const int grid = grid_of(len / per_lane, P.blocks_per_sm, P);
+        const int64_t lanes = int64_t(grid) * P.block;
+        w.nclaims = uint32_t(std::min(16 * lanes, len / 3) + 1);
+        w.start = int32_t(lanes / kWarp * SidPool::kFirst);
+        w.limit = int32_t(8 * lanes);
+        // sublist id and local offset share 31 bits of a 4-byte record: the longest offset for which
+        // they fit (8 bits for 2^30 elements). A warp may pass the limit once, by up to 32 ids.
+        for (w.lb = out->wide ? 16 : 12;; --w.lb) {
+            w.lcap = out->wide ? kLcap : (1 << w.lb) - 1;
+            w.cap = int32_t(9 * lanes + len / w.lcap + 2);
+            if (out->wide || int64_t(w.cap) <= (int64_t(1) << (31 - w.lb)) || w.lb <= 4) break;
+        }
+        out->lb = w.lb;
+        int4 *T = alloc.template get<int4>(w.cap);
+        if (!T) return ETL_ENOMEM;
+        lv[nl++] = Level{T, nullptr, w.start, w.cap, words, words + 1};
         PhaseTimer pt0("rank.walk0", s);
-        const int grid = walk_grid(len0, 12, int64_t(H.S0) + 1, P);
-        if (dual)
-            launch(k_walk0<true>, grid, P.block, 0, s, succ, len0, d_head, H, packed, rnext, rw1, rw2, ctr, dyn_cap,
-                   head1, status);
-        else
-            launch(k_walk0<false>, grid, P.block, 0, s, succ, len0, d_head, H, packed, rnext, rw1, rw2, ctr, dyn_cap,
-                   head1, status);
+        launch(k_walk0_in_place<S, DUAL>, grid, P.block, 0, s, static_cast<R *>(recs), w, T, words, words + 1, status);
+        note_launch();
+        st = last_launch();
+    } else {
+        const int k = std::min(P.k0_log2, len > (int64_t(1) << 20) ? 4 : 3);
+        Hash H;
+        H.mask = uint32_t((uint64_t(1) << ceil_log2(uint64_t(len))) - 1);
+        uint32_t lcap;
+        int32_t dyn_cap, cap;
+        for (;; --out->lb) {  // as above
+            lcap = out->wide ? uint32_t(kLcap) : (1u << out->lb) - 1u;
+            dyn_cap = int32_t(len / lcap + 2);
+            H.S0 = splitters(len, k);
+            // ids of dynamic sublists come out of the same power of two, so that the next level's hash
+            // does not cover twice the entries
+            H.S0 -= std::min(H.S0 / 2, uint32_t(dyn_cap) + 1);
+            cap = int32_t(H.S0) + 1 + dyn_cap;
+            if (out->wide || int64_t(cap) <= (int64_t(1) << (31 - out->lb)) || out->lb <= 4) break;
+        }
+        int4 *T = alloc.template get<int4>(cap);
+        if (!T) return ETL_ENOMEM;
+        lv[nl++] = Level{T, nullptr, int64_t(H.S0) + 1, cap, words, words + 1};
+        PhaseTimer pt0("rank.walk0", s);
+        launch(k_walk0<S, DUAL>, grid_of(int64_t(H.S0) + 1, 2048 / P.block, P), P.block, 0, s, succ, len, d_head, head,
+               H, static_cast<R *>(recs), out->lb, lcap, T, words, cap, words + 1, status);
         note_launch();
         st = last_launch();
     }
     if (st) return st;
 
-    struct Level {
-        const int32_t *succ, *w1, *w2;
-        int64_t base, cap;
-        const int32_t *d_add, *d_head;
-        int4 *loc;
-        int32_t *R, *O;
-    };
-    std::vector<Level> lv;
-    lv.push_back(Level{rnext, rw1, rw2, int64_t(H.S0) + 1, cap1, ctr + 1, head1, nullptr, nullptr, nullptr});
-
     // ---- upper levels until one CTA can finish the reduced list
-    while (lv.back().cap > kPjCap) {
-        Level &L = lv.back();
-        Hash h = make_hash(L.cap, P.k_log2);
-        int32_t dcap = int32_t(L.cap / kLcap + 2);
-        int64_t ncap = int64_t(h.S0) + 1 + dcap;
-        L.loc = ws.get<int4>(L.cap);
-        int32_t *nn = ws.get<int32_t>(ncap), *n1 = ws.get<int32_t>(ncap), *n2 = ws.get<int32_t>(ncap);
-        int32_t *c = ws.get<int32_t>(2), *hd = ws.get<int32_t>(1);
-        if (!ws.ok()) return ETL_ENOMEM;
-        memset_async(c, 0, 2 * sizeof(int32_t), s);
-        memset_async(L.loc, 0xff, size_t(L.cap) * sizeof(int4), s);
+    while (lv[nl - 1].cap > kTopCap) {
+        Level &L = lv[nl - 1];
+        const uint32_t most = splitters(L.cap, P.k_log2);
+        L.loc = alloc.template get<int4>(L.cap);
+        int4 *up = alloc.template get<int4>(int64_t(most) + 1);
+        if (!L.loc || !up || nl >= 32) return ETL_ENOMEM;
         {
             PhaseTimer ptw("rank.walk", s);
-            const int grid = walk_grid(L.cap, 28, int64_t(h.S0) + 1, P);
-            launch(k_walk, grid, P.block, 0, s, L.succ, L.w1, L.w2, L.base, L.d_add, L.cap, L.d_head, h, L.loc, nn, n1,
-                   n2, c, dcap, hd, status);
-        note_launch();
+            launch(k_walk, grid_of(int64_t(most) + 1, 2048 / P.block, P), P.block, 0, s, L.T, L.base, L.d_add, L.cap,
+                   L.d_head, most < uint32_t(kTopCap) ? 0 : P.k_log2, most, L.loc, up, words + 2 * nl,
+                   words + 2 * nl + 1, status);
+            note_launch();
             st = last_launch();
         }
         if (st) return st;
-        lv.push_back(Level{nn, n1, n2, int64_t(h.S0) + 1, ncap, c + 1, hd, nullptr, nullptr, nullptr});
+        lv[nl] = Level{up, nullptr, 0, int64_t(most) + 1, words + 2 * nl, words + 2 * nl + 1};
+        ++nl;
     }
 
     // ---- top
     {
-        Level &T = lv.back();
-        T.R = ws.get<int32_t>(T.cap);
-        T.O = ws.get<int32_t>(T.cap);
-        if (!ws.ok()) return ETL_ENOMEM;
-        PhaseTimer ptp("rank.pj", s);
-        launch(k_pointer_jump, 1, kPjThreads, 4 * kPjCap * 4, s, T.succ, T.w1, T.w2, T.base, T.d_add, T.cap, T.d_head,
-               expect_len, T.R, T.O, status);
+        const Level &L = lv[nl - 1];
+        PhaseTimer ptp("rank.top", s);
+        launch(k_top<S, DUAL, false>, 1, kTopThreads, top_smem(L.cap), s, nullptr, nullptr, 0, L.T, L.base, L.d_add,
+               L.cap, L.d_head, 0, expect_len, status);
         note_launch();
         st = last_launch();
         if (st) return st;
     }
     // ---- push prefixes back down
-    for (int i = int(lv.size()) - 2; i >= 0; --i) {
-        Level &L = lv[i];
-        L.R = ws.get<int32_t>(L.cap);
-        L.O = ws.get<int32_t>(L.cap);
-        if (!ws.ok()) return ETL_ENOMEM;
+    for (int i = nl - 2; i >= 0; --i) {
+        const Level &L = lv[i];
         int blocks = int(ceil_div(L.cap, 256));
         if (blocks > num_sms() * 32) blocks = num_sms() * 32;  // four waves of full occupancy
         PhaseTimer pte("rank.expand", s);
-        launch(k_expand, blocks, 256, 0, s, L.loc, L.base, L.d_add, L.cap, lv[i + 1].cap, lv[i + 1].R, lv[i + 1].O, L.R,
-               L.O);
+        launch(k_expand, blocks, 256, 0, s, L.T, L.loc, L.base, L.d_add, L.cap, lv[i + 1].T, lv[i + 1].cap);
         note_launch();
         st = last_launch();
         if (st) return st;
     }
-    out->packed = packed;
-    out->R = lv[0].R;
-    out->O = lv[0].O;
+    out->T = lv[0].T;
     out->rcap = lv[0].cap;
     return ETL_OK;
 }
 
-etl_status set_device_i32(int32_t *p, int32_t v, cudaStream_t s) {
-    launch(k_set_i32, 1, 1, 0, s, p, v);
+// The records take the place of the ranks, unless the caller's two arrays overlap.
+template <class A>
+etl_status rank_plain_list(const int32_t *succ, int64_t len, int32_t head, int32_t *rank, int32_t *status,
+                           const RankParams &P, A &alloc, cudaStream_t s) {
+    const bool wide = wide_slots(len), in_place = rank_in_place(len, false);
+    const bool overlap = succ < rank + len && rank < succ + len;
+    void *recs = wide ? static_cast<void *>(alloc.template get<Slot8::T>(len))
+                      : (overlap && !in_place) ? static_cast<void *>(alloc.template get<Slot4::T>(len)) : rank;
+    if (!recs) return ETL_ENOMEM;
+    int blocks = int(ceil_div(len, 256));
+    if (blocks > num_sms() * 16) blocks = num_sms() * 16;
+    void *list = const_cast<int32_t *>(succ);
+    if (in_place) {
+        PhaseTimer pt("rank.slots", s);
+        if (wide)
+            launch(k_list_slots<Slot8>, blocks, 256, 0, s, succ, len, static_cast<Slot8::T *>(recs));
+        else
+            launch(k_list_slots<Slot4>, blocks, 256, 0, s, succ, len, static_cast<Slot4::T *>(recs));
         note_launch();
+        list = recs;
+    }
+    etl_status rc = last_launch();
+    RankResult rr{};
+    if (!rc)
+        rc = wide ? rank_impl<Slot8, false>(list, recs, len, nullptr, head, len, status, P, alloc, s, &rr)
+                  : rank_impl<Slot4, false>(list, recs, len, nullptr, head, len, status, P, alloc, s, &rr);
+    if (rc) return rc;
+    PhaseTimer pt("rank.final", s);
+    launch(k_final_rank, blocks, 256, 0, s, rr, len, rank);
+    note_launch();
     return last_launch();
 }
 
-etl_status final_rank(const RankResult &r, int64_t len, int32_t *rank, cudaStream_t s) {
-    int blocks = int(ceil_div(len, 256));
-    const int cap = num_sms() * 16;
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    PhaseTimer pt("rank.final", s);
-    launch(k_final_rank, blocks, 256, 0, s, r.packed, len, r.R, r.rcap, rank);
-        note_launch();
-    return last_launch();
+}  // namespace
+
+etl_status list_rank(void *list, int64_t len, const int32_t *d_head, int32_t head, bool dual, int64_t expect_len,
+                     int32_t *status, Workspace &ws, RankResult *out) {
+    cudaStream_t s = ws.stream();
+    const RankParams &P = rank_params();
+    if (dual) return rank_impl<Slot8, true>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
+    if (wide_slots(len))
+        return rank_impl<Slot8, false>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
+    return rank_impl<Slot4, false>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
 }
 
 }  // namespace etl
+
+extern "C" etl_status etl_list_rank(const int32_t *succ, int64_t len, int32_t head, int32_t *rank, int32_t *status,
+                                    void *stream) {
+    using namespace etl;
+    if (!succ || !rank || len < 1 || len > int64_t(INT32_MAX) - 1 || head < 0 || head >= len) return ETL_EINVAL;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    Workspace ws(s);
+    int32_t *st = status ? status : ws.get<int32_t>(1);
+    if (!ws.ok()) return ETL_ENOMEM;
+    return rank_plain_list(succ, len, head, rank, st, rank_params(), ws, s);
+}
 
 // ------------------------------------------------------------------ list ranking without allocation
 //
@@ -547,7 +817,6 @@ namespace {
 
 constexpr int64_t kStaticMaxLen = int64_t(1) << 18;
 constexpr size_t kStaticBytes = size_t(3) << 20;
-constexpr int kStaticK0 = 4, kStaticK = 4;  // fixed splitter densities, so the layout is fixed
 
 static __device__ __align__(256) unsigned char g_rank_scratch[kStaticBytes];
 
@@ -555,7 +824,7 @@ struct StaticArena {
     char *base;
     size_t used, cap;
     template <class T>
-    T *take(int64_t count) {
+    T *get(int64_t count) {
         size_t off = (used + 255) & ~size_t(255);
         size_t bytes = size_t(count > 0 ? count : 1) * sizeof(T);
         if (off + bytes > cap) return nullptr;
@@ -607,9 +876,6 @@ etl_status static_scratch(void **out) {
     if (!g_static_addr[dev] || (have_id && g_static_ctx[dev] != id)) {
         void *p = nullptr;
         if (cudaGetSymbolAddress(&p, g_rank_scratch) != cudaSuccess || !p) return ETL_ECUDA;
-        if (cudaFuncSetAttribute(k_pointer_jump, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kPjCap * 4) !=
-            cudaSuccess)
-            return ETL_ECUDA;
         // the look-up made the device's primary context current if it was not yet
         g_static_ctx[dev] = current_context_id(&id) ? id : 0;
         g_static_addr[dev] = p;
@@ -631,78 +897,12 @@ extern "C" etl_status etl_list_rank_static(const int32_t *succ, int64_t len, int
     etl_status rc = static_scratch(&scratch);
     if (rc) return rc;
     StaticArena A{static_cast<char *>(scratch), 0, kStaticBytes};
-    const int grid = num_sms() * 8;
-    const int block = 256;
-
-    int32_t *word = A.take<int32_t>(4);  // [0] head, [1] status when the caller passes none
-    int32_t *st = status ? status : word + 1;
-    Hash H = make_hash(len, kStaticK0);
-    const int32_t dyn_cap = int32_t(len / kLcap + 2);
-    const int64_t cap1 = int64_t(H.S0) + 1 + dyn_cap;
-    uint2 *packed = A.take<uint2>(len);
-    int32_t *rnext = A.take<int32_t>(cap1), *rw1 = A.take<int32_t>(cap1), *rw2 = A.take<int32_t>(cap1);
-    int32_t *ctr = A.take<int32_t>(2), *head1 = A.take<int32_t>(1);
-    if (!word || !packed || !rnext || !rw1 || !rw2 || !ctr || !head1) return ETL_ENOMEM;
-
-    if (!status && cudaMemsetAsync(st, 0, sizeof(int32_t), s) != cudaSuccess) return ETL_ECUDA;
-    if (cudaMemsetAsync(ctr, 0, 2 * sizeof(int32_t), s) != cudaSuccess) return ETL_ECUDA;
-    launch(k_set_i32, 1, 1, 0, s, word, head);
-    note_launch();
-    launch(k_walk0<false>, grid, block, 0, s, succ, len, word, H, packed, rnext, rw1, rw2, ctr, dyn_cap, head1, st);
-    note_launch();
-    if ((rc = last_launch())) return rc;
-
-    struct Level {
-        const int32_t *succ, *w1, *w2;
-        int64_t base, cap;
-        const int32_t *d_add, *d_head;
-        int4 *loc;
-        int32_t *R, *O;
-    };
-    Level lv[8];
-    int nl = 0;
-    lv[nl++] = Level{rnext, rw1, rw2, int64_t(H.S0) + 1, cap1, ctr + 1, head1, nullptr, nullptr, nullptr};
-    while (lv[nl - 1].cap > kPjCap) {
-        if (nl >= 8) return ETL_ENOMEM;
-        Level &L = lv[nl - 1];
-        Hash h = make_hash(L.cap, kStaticK);
-        const int32_t dcap = int32_t(L.cap / kLcap + 2);
-        const int64_t ncap = int64_t(h.S0) + 1 + dcap;
-        L.loc = A.take<int4>(L.cap);
-        int32_t *nn = A.take<int32_t>(ncap), *n1 = A.take<int32_t>(ncap), *n2 = A.take<int32_t>(ncap);
-        int32_t *c = A.take<int32_t>(2), *hd = A.take<int32_t>(1);
-        if (!L.loc || !nn || !n1 || !n2 || !c || !hd) return ETL_ENOMEM;
-        if (cudaMemsetAsync(c, 0, 2 * sizeof(int32_t), s) != cudaSuccess) return ETL_ECUDA;
-        if (cudaMemsetAsync(L.loc, 0xff, size_t(L.cap) * sizeof(int4), s) != cudaSuccess) return ETL_ECUDA;
-        launch(k_walk, grid, block, 0, s, L.succ, L.w1, L.w2, L.base, L.d_add, L.cap, L.d_head, h, L.loc, nn, n1, n2, c,
-               dcap, hd, st);
-        note_launch();
-        if ((rc = last_launch())) return rc;
-        lv[nl++] = Level{nn, n1, n2, int64_t(h.S0) + 1, ncap, c + 1, hd, nullptr, nullptr, nullptr};
+    int32_t *st = status;
+    if (!st) {
+        st = A.get<int32_t>(1);
+        if (cudaMemsetAsync(st, 0, sizeof(int32_t), s) != cudaSuccess) return ETL_ECUDA;
     }
-    Level &T = lv[nl - 1];
-    T.R = A.take<int32_t>(T.cap);
-    T.O = A.take<int32_t>(T.cap);
-    if (!T.R || !T.O) return ETL_ENOMEM;
-    launch(k_pointer_jump, 1, kPjThreads, 4 * kPjCap * 4, s, T.succ, T.w1, T.w2, T.base, T.d_add, T.cap, T.d_head, len,
-           T.R, T.O, st);
-    note_launch();
-    if ((rc = last_launch())) return rc;
-    for (int i = nl - 2; i >= 0; --i) {
-        Level &L = lv[i];
-        L.R = A.take<int32_t>(L.cap);
-        L.O = A.take<int32_t>(L.cap);
-        if (!L.R || !L.O) return ETL_ENOMEM;
-        int blocks = int(ceil_div(L.cap, 256));
-        if (blocks > grid * 4) blocks = grid * 4;
-        launch(k_expand, blocks, 256, 0, s, L.loc, L.base, L.d_add, L.cap, lv[i + 1].cap, lv[i + 1].R, lv[i + 1].O, L.R,
-               L.O);
-        note_launch();
-        if ((rc = last_launch())) return rc;
-    }
-    int blocks = int(ceil_div(len, 256));
-    if (blocks > num_sms() * 16) blocks = num_sms() * 16;
-    launch(k_final_rank, blocks, 256, 0, s, packed, len, lv[0].R, lv[0].cap, rank);
-    note_launch();
-    return last_launch();
+    // fixed parameters, so that the layout is fixed (1.6 MB at the largest length; the slots are in the
+    // caller's rank array)
+    return rank_plain_list(succ, len, head, rank, st, RankParams{}, A, s);
 }
