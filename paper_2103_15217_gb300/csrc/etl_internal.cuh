@@ -176,19 +176,14 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 etl_status scan_exclusive_i32(const int32_t *in, int32_t *out, int64_t n, Workspace &ws);
 etl_status scan_exclusive_u8(const uint8_t *in, int32_t *out, int64_t n, Workspace &ws);
 
-// Stable LSD radix sort of (key, value) pairs by key, keys in [0, key_limit)
-// with key_limit <= 2^key_bits. Elements are in[0..count) where count =
-// *d_count if d_count != null else n_cap. With vals_in == null the value of
-// element i is i. Elements whose key is outside [0, key_limit) are dropped
-// (they do not appear in the output). On return kv points at the sorted
-// (key, value) pairs (inside the workspace) and *d_total (device) holds the
-// number of elements kept.
-struct SortResult {
-    const int2 *kv;
-    const int32_t *d_total;
-};
-etl_status radix_sort_pairs(const int32_t *keys_in, const int32_t *vals_in, const int32_t *d_count, int64_t n_cap,
-                            int key_bits, int32_t key_limit, Workspace &ws, SortResult *out);
+// Children of every node in ascending label order: head[v] = first child or -1, next[c] = next sibling
+// or -1 (-1 for roots too). parent: ids in [0, n), -1 at roots; anything else is dropped and sets the
+// status. For a batch, off / inst_of / bad say which instance a node belongs to (*bad: drop all), ids
+// are local to it, and gparent receives the global ones (-1 at roots, -2: dropped). root_cnt / root_of
+// (zeroed by the caller): roots per instance and the last one seen.
+etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, const int32_t *inst_of,
+                         const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
+                         int32_t *root_of, int32_t *status, Workspace &ws);
 
 // ----------------------------------------------------------------- list ranking
 
@@ -269,7 +264,7 @@ struct RankParams {
 RankParams &rank_params();
 
 struct SortParams {
-    int rounds = 8;       // 32-element rounds per warp in the radix passes: tiles of 256 * rounds elements
+    int rounds = 8;       // 32-element rounds per warp in the radix passes over long families: tiles of 256 * rounds
     bool ballot = true;   // rank equal digits in a warp by ballots instead of __match_any_sync
 };
 SortParams &sort_params();

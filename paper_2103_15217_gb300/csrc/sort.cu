@@ -1,70 +1,158 @@
-// Stable LSD radix sort of (key, value) int32 pairs, 8 bits per pass.
+// Children of every node in ascending label order, as linked lists (the grouping step of Sec. 2.1: the
+// paper sorts the arcs; a tour only needs each node's first child and next sibling).
 //
-// Used to group the arcs of a tree by their source node: children by parent
-// for a parent array, half-edges by tail for a spanning forest. This replaces
-// the lexicographic sort of array A into B in the DCEL construction of
-// Sec. 2.1: only the grouping by source is needed, and a stable sort keeps
-// each group in ascending value order.
-//
-// One pass = per-tile digit histograms -> exclusive scan over (digit, tile) ->
-// stable scatter. Inside a tile each warp ranks its 32-element rounds (peers
-// with the same digit by __match_any_sync or by eight ballots) with per-warp
-// smem counters, so the order of equal digits is preserved without any atomics
-// on global memory; the ranked tile is staged in shared memory in digit order
-// and written out in runs.
+//  * k_link_children pushes every node onto its parent's list, highest labels first:
+//    next[c] = exchange(head[parent[c]], c). Blocks start in the order of their index, so almost every
+//    list comes out ascending; only siblings whose pushes were in flight together can be swapped. The
+//    lanes of a warp that share a parent are linked by the warp and pushed as one run. One random
+//    exchange in an array of n words per node: 2^24 nodes in 0.13 ms, where counting the children,
+//    scanning the counts and a stable 3-pass radix sort of (parent, child) pairs took 0.54 ms, and a
+//    random tree's successors another 0.17 ms of random writes that the lists do not need.
+//  * k_check_children finds every link that does not ascend and sorts that family's list on the spot
+//    (up to kLight children, by one thread).
+//  * k_sort_heavy does longer families that are out of order: a stable LSD radix sort of their
+//    (parent, child) pairs, 8 bits per pass, in one cooperative launch, which returns at once when
+//    there are none (3 us). Inside a tile each warp ranks its 32-element rounds (peers with the same
+//    digit by __match_any_sync or by eight ballots) with per-warp smem counters; the ranked tile is
+//    staged in shared memory in digit order and written out in runs.
 #include "etl_internal.cuh"
 
 namespace etl {
 namespace {
 
+__device__ __forceinline__ int64_t gtid() { return blockIdx.x * int64_t(blockDim.x) + threadIdx.x; }
+__device__ __forceinline__ int64_t gstride() { return int64_t(gridDim.x) * blockDim.x; }
+
+constexpr int kLinkThreads = 256;
+constexpr int kLinkIlp = 2;  // labels per thread, from the highest down (1: 0.16 ms, 4: more siblings in flight together)
+constexpr int kLight = 32;   // children of a family that one thread sorts
+
+// off / inst_of / bad (batches): ids are local to the node's instance, gparent receives global ones
+template <bool BATCH>
+__global__ void __launch_bounds__(kLinkThreads)
+    k_link_children(const int32_t *__restrict__ parent, int32_t n, const int32_t *__restrict__ off,
+                    const int32_t *__restrict__ inst_of, const int32_t *__restrict__ bad,
+                    int32_t *__restrict__ gparent, int32_t *__restrict__ head, int32_t *__restrict__ next,
+                    int32_t *__restrict__ root_cnt, int32_t *__restrict__ root_of, int32_t *__restrict__ status) {
+    pdl_prologue();
+    const bool bad_offsets = BATCH && *bad;
+    const int64_t top = int64_t(gridDim.x - blockIdx.x) * (kLinkThreads * kLinkIlp);
+    int32_t par[kLinkIlp];
+#pragma unroll
+    for (int j = 0; j < kLinkIlp; ++j) {
+        const int64_t t = top - int64_t(j + 1) * kLinkThreads + threadIdx.x;
+        par[j] = t < n ? __ldcs(parent + t) : -1;
+    }
+#pragma unroll
+    for (int j = 0; j < kLinkIlp; ++j) {
+        const int64_t t = top - int64_t(j + 1) * kLinkThreads + threadIdx.x;
+        const int32_t v = int32_t(t), p = par[j];
+        int32_t g = -2;
+        if (t < n && !bad_offsets) {
+            int32_t inst = 0, base = 0, size = n;
+            if (BATCH) {
+                inst = inst_of[v];
+                base = off[inst];
+                size = off[inst + 1] - base;
+            }
+            if (p == -1) {
+                atomicAdd(&root_cnt[inst], 1);
+                root_of[inst] = v;
+                g = -1;
+            } else if (p < 0 || p >= size) {
+                set_status(status, ETL_EBADTREE);
+            } else {
+                g = p + base;
+                if (g == v) set_status(status, ETL_EBADTREE);
+            }
+        }
+        // lanes with the same parent form one run, linked in label order; its first lane pushes it
+        const int lane = threadIdx.x & 31;
+        const unsigned peers = __match_any_sync(kFull, g >= 0 ? g : -2 - lane);
+        const int first = __ffs(peers) - 1;
+        int32_t old = -1;
+        if (g >= 0 && lane == first) old = atomicExch(head + g, v);
+        old = __shfl_sync(kFull, old, first);
+        const unsigned above = lane < 31 ? peers >> (lane + 1) : 0u;
+        if (t < n) {
+            __stcs(next + v, above ? v + __ffs(above) : old);
+            if (BATCH) gparent[v] = g;
+        }
+    }
+}
+
+// Every link must ascend. The first to see one of a family that does not takes the family (its bit in
+// `seen`) and puts it on its block's list; the block sorts those together (one thread each), so that
+// the few walks do not hold up warps that are checking: 2^24 nodes of a random tree 0.19 -> 0.06 ms.
+// Threads that check may read links being rewritten; whatever they see, they find the bit set. On a
+// small tree most families have to be sorted, by as many blocks as there are (ILP 1).
+constexpr int kCheckThreads = 256;
+constexpr int64_t kCheckSmall = int64_t(1) << 19;
+
+__device__ void sort_family(int32_t p, int32_t n, int32_t *head, int32_t *next, uint32_t *heavy, int32_t *heavy_count) {
+    int32_t kids[kLight];
+    int k = 0;
+    int32_t c = __ldcg(head + p);
+    for (; c >= 0 && c < n && k < kLight; ++k) {  // insertion into ascending order
+        int i = k;
+        for (; i > 0 && kids[i - 1] > c; --i) kids[i] = kids[i - 1];
+        kids[i] = c;
+        c = __ldcg(next + c);
+    }
+    if (c >= 0) {  // too many for one thread
+        atomicOr(heavy + (p >> 5), 1u << (p & 31));
+        atomicAdd(heavy_count, 1);
+        return;
+    }
+    head[p] = kids[0];
+    for (int i = 0; i < k; ++i) next[kids[i]] = i + 1 < k ? kids[i + 1] : -1;
+}
+
+template <int ILP>
+__global__ void __launch_bounds__(kCheckThreads)
+    k_check_children(const int32_t *__restrict__ par, int32_t n, int32_t *head, int32_t *next,
+                     uint32_t *__restrict__ seen, uint32_t *__restrict__ heavy, int32_t *__restrict__ heavy_count) {
+    pdl_prologue();
+    constexpr int kTile = kCheckThreads * ILP;
+    __shared__ int32_t todo[2 * kTile];
+    __shared__ int count;
+    if (threadIdx.x == 0) count = 0;
+    __syncthreads();
+    const int64_t step = int64_t(gridDim.x) * kTile;
+    for (int64_t base = int64_t(blockIdx.x) * kTile; base < n; base += step) {
+        int32_t x[ILP];
+#pragma unroll
+        for (int j = 0; j < ILP; ++j) {
+            const int64_t t = base + j * kCheckThreads + threadIdx.x;
+            x[j] = t < n ? __ldcg(next + t) : -1;
+        }
+#pragma unroll
+        for (int j = 0; j < ILP; ++j) {
+            const int64_t t = base + j * kCheckThreads + threadIdx.x;
+            if (x[j] < 0 || x[j] > t) continue;
+            const int32_t p = par[t];
+            const uint32_t bit = 1u << (p & 31);
+            if (p >= 0 && p < n && !(atomicOr(seen + (p >> 5), bit) & bit)) todo[atomicAdd(&count, 1)] = p;
+        }
+        __syncthreads();
+        const int found = count;
+        if (found > kTile || base + step >= n) {
+            for (int i = threadIdx.x; i < found; i += kCheckThreads) sort_family(todo[i], n, head, next, heavy, heavy_count);
+            __syncthreads();
+            if (threadIdx.x == 0) count = 0;
+        }
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------ long families out of order
+
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / kWarp;
 constexpr int kRadix = 256;
 static_assert(kThreads == kRadix, "the scatter handles one digit per thread");
-// R = 32-element rounds per warp: a tile of 8 warps holds 256 * R elements (R = 8 or 16, chosen by
-// the SORT_ROUNDS tuning knob; larger tiles give longer runs per digit in the scatter)
-
-__device__ __forceinline__ int64_t count_of(const int32_t *d_count, int64_t n_cap) {
-    if (!d_count) return n_cap;
-    int64_t c = *d_count;
-    return c < 0 ? 0 : (c < n_cap ? c : n_cap);
-}
-
-// keys of the input: a plain array (first pass) or the .x of (key, value) pairs (later passes)
-__device__ __forceinline__ int32_t key_at(const int32_t *keys, const int2 *kv, int64_t i) {
-    return kv ? kv[i].x : keys[i];
-}
-
-template <int R>
-__global__ void __launch_bounds__(kThreads)
-    k_hist(const int32_t *__restrict__ keys, const int2 *__restrict__ kv, const int32_t *d_count, int64_t n_cap,
-           int shift, int32_t key_limit, int32_t *__restrict__ ghist, int nblocks) {
-    pdl_prologue();
-    constexpr int kRounds = R, kWarpTile = kWarp * R, kTile = kWarps * kWarpTile;
-    __shared__ int32_t h[kRadix];
-    const int64_t count = count_of(d_count, n_cap);
-    if (int64_t(blockIdx.x) * kTile >= count) {  // tile past the data: an all-zero histogram
-        for (int d = threadIdx.x; d < kRadix; d += kThreads) ghist[int64_t(d) * nblocks + blockIdx.x] = 0;
-        return;
-    }
-    for (int d = threadIdx.x; d < kRadix; d += kThreads) h[d] = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t base = int64_t(blockIdx.x) * kTile + warp * kWarpTile;
-    int32_t key[kRounds];
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {  // loads first, all in flight together
-        const int64_t idx = base + r * kWarp + lane;
-        key[r] = idx < count ? key_at(keys, kv, idx) : -1;
-    }
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        const int32_t k = key[r];
-        if (k >= 0 && k < key_limit) atomicAdd(&h[(k >> shift) & (kRadix - 1)], 1);
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < kRadix; d += kThreads) ghist[int64_t(d) * nblocks + blockIdx.x] = h[d];
-}
+// R = 32-element rounds per warp: a tile of 8 warps holds 256 * R elements (R = 8 or 16, the
+// SORT_ROUNDS tuning knob; larger tiles give longer runs per digit in the scatter)
 
 // lanes of the warp whose 8-bit digit equals this lane's, among the valid lanes (an invalid lane
 // matches itself only): __match_any_sync, or eight ballots on the digit's bits
@@ -81,145 +169,184 @@ __device__ __forceinline__ unsigned digit_peers(int d, bool valid, int lane) {
     return valid ? peers : (1u << lane);
 }
 
-// The tile's elements are first placed in shared memory in digit order (stable: by digit, then by
-// position in the tile), then written out by consecutive threads: equal digits form one run of the
-// output, so a warp's store touches a few runs instead of one segment per lane.
+// all blocks of the cooperative grid; false (in every block that gets there) if the wait ran out
+__device__ bool grid_barrier(uint32_t *bar, uint32_t target, int32_t *status) {
+    constexpr int kPolls = 1 << 24;  // about ten seconds
+    __syncthreads();
+    bool ok = true;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        int i = 0;
+        while (*reinterpret_cast<volatile uint32_t *>(bar) < target && i < kPolls) {
+            __nanosleep(64);
+            ++i;
+        }
+        ok = i < kPolls;
+        if (!ok) set_status(status, ETL_ETIMEOUT);
+        __threadfence();
+    }
+    return __syncthreads_and(ok);
+}
+
+// Pairs (parent, child) of the heavy families in ascending child order, sorted by parent. Every block
+// owns a contiguous part of a pass's input; ghist[digit * blocks + block] are the blocks' histograms.
 template <int R, bool BALLOT>
 __global__ void __launch_bounds__(kThreads)
-    k_scatter(const int32_t *__restrict__ keys, const int32_t *__restrict__ vals, const int2 *__restrict__ kv,
-              const int32_t *d_count, int64_t n_cap, int shift, int32_t key_limit, const int32_t *__restrict__ goff,
-              int nblocks, int2 *__restrict__ kv_out) {
-    pdl_prologue();
-    constexpr int kRounds = R, kWarpTile = kWarp * R, kTile = kWarps * kWarpTile;
+    k_sort_heavy(const int32_t *__restrict__ par, int32_t n, const uint32_t *__restrict__ heavy,
+                 const int32_t *__restrict__ heavy_count, int passes, int2 *buf0, int2 *buf1, int32_t *ghist,
+                 uint32_t *bar, int32_t *__restrict__ head, int32_t *__restrict__ next, int32_t *__restrict__ status) {
+    if (*heavy_count == 0) return;
+    constexpr int kWarpTile = kWarp * R, kTile = kWarps * kWarpTile;
     __shared__ int32_t wcnt[kWarps][kRadix];
-    __shared__ int32_t gbase[kRadix];
+    __shared__ int32_t gbase[kRadix];   // next output place of each digit
     __shared__ int32_t dstart[kRadix];  // first tile position of each digit (digit order)
     __shared__ int32_t wtot[kWarps];
     __shared__ int2 stage[kTile];
-    const int64_t count = count_of(d_count, n_cap);
-    if (int64_t(blockIdx.x) * kTile >= count) return;  // nothing of this tile to place
-    for (int i = threadIdx.x; i < kWarps * kRadix; i += kThreads) (&wcnt[0][0])[i] = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t base = int64_t(blockIdx.x) * kTile + warp * kWarpTile;
-    int32_t key[kRounds], val[kRounds], dig[kRounds], lrank[kRounds];
-    // all loads of the tile first, so that they are in flight together (the ranking rounds below
-    // are ordered by __syncwarp and would otherwise wait for one load each)
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        const int64_t idx = base + r * kWarp + lane;
-        key[r] = -1;
-        val[r] = 0;
-        if (idx < count) {
-            if (kv) {
-                const int2 x = __ldcs(kv + idx);
-                key[r] = x.x;
-                val[r] = x.y;
-            } else {
-                key[r] = __ldcs(keys + idx);
-                val[r] = vals ? __ldcs(vals + idx) : int32_t(idx);
-            }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, d = threadIdx.x;
+    const int blocks = gridDim.x, blk = blockIdx.x;
+    uint32_t arrivals = 0;
+    int64_t count = n;  // of the pass's input: all nodes first, then the pairs kept
+    for (int p = 0; p < passes; ++p) {
+        const int shift = 8 * p;
+        const int2 *in = p & 1 ? buf0 : buf1;
+        int2 *out = p & 1 ? buf1 : buf0;
+        const int64_t lo = count * blk / blocks, hi = count * (blk + 1) / blocks;
+        auto load = [&](int64_t i) -> int2 {  // parent -1: not one of a heavy family
+            if (i >= hi) return make_int2(-1, 0);
+            if (p > 0) return __ldcg(in + i);
+            const int32_t q = __ldg(par + i);
+            const bool h = q >= 0 && q < n && ((__ldg(heavy + (q >> 5)) >> (q & 31)) & 1u);
+            return make_int2(h ? q : -1, int32_t(i));
+        };
+        gbase[d] = 0;
+        __syncthreads();
+        for (int64_t i = lo + threadIdx.x; i < hi; i += kThreads) {
+            const int32_t k = load(i).x;
+            if (k >= 0) atomicAdd(&gbase[(k >> shift) & (kRadix - 1)], 1);
         }
+        __syncthreads();
+        ghist[int64_t(d) * blocks + blk] = gbase[d];
+        arrivals += blocks;
+        if (!grid_barrier(bar, arrivals, status)) return;
+        // this digit's elements in all blocks, and in the blocks before this one
+        int32_t all = 0, before = 0;
+        for (int b = 0; b < blocks; ++b) {
+            const int32_t c = __ldcg(ghist + int64_t(d) * blocks + b);
+            all += c;
+            if (b < blk) before += c;
+        }
+        int32_t inc = all;
+#pragma unroll
+        for (int o = 1; o < kWarp; o <<= 1) {
+            const int32_t y = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == kWarp - 1) wtot[warp] = inc;
+        __syncthreads();
+        int32_t wofs = 0, total = 0;
+        for (int w = 0; w < kWarps; ++w) {
+            if (w < warp) wofs += wtot[w];
+            total += wtot[w];
+        }
+        gbase[d] = wofs + inc - all + before;
+        __syncthreads();
+        for (int64_t base = lo; base < hi; base += kTile) {
+            for (int w = 0; w < kWarps; ++w) wcnt[w][d] = 0;
+            __syncthreads();
+            int2 x[R];
+            int32_t dig[R], lrank[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) x[r] = load(base + warp * kWarpTile + r * kWarp + lane);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const bool valid = x[r].x >= 0;
+                const int dd = valid ? ((x[r].x >> shift) & (kRadix - 1)) : 0;
+                const unsigned peers = digit_peers<BALLOT>(dd, valid, lane);
+                int pre = 0;
+                if (valid) pre = wcnt[warp][dd];
+                __syncwarp();
+                if (valid && lane == __ffs(peers) - 1) wcnt[warp][dd] = pre + __popc(peers);
+                __syncwarp();
+                dig[r] = valid ? dd : -1;
+                lrank[r] = pre + __popc(peers & lanemask_lt());
+            }
+            __syncthreads();
+            // counts of the warps -> offsets across warps; the digits' totals -> offsets across digits
+            int32_t run = 0;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const int32_t c = wcnt[w][d];
+                wcnt[w][d] = run;
+                run += c;
+            }
+            int32_t scan = run;
+#pragma unroll
+            for (int o = 1; o < kWarp; o <<= 1) {
+                const int32_t y = __shfl_up_sync(kFull, scan, o);
+                if (lane >= o) scan += y;
+            }
+            if (lane == kWarp - 1) wtot[warp] = scan;
+            __syncthreads();
+            int32_t ofs = 0, placed = 0;
+            for (int w = 0; w < kWarps; ++w) {
+                if (w < warp) ofs += wtot[w];
+                placed += wtot[w];
+            }
+            dstart[d] = ofs + scan - run;
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (dig[r] >= 0) stage[dstart[dig[r]] + wcnt[warp][dig[r]] + lrank[r]] = x[r];
+            __syncthreads();
+            for (int i = threadIdx.x; i < placed; i += kThreads) {
+                const int2 y = stage[i];
+                const int dd = (y.x >> shift) & (kRadix - 1);
+                out[gbase[dd] + (i - dstart[dd])] = y;
+            }
+            __syncthreads();
+            gbase[d] += run;
+        }
+        count = total;
+        arrivals += blocks;
+        if (!grid_barrier(bar, arrivals, status)) return;
     }
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        const int32_t k = key[r];
-        const bool valid = k >= 0 && k < key_limit;  // also false past the end (k = -1)
-        const int d = valid ? ((k >> shift) & (kRadix - 1)) : 0;
-        const unsigned peers = digit_peers<BALLOT>(d, valid, lane);
-        int pre = 0;
-        if (valid) pre = wcnt[warp][d];
-        __syncwarp();
-        if (valid && lane == __ffs(peers) - 1) wcnt[warp][d] = pre + __popc(peers);
-        __syncwarp();
-        dig[r] = valid ? d : -1;
-        lrank[r] = pre + __popc(peers & lanemask_lt());
-    }
-    __syncthreads();
-    // per digit (one per thread): counts of the warps -> exclusive offsets across warps, and the
-    // digit's total; then the digits' totals -> exclusive offsets across digits (block scan)
-    const int d = threadIdx.x;  // kThreads == kRadix
-    int32_t run = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        const int32_t t = wcnt[w][d];
-        wcnt[w][d] = run;
-        run += t;
-    }
-    gbase[d] = goff[int64_t(d) * nblocks + blockIdx.x];
-    int32_t inc = run;  // inclusive scan of the digits' totals: warp scan, then the warps' sums
-#pragma unroll
-    for (int o = 1; o < kWarp; o <<= 1) {
-        const int32_t y = __shfl_up_sync(kFull, inc, o);
-        if (lane >= o) inc += y;
-    }
-    if (lane == kWarp - 1) wtot[warp] = inc;
-    __syncthreads();
-    int32_t wofs = 0;
-    for (int w = 0; w < warp; ++w) wofs += wtot[w];
-    dstart[d] = wofs + inc - run;
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r)
-        if (dig[r] >= 0) stage[dstart[dig[r]] + wcnt[warp][dig[r]] + lrank[r]] = make_int2(key[r], val[r]);
-    __syncthreads();
-    int32_t placed = 0;  // elements of the tile with a valid key
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) placed += wtot[w];
-    for (int i = threadIdx.x; i < placed; i += kThreads) {
-        const int2 x = stage[i];
-        const int dd = (x.x >> shift) & (kRadix - 1);
-        kv_out[gbase[dd] + (i - dstart[dd])] = x;
+    const int2 *kv = passes & 1 ? buf0 : buf1;
+    for (int64_t i = gtid(); i < count; i += gstride()) {
+        const int2 x = __ldcg(kv + i);
+        const int32_t before = i > 0 ? __ldcg(&kv[i - 1].x) : -1;
+        const int2 y = i + 1 < count ? __ldcg(kv + i + 1) : make_int2(-1, -1);
+        next[x.y] = y.x == x.x ? y.y : -1;
+        if (before != x.x) head[x.x] = x.y;
     }
 }
 
-template <int R>
-etl_status radix_sort_impl(const int32_t *keys_in, const int32_t *vals_in, const int32_t *d_count, int64_t n_cap,
-                           int key_bits, int32_t key_limit, Workspace &ws, SortResult *out) {
-    constexpr int kTile = kWarps * kWarp * R;
-    cudaStream_t s = ws.stream();
-    const int64_t cap = n_cap > 0 ? n_cap : 1;
-    const int nblocks = int(ceil_div(cap, kTile));
-    const int passes = key_bits <= 8 ? 1 : (key_bits + 7) / 8;
-    if (key_bits < 31 && key_limit > (int32_t(1) << key_bits)) key_limit = int32_t(1) << key_bits;
-    int2 *buf[2] = {ws.get<int2>(cap), ws.get<int2>(cap)};
-    int32_t *ghist = ws.get<int32_t>(int64_t(kRadix) * nblocks);
+template <int R, bool BALLOT>
+etl_status sort_heavy(const int32_t *par, int32_t n, const uint32_t *heavy, const int32_t *heavy_count, uint32_t *bar,
+                      int32_t *head, int32_t *next, int32_t *status, Workspace &ws) {
+    auto kernel = k_sort_heavy<R, BALLOT>;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0) != cudaSuccess || per_sm < 1)
+        return ETL_ECUDA;
+    const int blocks = num_sms() * (per_sm < 2 ? per_sm : 2);
+    int2 *buf0 = ws.get<int2>(n), *buf1 = ws.get<int2>(n);
+    int32_t *ghist = ws.get<int32_t>(int64_t(kRadix) * blocks);
     if (!ws.ok()) return ETL_ENOMEM;
-    const int2 *kvin = nullptr;
-    const int32_t *cnt = d_count;
-    for (int p = 0; p < passes; ++p) {
-        int32_t *goff = ws.get<int32_t>(int64_t(kRadix) * nblocks + 1);
-        if (!ws.ok()) return ETL_ENOMEM;
-        const int shift = 8 * p;
-        etl_status st;
-        {
-            PhaseTimer pt("sort.hist", s);
-            launch(k_hist<R>, nblocks, kThreads, 0, s, keys_in, kvin, cnt, cap, shift, key_limit, ghist, nblocks);
-            note_launch();
-            st = last_launch();
-        }
-        if (st) return st;
-        st = scan_exclusive_i32(ghist, goff, int64_t(kRadix) * nblocks, ws);
-        if (st) return st;
-        int2 *out_kv = buf[p & 1];
-        {
-            PhaseTimer pt("sort.scatter", s);
-            if (sort_params().ballot)
-                launch(k_scatter<R, true>, nblocks, kThreads, 0, s, keys_in, vals_in, kvin, cnt, cap, shift, key_limit,
-                       goff, nblocks, out_kv);
-            else
-                launch(k_scatter<R, false>, nblocks, kThreads, 0, s, keys_in, vals_in, kvin, cnt, cap, shift, key_limit,
-                       goff, nblocks, out_kv);
-            note_launch();
-            st = last_launch();
-        }
-        if (st) return st;
-        kvin = out_kv;
-        cnt = goff + int64_t(kRadix) * nblocks;  // number of kept elements
-    }
-    out->kv = kvin;
-    out->d_total = cnt;
-    return ETL_OK;
+    const int bits = ceil_log2(uint64_t(n));
+    int passes = bits <= 8 ? 1 : (bits + 7) / 8;
+    PhaseTimer pt("lca.heavy", ws.stream());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = blocks;
+    cfg.blockDim = kThreads;
+    cfg.stream = ws.stream();
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, par, n, heavy, heavy_count, passes, buf0, buf1, ghist, bar, head, next, status);
+    note_launch();
+    return last_launch();
 }
 
 }  // namespace
@@ -229,11 +356,41 @@ SortParams &sort_params() {
     return p;
 }
 
-etl_status radix_sort_pairs(const int32_t *keys_in, const int32_t *vals_in, const int32_t *d_count, int64_t n_cap,
-                            int key_bits, int32_t key_limit, Workspace &ws, SortResult *out) {
-    if (sort_params().rounds == 16)
-        return radix_sort_impl<16>(keys_in, vals_in, d_count, n_cap, key_bits, key_limit, ws, out);
-    return radix_sort_impl<8>(keys_in, vals_in, d_count, n_cap, key_bits, key_limit, ws, out);
+etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, const int32_t *inst_of,
+                         const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
+                         int32_t *root_of, int32_t *status, Workspace &ws) {
+    cudaStream_t s = ws.stream();
+    const int64_t mask_words = ceil_div(n, 32);
+    uint32_t *words = ws.get<uint32_t>(2 * mask_words + 2);  // seen, heavy, heavy families, barrier
+    if (!ws.ok()) return ETL_ENOMEM;
+    uint32_t *heavy = words + mask_words, *bar = words + 2 * mask_words + 1;
+    int32_t *heavy_count = reinterpret_cast<int32_t *>(words + 2 * mask_words);
+    memset_async(words, 0, size_t(2 * mask_words + 2) * 4, s);
+    memset_async(head, 0xff, size_t(n) * 4, s);
+    const int32_t *par = off ? gparent : parent;
+    {
+        PhaseTimer pt("lca.link", s);
+        const int blocks = int(ceil_div(n, kLinkThreads * kLinkIlp));
+        launch(off ? k_link_children<true> : k_link_children<false>, blocks, kLinkThreads, 0, s, parent, n, off, inst_of,
+               bad, gparent, head, next, root_cnt, root_of, status);
+        note_launch();
+    }
+    {
+        PhaseTimer pt("lca.check", s);
+        const bool small = n <= kCheckSmall;
+        const int64_t blocks = ceil_div(n, kCheckThreads * (small ? 1 : 4)), most = int64_t(num_sms()) * 8;
+        launch(small ? k_check_children<1> : k_check_children<4>, int(blocks < most ? blocks : most), kCheckThreads, 0, s, par, n, head, next, words, heavy,
+               heavy_count);
+        note_launch();
+    }
+    etl_status st = last_launch();
+    if (st || n <= kLight) return st;
+    const SortParams &P = sort_params();
+    if (P.rounds == 16)
+        return P.ballot ? sort_heavy<16, true>(par, n, heavy, heavy_count, bar, head, next, status, ws)
+                        : sort_heavy<16, false>(par, n, heavy, heavy_count, bar, head, next, status, ws);
+    return P.ballot ? sort_heavy<8, true>(par, n, heavy, heavy_count, bar, head, next, status, ws)
+                    : sort_heavy<8, false>(par, n, heavy, heavy_count, bar, head, next, status, ws);
 }
 
 }  // namespace etl
