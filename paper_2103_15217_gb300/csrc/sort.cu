@@ -179,7 +179,7 @@ __device__ bool grid_barrier(uint32_t *bar, uint32_t target, int32_t *status) {
         atomicAdd(bar, 1u);
         int i = 0;
         while (*reinterpret_cast<volatile uint32_t *>(bar) < target && i < kPolls) {
-            __nanosleep(64);
+            __nanosleep(100);
             ++i;
         }
         ok = i < kPolls;
@@ -195,7 +195,7 @@ template <int R, bool BALLOT>
 __global__ void __launch_bounds__(kThreads)
     k_sort_heavy(const int32_t *__restrict__ par, int32_t n, const uint32_t *__restrict__ heavy,
                  const int32_t *__restrict__ heavy_count, int passes, int2 *buf0, int2 *buf1, int32_t *ghist,
-                 uint32_t *bar, int32_t *__restrict__ head, int32_t *__restrict__ next, int32_t *__restrict__ status) {
+                 int32_t *totals, uint32_t *bar, int32_t *__restrict__ head, int32_t *__restrict__ next, int32_t *__restrict__ status) {
     if (*heavy_count == 0) return;
     constexpr int kWarpTile = kWarp * R, kTile = kWarps * kWarpTile;
     __shared__ int32_t wcnt[kWarps][kRadix];
@@ -229,13 +229,34 @@ __global__ void __launch_bounds__(kThreads)
         ghist[int64_t(d) * blocks + blk] = gbase[d];
         arrivals += blocks;
         if (!grid_barrier(bar, arrivals, status)) return;
-        // this digit's elements in all blocks, and in the blocks before this one
-        int32_t all = 0, before = 0;
-        for (int b = 0; b < blocks; ++b) {
-            const int32_t c = __ldcg(ghist + int64_t(d) * blocks + b);
-            all += c;
-            if (b < blk) before += c;
+        // exclusive prefixes over the blocks, one digit's row at a time; its total goes to totals
+        for (int row = blk; row < kRadix; row += blocks) {
+            int32_t carry = 0;
+            for (int b0 = 0; b0 < blocks; b0 += kThreads) {
+                const int b = b0 + threadIdx.x;
+                int32_t *at = ghist + int64_t(row) * blocks + b;
+                const int32_t c = b < blocks ? __ldcg(at) : 0;
+                int32_t inc = c;
+#pragma unroll
+                for (int o = 1; o < kWarp; o <<= 1) {
+                    const int32_t y = __shfl_up_sync(kFull, inc, o);
+                    if (lane >= o) inc += y;
+                }
+                if (lane == kWarp - 1) wtot[warp] = inc;
+                __syncthreads();
+                int32_t wofs = carry;
+                for (int w = 0; w < kWarps; ++w) {
+                    if (w < warp) wofs += wtot[w];
+                    carry += wtot[w];
+                }
+                if (b < blocks) *at = wofs + inc - c;
+                __syncthreads();
+            }
+            if (threadIdx.x == 0) totals[row] = carry;
         }
+        arrivals += blocks;
+        if (!grid_barrier(bar, arrivals, status)) return;
+        const int32_t all = __ldcg(totals + d), before = __ldcg(ghist + int64_t(d) * blocks + blk);
         int32_t inc = all;
 #pragma unroll
         for (int o = 1; o < kWarp; o <<= 1) {
@@ -328,9 +349,11 @@ etl_status sort_heavy(const int32_t *par, int32_t n, const uint32_t *heavy, cons
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0) != cudaSuccess || per_sm < 1)
         return ETL_ECUDA;
-    const int blocks = num_sms() * (per_sm < 2 ? per_sm : 2);
+    // all that are resident at once, but no more than there are tiles
+    const int64_t tiles = ceil_div(n, kWarps * kWarp * R);
+    const int blocks = int(tiles < int64_t(num_sms()) * per_sm ? tiles : int64_t(num_sms()) * per_sm);
     int2 *buf0 = ws.get<int2>(n), *buf1 = ws.get<int2>(n);
-    int32_t *ghist = ws.get<int32_t>(int64_t(kRadix) * blocks);
+    int32_t *ghist = ws.get<int32_t>(int64_t(kRadix) * (blocks + 1)), *totals = ghist + int64_t(kRadix) * blocks;
     if (!ws.ok()) return ETL_ENOMEM;
     const int bits = ceil_log2(uint64_t(n));
     int passes = bits <= 8 ? 1 : (bits + 7) / 8;
@@ -344,7 +367,7 @@ etl_status sort_heavy(const int32_t *par, int32_t n, const uint32_t *heavy, cons
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, par, n, heavy, heavy_count, passes, buf0, buf1, ghist, bar, head, next, status);
+    cudaLaunchKernelEx(&cfg, kernel, par, n, heavy, heavy_count, passes, buf0, buf1, ghist, totals, bar, head, next, status);
     note_launch();
     return last_launch();
 }
