@@ -225,13 +225,40 @@ struct Slot8 {  // low word: successor / sublist id; high word: kRaw / kOff / lr
     __device__ static __forceinline__ uint32_t lo(T v) { return uint32_t(v >> 48) & 0x7fffu; }
     __device__ static __forceinline__ bool leaf(T v) { return (v >> 63) && !raw(v) && !off(v); }
 };
+// 4-byte slots of a tour (dual) with fewer than 2^29 elements: successor, bit 30: contracted leaf; -1;
+// kOff; record: top bit, sublist id (22 bits), lr (lr + 1) / 2 + lo (9 bits: lr < kLcap, lo <= lr). Short
+// sublists, but half the memory of 8-byte slots.
+struct Slot4d {
+    using T = uint32_t;
+    static constexpr uint32_t kOff = 0x7ffffffeu;
+    static constexpr int kLcap = 31, kSidBits = 22;
+    __device__ static __forceinline__ T exch(T *p, T v) { return atomicExch(p, v); }
+    __device__ static __forceinline__ bool off(T v) { return v == kOff; }
+    __device__ static __forceinline__ bool raw(T v) { return (!(v >> 31) && v != kOff) || v == 0xffffffffu; }
+    __device__ static __forceinline__ T make(int32_t succ) {  // leaf: top bit set
+        return succ < ETL_END ? (uint32_t(succ) & 0x3fffffffu) | 0x40000000u : uint32_t(succ);
+    }
+    __device__ static __forceinline__ T off_list() { return kOff; }
+    __device__ static __forceinline__ int32_t next(T v) {
+        return v == 0xffffffffu ? ETL_END : int32_t((v & 0x40000000u) ? (v & 0x3fffffffu) | 0x80000000u : v);
+    }
+    __device__ static __forceinline__ T rec(int32_t sid, uint32_t lr, uint32_t lo, int) {
+        return 0x80000000u | (uint32_t(sid) << 9) | (((lr * (lr + 1)) >> 1) + lo);
+    }
+    __device__ static __forceinline__ int32_t sid(T v, int) { return int32_t((v & 0x7fffffffu) >> 9); }
+    __device__ static __forceinline__ uint32_t lr(T v, int) {
+        const uint32_t k = v & 511u;
+        return uint32_t((sqrtf(float(8u * k + 1u)) - 1.0f) * 0.5f);  // exact: the root of a perfect square is
+    }
+    __device__ static __forceinline__ uint32_t lo(T v, uint32_t lr) { return (v & 511u) - ((lr * (lr + 1)) >> 1); }
+};
 inline bool wide_slots(int64_t len) { return len > (int64_t(1) << 30); }
 
 // Result of ranking one list: element e's record names its sublist; T[sid].x / T[sid].y are the number
 // of elements / of even-indexed elements before that sublist's first element. So rank(e) =
 // T[sid].x + lr and evens_before(e) = T[sid].y + lo.
 struct RankResult {
-    const void *recs;  // Slot8 records if wide, else Slot4
+    const void *recs;  // Slot8 records if wide; else Slot4 or, in dual mode, Slot4d ones
     bool wide;
     int lb;
     const int4 *T;
@@ -259,7 +286,7 @@ struct RankParams {
     int k0_log2 = 5;     // level-0 splitter density: one in 2^k0_log2 elements
     int k_log2 = 3;      // density at the upper levels (1 in 8: 1-4% faster than 1 in 16 on trees of 2^15 .. 2^22)
     int block = 128;     // threads per block of the walk kernels
-    int blocks_per_sm = 8;  // 1024 walkers per SM on lists larger than L2
+    int blocks_per_sm = 10;  // 1280 walkers per SM on lists ranked in place
 };
 RankParams &rank_params();
 
@@ -283,13 +310,14 @@ struct RmqParams {
 };
 RmqParams &rmq_params();
 
-// Ranks a list of len elements, from *d_head, or from `head` if d_head is null. list: if
-// rank_in_place(len, dual), len slots (Slot8 if dual or wide_slots(len), else Slot4), which the records
-// replace; otherwise len int32 successors, and the records get an array of their own. An element that
-// is on no list holds off_list() in a slot, Slot4::kOff as a successor; a contracted leaf's second
+// What list_rank takes: int32 successors (the records get an array of their own), or slots that the
+// records replace (8-byte slots: Slot8; 4-byte ones: Slot4, in dual mode Slot4d).
+enum class RankForm { kSeparate, kSlots8, kSlots4 };
+RankForm rank_form(int64_t len, bool dual);
+// Ranks a list of len elements in that form, from *d_head, or from `head` if d_head is null. An element
+// that is on no list holds off_list() in a slot, Slot4::kOff as a successor; a contracted leaf's second
 // element off_list() in a slot, -1 as a successor. dual: also counts even-indexed elements (the opening
 // brackets of a tour). expect_len: the total weight the list must have (-1: not checked).
-bool rank_in_place(int64_t len, bool dual);
 etl_status list_rank(void *list, int64_t len, const int32_t *d_head, int32_t head, bool dual, int64_t expect_len,
                      int32_t *status, Workspace &ws, RankResult *out);
 

@@ -33,6 +33,7 @@
 // (the node of least depth in the range is a child of the LCA) with the
 // answer read directly: one min, no argmin and no tie-breaking.
 #include <climits>
+#include <type_traits>
 
 #include "etl_internal.cuh"
 
@@ -70,7 +71,7 @@ __global__ void k_fill_inst(const int32_t *__restrict__ off, int32_t k, const in
 // 2v+1 with weight 2 (top bit set), and 2v+1 is off the list. Roots are never contracted. All accesses
 // are coalesced (the closing brackets' successors were scattered to random places before, which made
 // this step 0.26 ms for 2^24 nodes; now 0.08).
-template <bool SLOTS>
+template <class S>  // void: successors
 __global__ void k_tour_assemble(const int32_t *__restrict__ par, const int32_t *__restrict__ head,
                                 const int32_t *__restrict__ next, int32_t n, void *__restrict__ list) {
     pdl_prologue();
@@ -79,9 +80,10 @@ __global__ void k_tour_assemble(const int32_t *__restrict__ par, const int32_t *
         const int32_t c = x >= 0 ? 2 * x : p >= 0 ? 2 * p + 1 : ETL_END;  // leave t -> enter next sibling, or leave p
         const bool one = h < 0 && p >= 0;                                 // a leaf, and no root
         const int32_t a = one ? int32_t(uint32_t(c) | 0x80000000u) : h >= 0 ? 2 * h : 2 * int32_t(t) + 1;
-        if (SLOTS)
-            static_cast<ulonglong2 *>(list)[t] =
-                make_ulonglong2(Slot8::make(a), one ? Slot8::off_list() : Slot8::make(c));
+        if constexpr (std::is_same<S, Slot8>::value)
+            static_cast<ulonglong2 *>(list)[t] = make_ulonglong2(S::make(a), one ? S::off_list() : S::make(c));
+        else if constexpr (std::is_same<S, Slot4d>::value)
+            static_cast<uint2 *>(list)[t] = make_uint2(S::make(a), one ? S::off_list() : S::make(c));
         else
             static_cast<int2 *>(list)[t] = make_int2(a, one ? ETL_END : c);
     }
@@ -103,25 +105,51 @@ __global__ void k_link_roots(const int32_t *__restrict__ root_cnt, const int32_t
     }
 }
 
+// The two records of a node, side by side
+struct NodeRecs {
+    int32_t sa, sb;       // sublists of the opening and closing bracket
+    int32_t ra, rb, oa;   // their offsets, and the opening brackets before the first one, in the sublists
+    bool ok, leaf;        // both on the list; contracted: the closing bracket is ranked right after
+};
+__device__ __forceinline__ NodeRecs node_recs(ulonglong2 q) {
+    NodeRecs r;
+    r.leaf = Slot8::leaf(q.x) || Slot8::off(q.y);
+    r.ok = !Slot8::raw(q.x) && !Slot8::off(q.x) && (r.leaf || !Slot8::raw(q.y));
+    r.sa = Slot8::sid(q.x, 0);
+    r.sb = r.leaf ? r.sa : Slot8::sid(q.y, 0);
+    r.ra = int32_t(Slot8::lr(q.x, 0));
+    r.rb = int32_t(Slot8::lr(q.y, 0));
+    r.oa = int32_t(Slot8::lo(q.x));
+    return r;
+}
+__device__ __forceinline__ NodeRecs node_recs(uint2 q) {
+    NodeRecs r;
+    r.leaf = Slot4d::off(q.y);
+    r.ok = !Slot4d::raw(q.x) && !Slot4d::off(q.x) && (r.leaf || !Slot4d::raw(q.y));
+    r.sa = Slot4d::sid(q.x, 0);
+    r.sb = r.leaf ? r.sa : Slot4d::sid(q.y, 0);
+    r.ra = int32_t(Slot4d::lr(q.x, 0));
+    r.rb = int32_t(Slot4d::lr(q.y, 0));
+    r.oa = int32_t(Slot4d::lo(q.x, uint32_t(r.ra)));
+    return r;
+}
+
+template <class Q>
 __global__ void k_node_stats(RankResult rr, int32_t n, int32_t *__restrict__ pre, int32_t *__restrict__ depth,
                              int32_t *__restrict__ size, int32_t *__restrict__ order, int32_t *__restrict__ status) {
     pdl_prologue();
-    const ulonglong2 *recs = static_cast<const ulonglong2 *>(rr.recs);  // brackets 2v and 2v+1 side by side
+    const Q *recs = static_cast<const Q *>(rr.recs);
     for (int64_t t = gtid(); t < n; t += gstride()) {
-        const ulonglong2 q = __ldcs(recs + t);
-        // contracted: the closing bracket is ranked right after
-        const bool leaf = Slot8::leaf(q.x) || Slot8::off(q.y);
-        const int32_t sa = Slot8::sid(q.x, 0), sb = leaf ? sa : Slot8::sid(q.y, 0);
-        if (Slot8::raw(q.x) || Slot8::off(q.x) || (!leaf && Slot8::raw(q.y)) || sa < 0 || sa >= rr.rcap || sb < 0 ||
-            sb >= rr.rcap) {  // not on the list from the root: malformed input
-            set_status(status, ETL_EBADTREE);
+        const NodeRecs r = node_recs(__ldcs(recs + t));
+        if (!r.ok || r.sa < 0 || r.sa >= rr.rcap || r.sb < 0 || r.sb >= rr.rcap) {
+            set_status(status, ETL_EBADTREE);  // not on the list from the root: malformed input
             pre[t] = depth[t] = size[t] = -1;
             continue;
         }
-        const int2 A = __ldg(reinterpret_cast<const int2 *>(rr.T + sa));
-        const int32_t r0 = A.x + int32_t(Slot8::lr(q.x, 0));
-        const int32_t r1 = leaf ? r0 + 1 : __ldg(&rr.T[sb].x) + int32_t(Slot8::lr(q.y, 0));
-        const int32_t p = A.y + int32_t(Slot8::lo(q.x));
+        const int2 A = __ldg(reinterpret_cast<const int2 *>(rr.T + r.sa));
+        const int32_t r0 = A.x + r.ra;
+        const int32_t r1 = r.leaf ? r0 + 1 : __ldg(&rr.T[r.sb].x) + r.rb;
+        const int32_t p = A.y + r.oa;
         __stcs(pre + t, p);
         __stcs(depth + t, 2 * p - r0);
         __stcs(size + t, (r1 - r0 + 1) >> 1);
@@ -359,8 +387,8 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
     etl_status st = ETL_OK;
     {
         Workspace ws(s);
-        const bool slots = rank_in_place(2 * int64_t(n), true);
-        void *list = slots ? static_cast<void *>(ws.get<ulonglong2>(n)) : ws.get<int2>(n);  // 2n list elements
+        const RankForm form = rank_form(2 * int64_t(n), true);
+        void *list = form == RankForm::kSlots8 ? static_cast<void *>(ws.get<ulonglong2>(n)) : ws.get<int2>(n);  // 2n elements
         int32_t *head = ws.get<int32_t>(n), *next = ws.get<int32_t>(n);
         int32_t *misc = ws.get<int32_t>(2 + 2 * int64_t(k));  // list head, offsets invalid, roots per tree, a root
         int32_t *root_cnt = misc + 2, *root_of = root_cnt + k;
@@ -384,8 +412,10 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
             PhaseTimer pt("lca.succ", s);
             launch(k_link_roots, grid_for(k, 256), 256, 0, s, root_cnt, root_of, k, n, next, misc, h->status);
             note_launch();
-            launch(slots ? k_tour_assemble<true> : k_tour_assemble<false>, grid_for(n, 256), 256, 0, s, par, head, next,
-                   n, list);
+            launch(form == RankForm::kSlots8   ? k_tour_assemble<Slot8>
+                   : form == RankForm::kSlots4 ? k_tour_assemble<Slot4d>
+                                               : k_tour_assemble<void>,
+                   grid_for(n, 256), 256, 0, s, par, head, next, n, list);
             note_launch();
             st = last_launch();
         }
@@ -393,7 +423,8 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         if (!st) st = list_rank(list, 2 * int64_t(n), misc, 0, true, 2 * int64_t(n), h->status, ws, &rr);
         if (!st) {
             PhaseTimer pt("lca.node_stats", s);
-            launch(k_node_stats, grid_for(n, 256), 256, 0, s, rr, n, h->pre, h->depth, h->size, h->order, h->status);
+            launch(rr.wide ? k_node_stats<ulonglong2> : k_node_stats<uint2>, grid_for(n, 256), 256, 0, s, rr, n, h->pre, h->depth,
+                   h->size, h->order, h->status);
             note_launch();
             launch(k_check_instances, grid_for(k, 256), 256, 0, s, root_of, batch ? h->node_off : nullptr, k, n, h->pre,
                    h->size, h->status);

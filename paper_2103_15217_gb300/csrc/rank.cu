@@ -47,6 +47,7 @@
 // and 2v+1 itself is off the list.
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "etl_internal.cuh"
 
@@ -228,8 +229,21 @@ __global__ void k_walk0_in_place(typename S::T *__restrict__ slots, Walk0 W, int
     uint32_t lr = 0, lo = 0;
     bool active = false, claim = false, is_head = false;
     while (true) {
-        const bool want = !active && w < W.nclaims;
-        pool.refill(ctr, W.start, W.limit, want && sid < 0, sid);
+        const bool want = !active && w < W.nclaims, full = active && lr >= uint32_t(W.lcap);
+        int32_t ns = sid;
+        pool.refill(ctr, W.start, W.limit, (want && sid < 0) || full, ns);
+        if (full) {  // the walk goes on in a new sublist
+            if (ns < W.cap) {
+                T[sid] = make_int4(int32_t(lr), int32_t(lo), ns, 0);
+                lr = lo = 0;
+            } else {
+                set_status(status, ETL_ETIMEOUT);
+                T[sid] = make_int4(int32_t(lr), int32_t(lo), kEndT, 0);
+                active = false;
+                ns = -1;
+            }
+        }
+        sid = ns;
         if (want) {
             is_head = w == 0;
             const int64_t e = is_head ? int64_t(head) : candidate(w, W.len);
@@ -281,17 +295,6 @@ __global__ void k_walk0_in_place(typename S::T *__restrict__ slots, Walk0 W, int
                 done = true;
             } else {
                 cur = nxt;
-                if (lr >= uint32_t(W.lcap)) {
-                    const int32_t ns = W.start + atomicAdd(ctr, 1);
-                    if (ns >= W.cap) {
-                        set_status(status, ETL_ETIMEOUT);
-                        done = true;
-                    } else {
-                        T[sid] = make_int4(int32_t(lr), int32_t(lo), ns, 0);
-                        sid = ns;
-                        lr = lo = 0;
-                    }
-                }
             }
         }
         if (done) {
@@ -569,8 +572,12 @@ RankParams &rank_params() {
 }
 
 // Successors and records (8 bytes per element, 12 in dual mode) of up to 96 of the 129 MB L2 are kept in
-// separate arrays; longer lists are ranked in place.
-bool rank_in_place(int64_t len, bool dual) { return len * (dual ? 12 : 8) > (int64_t(96) << 20); }
+// separate arrays; longer lists are ranked in place, in 4-byte slots where the records fit them.
+RankForm rank_form(int64_t len, bool dual) {
+    if (len * (dual ? 12 : 8) <= (int64_t(96) << 20)) return RankForm::kSeparate;
+    if (dual) return len <= (int64_t(1) << 26) ? RankForm::kSlots4 : RankForm::kSlots8;
+    return wide_slots(len) ? RankForm::kSlots8 : RankForm::kSlots4;
+}
 
 namespace {
 
@@ -593,7 +600,8 @@ template <class S, bool DUAL, class A>
 etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head, int32_t head, int64_t expect_len,
                      int32_t *status, const RankParams &P, A &alloc, cudaStream_t s, RankResult *out) {
     using R = typename S::T;
-    const bool in_place = rank_in_place(len, DUAL);
+    const bool in_place = rank_form(len, DUAL) != RankForm::kSeparate;
+    constexpr bool kNarrow = std::is_same<S, Slot4d>::value;
     out->wide = sizeof(R) == 8;
     out->lb = out->wide ? 16 : 12;
     if (in_place) recs = list;
@@ -631,18 +639,26 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         w.len = len;
         w.d_head = d_head;
         w.head = head;
-        const int64_t per_lane = int64_t(1) << (P.k0_log2 - 1);
+        const int64_t per_lane = int64_t(4) << P.k0_log2;
         const int grid = grid_of(len / per_lane, P.blocks_per_sm, P);
         const int64_t lanes = int64_t(grid) * P.block;
         w.nclaims = uint32_t(std::min(16 * lanes, len / 3) + 1);
         w.start = int32_t(lanes / kWarp * SidPool::kFirst);
-        w.limit = int32_t(8 * lanes);
-        // sublist id and local offset share 31 bits of a 4-byte record: the longest offset for which
-        // they fit (8 bits for 2^30 elements). A warp may pass the limit once, by up to 32 ids.
-        for (w.lb = out->wide ? 16 : 12;; --w.lb) {
-            w.lcap = out->wide ? kLcap : (1 << w.lb) - 1;
-            w.cap = int32_t(9 * lanes + len / w.lcap + 2);
-            if (out->wide || int64_t(w.cap) <= (int64_t(1) << (31 - w.lb)) || w.lb <= 4) break;
+        // a warp may pass the limit once, by up to 32 ids, and has up to 31 left over in the end
+        if (kNarrow) {
+            w.lcap = Slot4d::kLcap;
+            const int64_t most = (int64_t(1) << Slot4d::kSidBits) - 2 * lanes - (len / w.lcap + 2);
+            w.limit = int32_t(std::min(8 * lanes, most));
+            w.cap = int32_t(w.limit + 2 * lanes + len / w.lcap + 2);
+        } else {
+            // sublist id and local offset share 31 bits of a 4-byte record: the longest offset for which
+            // they fit (8 bits for 2^30 elements)
+            w.limit = int32_t(8 * lanes);
+            for (w.lb = out->wide ? 16 : 12;; --w.lb) {
+                w.lcap = out->wide ? kLcap : (1 << w.lb) - 1;
+                w.cap = int32_t(w.limit + 2 * lanes + len / w.lcap + 2);
+                if (out->wide || int64_t(w.cap) <= (int64_t(1) << (31 - w.lb)) || w.lb <= 4) break;
+            }
         }
         out->lb = w.lb;
         int4 *T = alloc.template get<int4>(w.cap);
@@ -729,7 +745,7 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
 template <class A>
 etl_status rank_plain_list(const int32_t *succ, int64_t len, int32_t head, int32_t *rank, int32_t *status,
                            const RankParams &P, A &alloc, cudaStream_t s) {
-    const bool wide = wide_slots(len), in_place = rank_in_place(len, false);
+    const bool wide = wide_slots(len), in_place = rank_form(len, false) != RankForm::kSeparate;
     const bool overlap = succ < rank + len && rank < succ + len;
     void *recs = wide ? static_cast<void *>(alloc.template get<Slot8::T>(len))
                       : (overlap && !in_place) ? static_cast<void *>(alloc.template get<Slot4::T>(len)) : rank;
@@ -764,6 +780,8 @@ etl_status list_rank(void *list, int64_t len, const int32_t *d_head, int32_t hea
                      int32_t *status, Workspace &ws, RankResult *out) {
     cudaStream_t s = ws.stream();
     const RankParams &P = rank_params();
+    if (dual && rank_form(len, true) == RankForm::kSlots4)
+        return rank_impl<Slot4d, true>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
     if (dual) return rank_impl<Slot8, true>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
     if (wide_slots(len))
         return rank_impl<Slot8, false>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
