@@ -5,24 +5,25 @@
 //   finds the roots of its two ends (with path halving) and hooks the larger
 //   root under the smaller one with a CAS. A CAS that succeeds joins two
 //   different trees, so its edge is a forest edge; exactly n - c succeed.
+//   The successful edges are appended to the forest's list as they are found.
 // Phase 2, Euler tour of the forest (Sec. 2.1): forest edge t owns half-edges
-//   2t = (u_t, v_t) and 2t+1 = (v_t, u_t), so twin(a) = a ^ 1. A counting
-//   sort by tail (atomic slots; the order inside a vertex's group is free,
-//   any cyclic order gives an Euler tour) groups the half-edges of every
-//   vertex (array B); next(a) is
-//   the following entry of B with the same tail, cyclically; succ(a) =
-//   next(twin(a)). Each component's cyclic list is cut in front of the first
-//   half-edge of its root (the smallest vertex, which is where hooking ends),
-//   and the component lists are chained into one list behind a virtual head,
-//   which is ranked once (rank.cu).
-// Phase 3, low / high: with tin(x) = rank of the half-edge entering x (a root
-//   gets the position just before its component), the subtree of u is the
-//   tour interval [tin(u), tout(u)], tout(u) = rank of the half-edge leaving
-//   u. nlo(x) / nhi(x) = min / max of tin(x) and tin(w) over non-forest
-//   edges (x, w), by atomics (the paper uses a segmented reduction);
-//   placed at tin(x) in tour order, low(u) / high(u) are range-min / -max
-//   queries over [tin(u), tout(u)]: one blocked table of (L, H) pairs by
-//   default, else two full sparse tables (rmq.cu).
+//   2t = (u_t, v_t) and 2t+1 = (v_t, u_t), so twin(a) = a ^ 1. Every half-edge
+//   is pushed onto its tail's list (one exchange; the order inside a vertex's
+//   group is free, any cyclic order gives an Euler tour); next(a) is the entry
+//   after it, cyclically; succ(a) = next(twin(a)). Each component's cyclic list
+//   is cut in front of the first half-edge of its root, and the component
+//   lists are chained into one list in any order, which is ranked once
+//   (rank.cu). Tour position = rank + 1; position 0 stands before the tour.
+// Phase 3, low / high: with tin(x) = position of the half-edge entering x (a
+//   root gets the position just before its component), the subtree of u is the
+//   tour interval [tin(u), tout(u)], tout(u) = position of the half-edge
+//   leaving u. Position p starts with (low, high) = (p, p); every non-forest
+//   edge (x, w) updates the entries at tin(x) and tin(w) by atomic min / max
+//   (the paper uses a segmented reduction); low(u) / high(u) are range-min /
+//   -max queries over [tin(u), tout(u)]: one blocked table of (L, H) pairs by
+//   default, else two full sparse tables (rmq.cu). (An entry (p, p) at a
+//   position p inside the interval, also where no vertex is entered, cannot
+//   take the minimum below tin(u) or the maximum above tout(u).)
 // Phase 4, the test: forest edge {u, parent(u)} is a bridge iff
 //   low(u) >= tin(u) and high(u) <= tout(u), i.e. no non-forest edge leaves
 //   the subtree of u. (Sec. 4.1 states the condition the other way round;
@@ -37,30 +38,50 @@ namespace {
 
 constexpr int64_t kFindCap = int64_t(1) << 26;  // bound on pointer-chasing steps of one edge
 
-__global__ void k_init(int32_t n, int32_t *__restrict__ par, int32_t *__restrict__ deg, int32_t *__restrict__ tin) {
+// forest: [0] edges found, [1] first half-edge of the component list (the ranked list's head)
+__global__ void k_init(int32_t n, int32_t *__restrict__ par, int32_t *__restrict__ head, int32_t *__restrict__ tin,
+                       int32_t *__restrict__ forest) {
     pdl_prologue();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        forest[0] = 0;
+        forest[1] = ETL_END;
+    }
     for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n; v += int64_t(gridDim.x) * blockDim.x) {
         par[v] = int32_t(v);
-        deg[v] = 0;
+        head[v] = -1;
         tin[v] = 0;
     }
 }
 
-// root of x with path halving; -1 if the step budget runs out
-__device__ __forceinline__ int32_t find_root(int32_t *par, int32_t x, int64_t &budget) {
+// both ends of edge e; one 8-byte load if the caller's array allows it
+__device__ __forceinline__ int2 load_edge(const int32_t *__restrict__ edges, int64_t e, bool aligned) {
+    return aligned ? __ldcs(reinterpret_cast<const int2 *>(edges) + e)
+                   : make_int2(__ldcs(edges + 2 * e), __ldcs(edges + 2 * e + 1));
+}
+inline bool edges_aligned(const int32_t *edges) { return (reinterpret_cast<uintptr_t>(edges) & 7) == 0; }
+
+// Root of x with path halving; -1 if the step budget runs out. giant (or -1): a root that stays one while
+// this runs, so that pointing at it ends the walk without another load. A node's pointer is read from
+// L2, its parent's through L1 unless `fresh`: parents are few and popular (a large component's root is on
+// every other path, and reads of one address are served one after another by its L2 slice). A stale
+// pointer does no harm: it still leads to an ancestor, a root that is none any more makes the hook's CAS
+// fail or lets it point at an inner node of higher rank; after a failed hook the pointers are read fresh.
+__device__ __forceinline__ int32_t find_root(int32_t *par, int32_t x, int64_t &budget, int32_t giant = -1,
+                                             bool fresh = true) {
     while (budget-- > 0) {
         const int32_t p = __ldcg(par + x);
-        if (p == x) return x;
-        const int32_t gp = __ldcg(par + p);
+        if (p == x || p == giant) return p;
+        const int32_t gp = fresh ? __ldcg(par + p) : __ldca(par + p);
         if (gp == p) return p;
-        par[x] = gp;  // only non-roots are rewritten, always to an ancestor
+        atomicExch(par + x, gp);  // only non-roots are rewritten, always to an ancestor
+        if (gp == giant) return gp;
         x = gp;
     }
     return -1;
 }
 
-// The edges are cut into chunks of kHookChunk consecutive edges, one chunk per block step; one
-// launch hooks positions c0 .. c1 - 1 of the chunk sequence. With `spread` (batches of graphs) the
+// The edges are cut into chunks of kHookChunk consecutive edges; one launch hooks positions c0 .. c1 - 1
+// of the chunk sequence, kHookIlp positions per block step. With `spread` (batches of graphs) the
 // chunks are grouped into superchunks of kHookSuper that are visited in a permuted order
 // (superchunk s of the sequence is s * P mod nsuper, P = 2^31 - 1, a prime above any superchunk
 // count, so the map is a bijection), the chunks of a superchunk in order. The blocks running at one
@@ -70,6 +91,8 @@ __device__ __forceinline__ int32_t find_root(int32_t *par, int32_t x, int64_t &b
 // sequence samples every graph of the batch, not the first ones only. A single graph keeps the
 // contiguous order, which measured faster on it (0.7 against 1.3 ms on 2^25 shuffled edges).
 constexpr int kHookChunk = 256;
+constexpr int kHookIlp = 4;
+constexpr int64_t kHookAtOnce = 98304;  // edges hooked in one launch, without a first slice
 constexpr int kHookSuper = 32;
 
 // number of positions of the chunk sequence over m edges (whole superchunks)
@@ -92,45 +115,111 @@ __device__ __forceinline__ bool hook_above(int32_t a, int32_t b, int32_t giant) 
     return a == giant || (b != giant && a < b);
 }
 
-// skip (may be null): edges to leave out; is_tree (may be null): 1 for edges whose hook succeeded
+// Most edges join two vertices that already point at the same node; those cost two loads, all of a
+// block step's in flight together. The others go to a queue in shared memory, and the block finds and
+// hooks them 256 at a time with every lane busy (one lane's walk to a root held up the other 31 before).
+// The edges that join two trees are appended to the forest's list, one counter update per round. Easy
+// graph of 2^22 vertices and 2^25 edges: 735 us before, 680 with the queue, 530 with the giant root known
+// to find_root, 500 with the halving done by exchanges (a plain store to a sector that others read takes
+// over 1 us); the two loads per edge of its 31.4M later edges alone take 210 us. Batch of 512 graphs: 1430
+// -> 580 us. Graphs of up to kHookAtOnce edges skip the first slice: 2^14 vertices, 2^16 edges 65 -> 50 us.
+// skip (may be null): edges to leave out; is_tree (may be null): 1 for edges whose hook succeeded, and
+// then forest_count, tuv (both ends of forest edge t) and tedge (its edge) are written too
 __global__ void __launch_bounds__(kHookChunk)
-    k_hook(const int32_t *__restrict__ edges, int64_t m, int64_t c0, int64_t c1, bool spread, int32_t n,
-           int32_t *__restrict__ par, uint8_t *__restrict__ is_tree, const uint8_t *__restrict__ skip,
-           const int32_t *__restrict__ d_giant, int32_t *__restrict__ status) {
+    k_hook(const int32_t *__restrict__ edges, bool aligned, int64_t m, int64_t c0, int64_t c1, int ilp, bool spread,
+           int32_t n, int32_t *__restrict__ par, uint8_t *__restrict__ is_tree, const uint8_t *__restrict__ skip,
+           const int32_t *__restrict__ d_giant, int32_t *__restrict__ forest_count, int2 *__restrict__ tuv,
+           int32_t *__restrict__ tedge, int32_t *__restrict__ status) {
     pdl_prologue();
-    const int32_t giant = d_giant ? *d_giant : -1;
+    __shared__ int32_t qa[kHookChunk * (kHookIlp + 1)], qb[kHookChunk * (kHookIlp + 1)], qe[kHookChunk * (kHookIlp + 1)];
+    __shared__ int queued, wins[kHookChunk / 32], first;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t giant = d_giant ? *d_giant : 0;  // vertex 0 ranks above all by its id
     const int64_t nsuper = ((m + kHookChunk - 1) / kHookChunk + kHookSuper - 1) / kHookSuper;
-    for (int64_t c = c0 + blockIdx.x; c < c1; c += gridDim.x) {
-        const int64_t e = hook_chunk(c, nsuper, spread) * kHookChunk + threadIdx.x;
-        if (e >= m) continue;
-        int32_t a = __ldcs(edges + 2 * e), b = __ldcs(edges + 2 * e + 1);
-        uint8_t tree = 0;
-        if (skip && skip[e]) {
-            // left out
-        } else if (a < 0 || a >= n || b < 0 || b >= n) {
-            set_status(status, ETL_EBADGRAPH);
-        } else {
-            int64_t budget = kFindCap;
-            // both ends already point at the same node: same set, nothing to hook
-            const bool same = __ldcg(par + a) == __ldcg(par + b);
-            while (!same) {
-                const int32_t ra = find_root(par, a, budget), rb = find_root(par, b, budget);
-                if (ra < 0 || rb < 0) {
-                    set_status(status, ETL_ETIMEOUT);
-                    break;
-                }
-                if (ra == rb) break;
-                const bool a_up = hook_above(ra, rb, giant);
-                const int32_t hi = a_up ? rb : ra, lo = a_up ? ra : rb;  // hi goes under lo
-                if (atomicCAS(par + hi, hi, lo) == hi) {
-                    tree = 1;
-                    break;
-                }
-                a = ra;  // someone hooked one of the roots meanwhile: retry from them
-                b = rb;
+    if (threadIdx.x == 0) queued = 0;
+    __syncthreads();
+    const int64_t step = int64_t(gridDim.x) * ilp;
+    for (int64_t c = c0 + int64_t(blockIdx.x) * ilp; c < c1; c += step) {
+        int2 ab[kHookIlp];
+        int64_t e[kHookIlp];
+        bool ok[kHookIlp];
+        int32_t pa[kHookIlp], pb[kHookIlp];
+#pragma unroll
+        for (int j = 0; j < kHookIlp; ++j) {
+            e[j] = j < ilp && c + j < c1 ? hook_chunk(c + j, nsuper, spread) * kHookChunk + threadIdx.x : m;
+            ok[j] = e[j] < m;
+            if (ok[j]) ab[j] = load_edge(edges, e[j], aligned);
+        }
+#pragma unroll
+        for (int j = 0; j < kHookIlp; ++j) {
+            if (!ok[j]) continue;
+            if (is_tree) is_tree[e[j]] = 0;
+            if (skip && skip[e[j]]) {
+                ok[j] = false;
+            } else if (ab[j].x < 0 || ab[j].x >= n || ab[j].y < 0 || ab[j].y >= n) {
+                set_status(status, ETL_EBADGRAPH);
+                ok[j] = false;
+            } else {
+                pa[j] = __ldcg(par + ab[j].x);
+                pb[j] = __ldcg(par + ab[j].y);
             }
         }
-        if (is_tree) is_tree[e] = tree;
+#pragma unroll
+        for (int j = 0; j < kHookIlp; ++j)
+            if (ok[j] && pa[j] != pb[j]) {
+                const int i = atomicAdd(&queued, 1);
+                qa[i] = ab[j].x;
+                qb[i] = ab[j].y;
+                qe[i] = int32_t(e[j]);
+            }
+        __syncthreads();
+        const int have = queued, keep = c + step < c1 ? have & (kHookChunk - 1) : 0;  // full rounds, all in the end
+        for (int i0 = keep; i0 < have; i0 += kHookChunk) {
+            const int i = i0 + threadIdx.x;
+            bool won = false;
+            if (i < have) {
+                int32_t a = qa[i], b = qb[i];
+                int64_t budget = kFindCap;
+                bool fresh = false;
+                while (true) {
+                    const int32_t ra = find_root(par, a, budget, giant, fresh), rb = find_root(par, b, budget, giant, fresh);
+                    if (ra < 0 || rb < 0) {
+                        set_status(status, ETL_ETIMEOUT);
+                        break;
+                    }
+                    if (ra == rb) break;
+                    const bool a_up = hook_above(ra, rb, giant);
+                    const int32_t hi = a_up ? rb : ra, lo = a_up ? ra : rb;  // hi goes under lo
+                    if (atomicCAS(par + hi, hi, lo) == hi) {
+                        won = true;
+                        break;
+                    }
+                    a = ra;  // someone hooked one of the roots meanwhile: retry from them
+                    b = rb;
+                    fresh = true;
+                }
+            }
+            if (!is_tree) continue;
+            const unsigned ball = __ballot_sync(kFull, won);
+            if (lane == 0) wins[warp] = __popc(ball);
+            __syncthreads();
+            int before = __popc(ball & lanemask_lt()), total = 0;
+            for (int w = 0; w < kHookChunk / 32; ++w) {
+                if (w < warp) before += wins[w];
+                total += wins[w];
+            }
+            if (threadIdx.x == 0 && total) first = atomicAdd(forest_count, total);
+            __syncthreads();
+            if (won) {
+                const int64_t t = int64_t(first) + before;
+                is_tree[qe[i]] = 1;
+                tuv[t] = make_int2(qa[i], qb[i]);
+                tedge[t] = qe[i];
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) queued = keep;
+        __syncthreads();
     }
 }
 
@@ -138,11 +227,11 @@ __global__ void k_compress(int32_t n, int32_t *__restrict__ par, int32_t *__rest
     pdl_prologue();
     for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n; v += int64_t(gridDim.x) * blockDim.x) {
         int64_t budget = kFindCap;
-        const int32_t r = find_root(par, int32_t(v), budget);
+        const int32_t p = __ldcg(par + v), r = find_root(par, p, budget);
         if (r < 0)
             set_status(status, ETL_ETIMEOUT);
-        else
-            par[v] = r;
+        else if (r != p)
+            atomicExch(par + v, r);
     }
 }
 
@@ -183,239 +272,156 @@ __global__ void __launch_bounds__(kGiantSample) k_giant(const int32_t *__restric
     if (i == 0) *giant = best ? int32_t(~uint32_t(best & 0xffffffffu)) : -1;
 }
 
-// forest edges packed in edge order: tuv[2t] = u, tuv[2t+1] = v, tedge[t] = e
-__global__ void k_forest_edges(const int32_t *__restrict__ edges, int64_t m, const uint8_t *__restrict__ is_tree,
-                               const int32_t *__restrict__ tpos, int32_t *__restrict__ tuv,
-                               int32_t *__restrict__ tedge, int32_t *__restrict__ n_arcs) {
+// next[a] = the half-edge pushed onto its tail's list before a (-1: none). Half-edges of one tail in a
+// warp are linked by the warp and pushed as one run.
+__global__ void k_link_arcs(const int32_t *__restrict__ tuv, const int32_t *__restrict__ forest,
+                            int32_t *__restrict__ head, int32_t *__restrict__ next) {
     pdl_prologue();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *n_arcs = 2 * tpos[m];
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < m; e += int64_t(gridDim.x) * blockDim.x) {
-        if (is_tree[e]) {
-            const int32_t t = tpos[e];
-            tuv[2 * t] = edges[2 * e];
-            tuv[2 * t + 1] = edges[2 * e + 1];
-            tedge[t] = int32_t(e);
-        }
+    const int64_t len = 2 * int64_t(*forest);
+    const int lane = threadIdx.x & 31;
+    for (int64_t base = blockIdx.x * int64_t(blockDim.x); base < len; base += int64_t(gridDim.x) * blockDim.x) {
+        const int64_t a = base + threadIdx.x;
+        const int32_t x = a < len ? tuv[a] : -1;
+        const unsigned peers = __match_any_sync(kFull, x >= 0 ? x : -1 - lane);
+        const int first = __ffs(peers) - 1;
+        int32_t old = -1;
+        if (x >= 0 && lane == first) old = atomicExch(head + x, int32_t(a));
+        old = __shfl_sync(kFull, old, first);
+        const unsigned above = lane < 31 ? peers >> (lane + 1) : 0u;
+        if (a < len) next[a] = above ? int32_t(a) + __ffs(above) : old;
     }
 }
 
-// half-edges per tail vertex
-__global__ void k_arc_count(const int32_t *__restrict__ tuv, const int32_t *__restrict__ d_len,
-                            int32_t *__restrict__ deg) {
-    pdl_prologue();
-    const int64_t len = *d_len;
-    for (int64_t a = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; a < len; a += int64_t(gridDim.x) * blockDim.x)
-        atomicAdd(&deg[tuv[a]], 1);
-}
-
-// B[i] = (half-edge, tail) grouped by tail: off[x] .. off[x+1]-1 are the half-edges leaving x
-__global__ void k_arc_scatter(const int32_t *__restrict__ tuv, const int32_t *__restrict__ d_len,
-                              const int32_t *__restrict__ off, int32_t *__restrict__ deg, int2 *__restrict__ B) {
-    pdl_prologue();
-    const int64_t len = *d_len;
-    for (int64_t a = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; a < len; a += int64_t(gridDim.x) * blockDim.x) {
+// What follows the twin of half-edge a (tail x): the next half-edge of x. The last one is followed by the
+// first, but at a component's root, where the list is cut: there by the first half-edge of the component
+// chained before. on: lanes with a half-edge (all lanes call)
+__device__ __forceinline__ int32_t arc_after(int32_t a, int32_t nb, bool on, const int32_t *__restrict__ tuv,
+                                             const int32_t *__restrict__ par, const int32_t *__restrict__ head,
+                                             int32_t *__restrict__ chain) {
+    bool cut = false;
+    if (on && nb < 0) {
         const int32_t x = tuv[a];
-        const int32_t k = atomicSub(&deg[x], 1) - 1;
-        B[off[x] + k] = make_int2(int32_t(a), x);
+        nb = head[x];
+        cut = par[x] == x;
     }
+    const unsigned m = __ballot_sync(kFull, cut);
+    if (m) {  // the warp's roots form one run of the component list
+        const int lane = threadIdx.x & 31, first = __ffs(m) - 1;
+        const unsigned above = lane < 31 ? m >> (lane + 1) : 0u;
+        const int32_t after = __shfl_sync(kFull, nb, above ? lane + __ffs(above) : lane);
+        int32_t old = ETL_END;
+        if (lane == first) old = atomicExch(chain, nb);
+        old = __shfl_sync(kFull, old, first);
+        if (cut) nb = above ? after : old;
+    }
+    return nb;
 }
 
-// succ(twin(b)) := next(b) for every half-edge b at position i of B; half-edge
-// slots beyond the forest (and the virtual head, set later) are inert
+// the list's elements (len of them, half-edges beyond the forest off it), twins side by side
 template <class S>
-__global__ void k_forest_succ(const int2 *__restrict__ B, const int32_t *__restrict__ d_len, int64_t cap,
-                              const int32_t *__restrict__ off, typename S::T *__restrict__ succ) {
+__global__ void k_forest_list(const int32_t *__restrict__ tuv, int32_t *__restrict__ forest,
+                              const int32_t *__restrict__ par, const int32_t *__restrict__ head,
+                              const int32_t *__restrict__ next, int64_t len, typename S::T *__restrict__ list) {
     pdl_prologue();
-    const int64_t len = *d_len;
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < cap; i += int64_t(gridDim.x) * blockDim.x) {
-        if (i < len) {
-            const int2 bx = B[i];
-            // the group of tail bx.y continues at i + 1 iff that entry has the same tail; only the last
-            // entry of a group reads the group's start
-            const int2 nx = i + 1 < len ? B[i + 1] : make_int2(-1, -1);
-            const int32_t nb = nx.y == bx.y ? nx.x : B[off[bx.y]].x;
-            succ[bx.x ^ 1] = S::make(nb);
-        } else {
-            succ[i] = S::off_list();
-        }
+    const int64_t T = forest[0], pairs = (len + 1) / 2;
+    for (int64_t base = blockIdx.x * int64_t(blockDim.x); base < pairs; base += int64_t(gridDim.x) * blockDim.x) {
+        const int64_t t = base + threadIdx.x;
+        const bool on = t < T;
+        const int2 nb = on ? __ldcs(reinterpret_cast<const int2 *>(next) + t) : make_int2(0, 0);
+        const int32_t s1 = arc_after(int32_t(2 * t), nb.x, on, tuv, par, head, forest + 1);
+        const int32_t s0 = arc_after(int32_t(2 * t + 1), nb.y, on, tuv, par, head, forest + 1);
+        if (2 * t < len) list[2 * t] = on ? S::make(s0) : S::off_list();
+        if (2 * t + 1 < len) list[2 * t + 1] = on ? S::make(s1) : S::off_list();
     }
 }
 
-__global__ void k_root_flags(int32_t n, const int32_t *__restrict__ par, const int32_t *__restrict__ off,
-                             uint8_t *__restrict__ flag) {
-    pdl_prologue();
-    for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n; v += int64_t(gridDim.x) * blockDim.x)
-        flag[v] = (par[v] == v && off[v + 1] > off[v]) ? 1 : 0;
-}
-
-__global__ void k_root_list(int32_t n, const uint8_t *__restrict__ flag, const int32_t *__restrict__ rpos,
-                            int32_t *__restrict__ roots) {
-    pdl_prologue();
-    for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n; v += int64_t(gridDim.x) * blockDim.x)
-        if (flag[v]) roots[rpos[v]] = int32_t(v);
-}
-
-// cut each component's cyclic tour in front of its root's first half-edge and
-// chain the components: virtual head -> comp 0 -> comp 1 -> ... -> end
-template <class S>
-__global__ void k_chain(int32_t n, const int32_t *__restrict__ rpos, const int32_t *__restrict__ roots,
-                        const int2 *__restrict__ B, const int32_t *__restrict__ off, int32_t vhead,
-                        typename S::T *__restrict__ succ) {
-    pdl_prologue();
-    const int32_t c = rpos[n];
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        succ[vhead] = S::make(c > 0 ? B[off[roots[0]]].x : ETL_END);
-    for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < c; k += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t r = roots[k];
-        const int32_t tail = B[off[r + 1] - 1].x ^ 1;  // the half-edge whose successor was the head
-        succ[tail] = S::make((k + 1 < c) ? B[off[roots[k + 1]]].x : ETL_END);
-    }
-}
-
-// tour positions of forest edges: the half-edge ranked first goes down into the child
-__global__ void k_forest_tin(RankResult rr, const int32_t *__restrict__ d_arcs, const int32_t *__restrict__ tuv,
+// tour positions of forest edges: the half-edge ranked first goes down into the child; and of roots
+__global__ void k_forest_tin(RankResult rr, const int32_t *__restrict__ forest, int32_t n, const int2 *__restrict__ tuv,
+                             const int32_t *__restrict__ par, const int32_t *__restrict__ head,
                              int32_t *__restrict__ tin, int32_t *__restrict__ child, int32_t *__restrict__ etin,
                              int32_t *__restrict__ etout) {
     pdl_prologue();
-    const int64_t T = *d_arcs / 2;
-    for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < T; t += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t T = *forest;
+    for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < n; t += int64_t(gridDim.x) * blockDim.x) {
+        const int32_t h = par[t] == t ? head[t] : -1;
+        if (h >= 0) tin[t] = ~rank_at(rr, h);  // a root's, just before its first half-edge, is marked by its sign
+        if (t >= T) continue;
         const int32_t r0 = rank_at(rr, 2 * t), r1 = rank_at(rr, 2 * t + 1);
         if (r0 < 0 || r1 < 0) {  // cannot happen for a forest built above; keep memory safe
-            child[t] = 0;
+            if (child) child[t] = 0;
             etin[t] = etout[t] = -1;
             continue;
         }
-        const int32_t c = r0 < r1 ? tuv[2 * t + 1] : tuv[2 * t];
-        const int32_t a = min(r0, r1), b = max(r0, r1);
+        const int2 uv = tuv[t];
+        const int32_t c = r0 < r1 ? uv.y : uv.x;
+        const int32_t a = min(r0, r1) + 1, b = max(r0, r1) + 1;
         tin[c] = a;
-        child[t] = c;
+        if (child) child[t] = c;
         etin[t] = a;
         etout[t] = b;
     }
 }
 
-__global__ void k_root_tin(int32_t n, const int32_t *__restrict__ rpos, const int32_t *__restrict__ roots,
-                           const int2 *__restrict__ B, const int32_t *__restrict__ off, RankResult rr,
-                           int32_t *__restrict__ tin) {
+// low / high of position p are L[p << shift], H[p << shift]
+__global__ void k_lowhigh_init(int64_t P, int32_t *__restrict__ L, int32_t *__restrict__ H, int shift) {
     pdl_prologue();
-    const int32_t c = rpos[n];
-    for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < c; k += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t r = roots[k];
-        const int32_t p = rank_at(rr, B[off[r]].x);
-        tin[r] = p < 0 ? -1 : p - 1;
-    }
+    for (int64_t p = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; p < P; p += int64_t(gridDim.x) * blockDim.x)
+        L[p << shift] = H[p << shift] = int32_t(p);
 }
 
-__global__ void k_nlo_init(int32_t n, const int32_t *__restrict__ tin, int32_t *__restrict__ nlo,
-                           int32_t *__restrict__ nhi) {
-    pdl_prologue();
-    for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n; v += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t x = tin[v];
-        nlo[v] = x;
-        nhi[v] = x;
-    }
-}
-
-__global__ void k_nontree_minmax(const int32_t *__restrict__ edges, int64_t m, int32_t n,
-                                 const uint8_t *__restrict__ is_tree, const int32_t *__restrict__ tin,
-                                 int32_t *__restrict__ nlo, int32_t *__restrict__ nhi) {
+__global__ void k_nontree_minmax(const int32_t *__restrict__ edges, bool aligned, int64_t m, int32_t n,
+                                 const uint8_t *__restrict__ is_tree, const int32_t *__restrict__ tin, int64_t P,
+                                 int32_t *__restrict__ L, int32_t *__restrict__ H, int shift) {
     pdl_prologue();
     for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < m; e += int64_t(gridDim.x) * blockDim.x) {
         if (__ldcs(is_tree + e)) continue;
-        const int32_t a = __ldcs(edges + 2 * e), b = __ldcs(edges + 2 * e + 1);
+        const int2 ab = load_edge(edges, e, aligned);
+        const int32_t a = ab.x, b = ab.y;
         if (a < 0 || a >= n || b < 0 || b >= n || a == b) continue;
-        const int32_t ta = __ldg(tin + a), tb = __ldg(tin + b);
-        // nlo(x) and nhi(x) start at tin(x): of the four updates only the one lowering the later
-        // end's nlo and the one raising the earlier end's nhi can change anything
-        if (ta < tb) {
-            atomicMax(nhi + a, tb);
-            atomicMin(nlo + b, ta);
-        } else if (tb < ta) {
-            atomicMax(nhi + b, ta);
-            atomicMin(nlo + a, tb);
-        }
+        int32_t ta = __ldg(tin + a), tb = __ldg(tin + b);
+        const bool root = ta < 0 || tb < 0;  // then it is the earlier end
+        if (ta < 0) ta = ~ta;
+        if (tb < 0) tb = ~tb;
+        const int64_t lo = min(ta, tb), hi = max(ta, tb);
+        if (hi >= P || lo == hi) continue;
+        // of the four updates only the one lowering the later end's low and the one raising the earlier
+        // end's high can change anything; a root's entry is in no interval of its component (its position
+        // is the last one of another component's)
+        if (!root) atomicMax(H + (lo << shift), int32_t(hi));
+        atomicMin(L + (hi << shift), int32_t(lo));
     }
 }
 
-// nlo / nhi of every non-root vertex at its tour position; identities at the
-// positions of half-edges going up and at the virtual head (position 0)
-__global__ void k_place(const int32_t *__restrict__ d_arcs, const int32_t *__restrict__ child,
-                        const int32_t *__restrict__ etin, const int32_t *__restrict__ etout,
-                        const int32_t *__restrict__ nlo, const int32_t *__restrict__ nhi, int64_t P,
-                        int32_t *__restrict__ L, int32_t *__restrict__ H) {
-    pdl_prologue();
-    const int64_t T = *d_arcs / 2;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        L[0] = INT_MAX;
-        H[0] = INT_MIN;
-    }
-    for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < T; t += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t c = child[t], a = etin[t], b = etout[t];
-        if (a < 0 || b >= P || a >= b) continue;
-        L[a] = nlo[c];
-        H[a] = nhi[c];
-        L[b] = INT_MAX;
-        H[b] = INT_MIN;
-    }
-}
-
-// blocked form: L and H interleaved (x = L, y = H) in one table of int2
-__global__ void k_place2(const int32_t *__restrict__ d_arcs, const int32_t *__restrict__ child,
-                         const int32_t *__restrict__ etin, const int32_t *__restrict__ etout,
-                         const int32_t *__restrict__ nlo, const int32_t *__restrict__ nhi, int64_t P,
-                         int2 *__restrict__ LH) {
-    pdl_prologue();
-    const int64_t T = *d_arcs / 2;
-    const int2 id = make_int2(INT_MAX, INT_MIN);
-    if (blockIdx.x == 0 && threadIdx.x == 0) LH[0] = id;
-    for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < T; t += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t c = child[t], a = etin[t], b = etout[t];
-        if (a < 0 || b >= P || a >= b) continue;
-        LH[a] = make_int2(nlo[c], nhi[c]);
-        LH[b] = id;
-    }
-}
-
-__global__ void k_bridge_test2(const int32_t *__restrict__ d_arcs, const int32_t *__restrict__ etin,
+// bridges among the forest edges; the mask is zero before, and stays so on a data error
+__global__ void k_bridge_test2(const int32_t *__restrict__ forest, const int32_t *__restrict__ etin,
                                const int32_t *__restrict__ etout, BlockedView<OpMinMax> lh, int64_t P,
-                               uint8_t *__restrict__ tflag) {
+                               const int32_t *__restrict__ tedge, const int32_t *__restrict__ status,
+                               uint8_t *__restrict__ is_bridge) {
     pdl_prologue();
-    const int64_t T = *d_arcs / 2;
+    const int64_t T = *status == 0 ? *forest : 0;
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < T; t += int64_t(gridDim.x) * blockDim.x) {
         const int32_t a = etin[t], b = etout[t];
-        if (a < 0 || b >= P || a >= b) {
-            tflag[t] = 0;
-            continue;
-        }
+        if (a < 0 || b >= P || a >= b) continue;
+        const int2 own = __ldg(lh.x + a);  // the child's own edges alone mostly show that it is none
+        if (own.x < a || own.y > b) continue;
         const int2 r = blocked_query<OpMinMax>(lh, a, b);  // (low, high) of the subtree
-        tflag[t] = (r.x >= a && r.y <= b) ? 1 : 0;
+        if (r.x >= a && r.y <= b) is_bridge[tedge[t]] = 1;
     }
 }
 
-__global__ void k_bridge_test(const int32_t *__restrict__ d_arcs, const int32_t *__restrict__ etin,
+__global__ void k_bridge_test(const int32_t *__restrict__ forest, const int32_t *__restrict__ etin,
                               const int32_t *__restrict__ etout, const int32_t *__restrict__ Lt,
-                              const int32_t *__restrict__ Ht, int64_t P, int64_t ld, uint8_t *__restrict__ tflag) {
+                              const int32_t *__restrict__ Ht, int64_t P, int64_t ld, const int32_t *__restrict__ tedge,
+                              const int32_t *__restrict__ status, uint8_t *__restrict__ is_bridge) {
     pdl_prologue();
-    const int64_t T = *d_arcs / 2;
+    const int64_t T = *status == 0 ? *forest : 0;
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < T; t += int64_t(gridDim.x) * blockDim.x) {
         const int32_t a = etin[t], b = etout[t];
-        if (a < 0 || b >= P || a >= b) {
-            tflag[t] = 0;
-            continue;
-        }
+        if (a < 0 || b >= P || a >= b) continue;
         const int32_t low = sparse_query<false>(Lt, ld, a, b);
         const int32_t high = sparse_query<true>(Ht, ld, a, b);
-        tflag[t] = (low >= a && high <= b) ? 1 : 0;
+        if (low >= a && high <= b) is_bridge[tedge[t]] = 1;
     }
-}
-
-__global__ void k_finalize(int64_t m, const uint8_t *__restrict__ is_tree, const int32_t *__restrict__ tpos,
-                           const uint8_t *__restrict__ tflag, const int32_t *__restrict__ status,
-                           uint8_t *__restrict__ is_bridge) {
-    pdl_prologue();
-    const bool bad = *status != 0;
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < m; e += int64_t(gridDim.x) * blockDim.x)
-        is_bridge[e] = (!bad && is_tree[e]) ? tflag[tpos[e]] : 0;
 }
 
 }  // namespace
@@ -434,20 +440,24 @@ int grid_for(int64_t work, int threads) {
     return int(blocks < 1 ? 1 : blocks);
 }
 
-}  // namespace
-}  // namespace etl
-
-namespace etl {
-namespace {
+// chunks per block step: as many as leave every resident block a step; and the grid
+int hook_ilp(int64_t chunks) {
+    const int64_t each = chunks / (int64_t(num_sms()) * (2048 / kHookChunk));
+    return int(each < 1 ? 1 : each < kHookIlp ? each : kHookIlp);
+}
+int hook_grid(int64_t chunks) {
+    const int64_t blocks = ceil_div(chunks, hook_ilp(chunks)), most = int64_t(num_sms()) * (2048 / kHookChunk);
+    return int(blocks < most ? (blocks < 1 ? 1 : blocks) : most);
+}
 
 // ---- the hybrid of Sec. 4.3: parents and levels of the rooted forest from its Euler tour, then
 // Chaitanya-Kothapalli marking: every non-tree edge walks both ends up to their LCA and marks the
 // tree edges on the way (a tree edge is named by its child); unmarked tree edges are bridges
 
-__global__ void k_tour_pm(const int32_t *__restrict__ d_arcs, const int32_t *__restrict__ etin,
+__global__ void k_tour_pm(const int32_t *__restrict__ forest, const int32_t *__restrict__ etin,
                           const int32_t *__restrict__ etout, int64_t P, int32_t *__restrict__ val) {
     pdl_prologue();
-    const int64_t T = *d_arcs / 2;
+    const int64_t T = *forest;
     if (blockIdx.x == 0 && threadIdx.x == 0) val[0] = 0;  // the virtual head
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < T; t += int64_t(gridDim.x) * blockDim.x) {
         const int32_t a = etin[t], b = etout[t];
@@ -457,12 +467,12 @@ __global__ void k_tour_pm(const int32_t *__restrict__ d_arcs, const int32_t *__r
     }
 }
 
-__global__ void k_tree_records(int32_t n, const int32_t *__restrict__ d_arcs, const int32_t *__restrict__ tuv,
+__global__ void k_tree_records(int32_t n, const int32_t *__restrict__ forest, const int32_t *__restrict__ tuv,
                                const int32_t *__restrict__ child, const int32_t *__restrict__ etin,
                                const int32_t *__restrict__ excl, int64_t P, int2 *__restrict__ trec,
                                uint8_t *__restrict__ mark) {
     pdl_prologue();
-    const int64_t T = *d_arcs / 2;
+    const int64_t T = *forest;
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < T; t += int64_t(gridDim.x) * blockDim.x) {
         const int32_t c = child[t], a = etin[t];
         if (a < 0 || a >= P) continue;
@@ -507,18 +517,18 @@ __global__ void k_ck_mark(const int32_t *__restrict__ edges, int64_t m, int32_t 
     }
 }
 
-__global__ void k_ck_flags(const int32_t *__restrict__ d_arcs, const int32_t *__restrict__ child,
-                           const uint8_t *__restrict__ mark, uint8_t *__restrict__ tflag) {
+__global__ void k_ck_bridges(const int32_t *__restrict__ forest, const int32_t *__restrict__ child,
+                             const uint8_t *__restrict__ mark, const int32_t *__restrict__ tedge,
+                             const int32_t *__restrict__ status, uint8_t *__restrict__ is_bridge) {
     pdl_prologue();
-    const int64_t T = *d_arcs / 2;
+    const int64_t T = *status == 0 ? *forest : 0;
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < T; t += int64_t(gridDim.x) * blockDim.x)
-        tflag[t] = mark[child[t]] ? 0 : 1;
+        if (!mark[child[t]]) is_bridge[tedge[t]] = 1;
 }
 
-etl_status hybrid_marking(const int32_t *edges, int64_t m, int32_t n, const uint8_t *is_tree, const int32_t *tpos,
-                          const int32_t *tuv, const int32_t *n_arcs, const int32_t *child, const int32_t *etin,
-                          const int32_t *etout, int64_t P, uint8_t *tflag, int32_t *st, Workspace &ws) {
-    (void)tpos;
+etl_status hybrid_marking(const int32_t *edges, int64_t m, int32_t n, const uint8_t *is_tree, const int32_t *tuv,
+                          const int32_t *tedge, const int32_t *forest, const int32_t *child, const int32_t *etin,
+                          const int32_t *etout, int64_t P, uint8_t *is_bridge, int32_t *st, Workspace &ws) {
     cudaStream_t s = ws.stream();
     int32_t *val = ws.get<int32_t>(P), *excl = ws.get<int32_t>(P + 1);
     int2 *trec = ws.get<int2>(n);
@@ -527,7 +537,7 @@ etl_status hybrid_marking(const int32_t *edges, int64_t m, int32_t n, const uint
     const int gn = grid_for(n, 256);
     {
         PhaseTimer pt("hybrid.levels", s);
-        launch(k_tour_pm, gn, 256, 0, s, n_arcs, etin, etout, P, val);
+        launch(k_tour_pm, gn, 256, 0, s, forest, etin, etout, P, val);
         note_launch();
     }
     etl_status rc = last_launch();
@@ -536,11 +546,11 @@ etl_status hybrid_marking(const int32_t *edges, int64_t m, int32_t n, const uint
     PhaseTimer pt("hybrid.mark", s);
     launch(k_tree_records_init, gn, 256, 0, s, n, trec);
     note_launch();
-    launch(k_tree_records, gn, 256, 0, s, n, n_arcs, tuv, child, etin, excl, P, trec, mark);
+    launch(k_tree_records, gn, 256, 0, s, n, forest, tuv, child, etin, excl, P, trec, mark);
     note_launch();
     launch(k_ck_mark, grid_for(m, 256), 256, 0, s, edges, m, n, is_tree, trec, mark, st);
     note_launch();
-    launch(k_ck_flags, gn, 256, 0, s, n_arcs, child, mark, tflag);
+    launch(k_ck_bridges, gn, 256, 0, s, forest, child, mark, tedge, st, is_bridge);
     note_launch();
     return last_launch();
 }
@@ -551,32 +561,32 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
                         Workspace &ws, bool hybrid = false, bool spread = false) {
     cudaStream_t s = ws.stream();
     const int64_t A = 2 * int64_t(n - 1);  // half-edge capacity of a spanning forest
-    const int64_t N = A + 1;                // + the virtual head, at index A
-    const int64_t P = N;                    // tour positions 0 .. A
+    const int64_t N = A > 0 ? A : 1;        // elements of the ranked list
+    const int64_t P = A + 1;                // tour positions 0 .. A
     const int levels = sparse_levels(P);
     const int64_t ld = sparse_ld(P);
-    const bool blocked = rmq_params().blocked;
+    const bool blocked = rmq_params().blocked, aligned = edges_aligned(edges);
     const BlockedLayout bl = blocked_layout(P, P);
-    int32_t *par = ws.get<int32_t>(n), *deg = ws.get<int32_t>(n), *off = ws.get<int32_t>(int64_t(n) + 1);
-    int2 *B = ws.get<int2>(A > 0 ? A : 1);
-    int32_t *tin = ws.get<int32_t>(n), *nlo = ws.get<int32_t>(n), *nhi = ws.get<int32_t>(n);
-    uint8_t *is_tree = ws.get<uint8_t>(m), *rflag = ws.get<uint8_t>(n);
-    int32_t *tpos = ws.get<int32_t>(m + 1), *rpos = ws.get<int32_t>(int64_t(n) + 1), *roots = ws.get<int32_t>(n);
-    int32_t *tuv = ws.get<int32_t>(A > 0 ? A : 1), *tedge = ws.get<int32_t>(n);
-    int32_t *n_arcs = ws.get<int32_t>(1), *giant = ws.get<int32_t>(1);
+    int32_t *par = ws.get<int32_t>(n), *head = ws.get<int32_t>(n), *tin = ws.get<int32_t>(n);
+    uint8_t *is_tree = ws.get<uint8_t>(m);
+    int2 *tuv = ws.get<int2>(n);
+    int32_t *arcs = reinterpret_cast<int32_t *>(tuv), *next = ws.get<int32_t>(N + 1);  // tail of / half-edge after each
+    int32_t *tedge = ws.get<int32_t>(n);
+    int32_t *forest = ws.get<int32_t>(2), *giant = ws.get<int32_t>(1);
     const bool wide = wide_slots(N);
-    void *succ = wide ? static_cast<void *>(ws.get<Slot8::T>(N)) : static_cast<void *>(ws.get<Slot4::T>(N));  // slots or successors
-    int32_t *child = ws.get<int32_t>(n), *etin = ws.get<int32_t>(n), *etout = ws.get<int32_t>(n);
-    uint8_t *tflag = ws.get<uint8_t>(n);
+    void *list = wide ? static_cast<void *>(ws.get<Slot8::T>(N)) : static_cast<void *>(ws.get<Slot4::T>(N));  // slots or successors
+    int32_t *child = hybrid ? ws.get<int32_t>(n) : nullptr;
+    int32_t *etin = ws.get<int32_t>(n), *etout = ws.get<int32_t>(n);
     int32_t *Lt = (hybrid || blocked) ? nullptr : ws.get<int32_t>(ld * levels);
     int32_t *Ht = (hybrid || blocked) ? nullptr : ws.get<int32_t>(ld * levels);
     int2 *LH = (!hybrid && blocked) ? ws.get<int2>(bl.elems()) : nullptr;
     if (!ws.ok()) return ETL_ENOMEM;
     etl_status rc = ETL_OK;
     const int gn = grid_for(n, 256), gm = grid_for(m, 256), gA = grid_for(N, 256);
+    memset_async(is_bridge, 0, size_t(m), s);
     {
         PhaseTimer pt("br.init", s);
-        launch(k_init, gn, 256, 0, s, n, par, deg, tin);
+        launch(k_init, gn, 256, 0, s, n, par, head, tin, forest);
         note_launch();
     }
     {
@@ -585,9 +595,9 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
         // With `doubling`, the rest goes in slices that double in size, each followed by a
         // compression, so that no phase builds long paths in a fresh part of the forest.
         const CcParams &C = cc_params();
-        const int64_t slice = int64_t(C.first_slice_quarters) * n / 4;
         const int64_t nchunks = hook_positions(m);
-        int64_t w = ceil_div(slice > 0 ? slice : 1, kHookChunk);  // chunks in the current slice
+        const int64_t slice = int64_t(C.first_slice_quarters) * n / 4;
+        int64_t w = m <= kHookAtOnce ? nchunks : ceil_div(slice > 0 ? slice : 1, kHookChunk);  // chunks in the current slice
         PhaseTimer pt("br.hook", s);
         for (int64_t c0 = 0; c0 < nchunks;) {
             const int64_t c1 = (C.doubling || c0 == 0) ? (c0 + w < nchunks ? c0 + w : nchunks) : nchunks;
@@ -599,89 +609,41 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
                     note_launch();
                 }
             }
-            launch(k_hook, grid_for((c1 - c0) * kHookChunk, kHookChunk), kHookChunk, 0, s, edges, m, c0, c1, spread, n,
-                   par, is_tree, nullptr, (c0 > 0 && C.giant) ? giant : nullptr, st);
+            launch(k_hook, hook_grid(c1 - c0), kHookChunk, 0, s, edges, aligned, m, c0, c1,
+                   hook_ilp(c1 - c0), spread, n, par, is_tree, nullptr, (c0 > 0 && C.giant) ? giant : nullptr, forest, tuv, tedge, st);
             note_launch();
             c0 = c1;
             w *= 2;
         }
     }
-    {
-        PhaseTimer pt("br.compress", s);
-        launch(k_compress, gn, 256, 0, s, n, par, st);
-        note_launch();
-    }
     rc = last_launch();
-    if (!rc) rc = scan_exclusive_u8(is_tree, tpos, m, ws);
     if (!rc) {
-        PhaseTimer pt("br.forest_edges", s);
-        launch(k_forest_edges, gm, 256, 0, s, edges, m, is_tree, tpos, tuv, tedge, n_arcs);
-        note_launch();
-        rc = last_launch();
-    }
-    if (!rc) {
-        PhaseTimer pt("br.group", s);
-        launch(k_arc_count, gA, 256, 0, s, tuv, n_arcs, deg);
-        note_launch();
-        rc = last_launch();
-    }
-    if (!rc) rc = scan_exclusive_i32(deg, off, n, ws);
-    if (!rc) {
-        PhaseTimer pt("br.forest_succ", s);
-        launch(k_arc_scatter, gA, 256, 0, s, tuv, n_arcs, off, deg, B);
+        PhaseTimer pt("br.forest_list", s);
+        launch(k_link_arcs, gA, 256, 0, s, arcs, forest, head, next);
         note_launch();
         if (wide)
-            launch(k_forest_succ<Slot8>, gA, 256, 0, s, B, n_arcs, N, off, static_cast<Slot8::T *>(succ));
+            launch(k_forest_list<Slot8>, gA, 256, 0, s, arcs, forest, par, head, next, N, static_cast<Slot8::T *>(list));
         else
-            launch(k_forest_succ<Slot4>, gA, 256, 0, s, B, n_arcs, N, off, static_cast<Slot4::T *>(succ));
-        note_launch();
-        launch(k_root_flags, gn, 256, 0, s, n, par, off, rflag);
-        note_launch();
-        rc = last_launch();
-    }
-    if (!rc) rc = scan_exclusive_u8(rflag, rpos, n, ws);
-    if (!rc) {
-        PhaseTimer pt("br.chain", s);
-        launch(k_root_list, gn, 256, 0, s, n, rflag, rpos, roots);
-        note_launch();
-        if (wide)
-            launch(k_chain<Slot8>, gn, 256, 0, s, n, rpos, roots, B, off, int32_t(A), static_cast<Slot8::T *>(succ));
-        else
-            launch(k_chain<Slot4>, gn, 256, 0, s, n, rpos, roots, B, off, int32_t(A), static_cast<Slot4::T *>(succ));
+            launch(k_forest_list<Slot4>, gA, 256, 0, s, arcs, forest, par, head, next, N, static_cast<Slot4::T *>(list));
         note_launch();
         rc = last_launch();
     }
     RankResult rr{};
-    if (!rc) rc = list_rank(succ, N, nullptr, int32_t(A), false, -1, st, ws, &rr);
+    if (!rc) rc = list_rank(list, N, forest + 1, 0, false, -1, st, ws, &rr);
     if (!rc) {
-        const int gt = grid_for(n, 256);
-        PhaseTimer pt("br.lowhigh_prep", s);
-        launch(k_forest_tin, gt, 256, 0, s, rr, n_arcs, tuv, tin, child, etin, etout);
-        note_launch();
-        launch(k_root_tin, gn, 256, 0, s, n, rpos, roots, B, off, rr, tin);
+        PhaseTimer pt("br.tin", s);
+        launch(k_forest_tin, gn, 256, 0, s, rr, forest, n, tuv, par, head, tin, child, etin, etout);
         note_launch();
         rc = last_launch();
     }
-    if (hybrid) {
-        if (!rc) rc = hybrid_marking(edges, m, n, is_tree, tpos, tuv, n_arcs, child, etin, etout, P, tflag, st, ws);
-        if (!rc) {
-            launch(k_finalize, gm, 256, 0, s, m, is_tree, tpos, tflag, st, is_bridge);
-            note_launch();
-            rc = last_launch();
-        }
-        return rc;
-    }
+    if (hybrid)
+        return rc ? rc : hybrid_marking(edges, m, n, is_tree, arcs, tedge, forest, child, etin, etout, P, is_bridge, st, ws);
     if (!rc) {
-        const int gt = grid_for(n, 256);
         PhaseTimer pt("br.lowhigh_prep", s);
-        launch(k_nlo_init, gn, 256, 0, s, n, tin, nlo, nhi);
+        int32_t *L = blocked ? reinterpret_cast<int32_t *>(LH) : Lt, *H = blocked ? L + 1 : Ht;
+        launch(k_lowhigh_init, grid_for(P, 256), 256, 0, s, P, L, H, blocked ? 1 : 0);
         note_launch();
-        launch(k_nontree_minmax, gm, 256, 0, s, edges, m, n, is_tree, tin, nlo, nhi);
-        note_launch();
-        if (blocked)
-            launch(k_place2, gt, 256, 0, s, n_arcs, child, etin, etout, nlo, nhi, P, LH);
-        else
-            launch(k_place, gt, 256, 0, s, n_arcs, child, etin, etout, nlo, nhi, P, Lt, Ht);
+        launch(k_nontree_minmax, gm, 256, 0, s, edges, aligned, m, n, is_tree, tin, P, L, H, blocked ? 1 : 0);
         note_launch();
         rc = last_launch();
     }
@@ -694,12 +656,10 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
     if (!rc) {
         PhaseTimer pt("br.test", s);
         if (blocked)
-            launch(k_bridge_test2, grid_for(n, 256), 256, 0, s, n_arcs, etin, etout, blocked_view<OpMinMax>(LH, bl), P,
-                   tflag);
+            launch(k_bridge_test2, gn, 256, 0, s, forest, etin, etout, blocked_view<OpMinMax>(LH, bl), P, tedge, st,
+                   is_bridge);
         else
-            launch(k_bridge_test, grid_for(n, 256), 256, 0, s, n_arcs, etin, etout, Lt, Ht, P, ld, tflag);
-        note_launch();
-        launch(k_finalize, gm, 256, 0, s, m, is_tree, tpos, tflag, st, is_bridge);
+            launch(k_bridge_test, gn, 256, 0, s, forest, etin, etout, Lt, Ht, P, ld, tedge, st, is_bridge);
         note_launch();
         rc = last_launch();
     }
@@ -826,8 +786,8 @@ extern "C" etl_status two_edge_cc(const int32_t *edges, int64_t m, int32_t n, in
     launch(k_iota, gn, 256, 0, s, n, label);
     note_launch();
     if (m > 0) {  // connected components of the graph without its bridges; labels = smallest vertex
-        launch(k_hook, grid_for(m, kHookChunk), kHookChunk, 0, s, edges, m, 0, hook_positions(m), false, n, label,
-               nullptr, is_bridge, nullptr, st);
+        launch(k_hook, hook_grid(hook_positions(m)), kHookChunk, 0, s, edges, edges_aligned(edges), m, 0,
+               hook_positions(m), hook_ilp(hook_positions(m)), false, n, label, nullptr, is_bridge, nullptr, nullptr, nullptr, nullptr, st);
         note_launch();
         launch(k_compress, gn, 256, 0, s, n, label, st);
         note_launch();
