@@ -66,6 +66,9 @@ inline bool edges_aligned(const int32_t *edges) { return (reinterpret_cast<uintp
 // every other path, and reads of one address are served one after another by its L2 slice). A stale
 // pointer does no harm: it still leads to an ancestor, a root that is none any more makes the hook's CAS
 // fail or lets it point at an inner node of higher rank; after a failed hook the pointers are read fresh.
+// MIN (only where ancestors have smaller ids): pointers never move down again, whatever order the writes
+// of several lanes come in.
+template <bool MIN = false>
 __device__ __forceinline__ int32_t find_root(int32_t *par, int32_t x, int64_t &budget, int32_t giant = -1,
                                              bool fresh = true) {
     while (budget-- > 0) {
@@ -73,7 +76,10 @@ __device__ __forceinline__ int32_t find_root(int32_t *par, int32_t x, int64_t &b
         if (p == x || p == giant) return p;
         const int32_t gp = fresh ? __ldcg(par + p) : __ldca(par + p);
         if (gp == p) return p;
-        atomicExch(par + x, gp);  // only non-roots are rewritten, always to an ancestor
+        if (MIN)
+            atomicMin(par + x, gp);
+        else
+            atomicExch(par + x, gp);  // only non-roots are rewritten, always to an ancestor
         if (gp == giant) return gp;
         x = gp;
     }
@@ -223,20 +229,27 @@ __global__ void __launch_bounds__(kHookChunk)
     }
 }
 
+// Points every vertex at its root. EXACT: at the root itself in the end (the labels of components hooked in
+// id order); otherwise a lane that halves a path late may leave a vertex at an inner node.
+template <bool EXACT>
 __global__ void k_compress(int32_t n, int32_t *__restrict__ par, int32_t *__restrict__ status) {
     pdl_prologue();
     for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n; v += int64_t(gridDim.x) * blockDim.x) {
         int64_t budget = kFindCap;
-        const int32_t p = __ldcg(par + v), r = find_root(par, p, budget);
-        if (r < 0)
+        const int32_t p = __ldcg(par + v), r = find_root<EXACT>(par, p, budget);
+        if (r < 0) {
             set_status(status, ETL_ETIMEOUT);
-        else if (r != p)
-            atomicExch(par + v, r);
+        } else if (r != p) {
+            if (EXACT)
+                atomicMin(par + v, r);
+            else
+                atomicExch(par + v, r);
+        }
     }
 }
 
-// The most frequent root among kGiantSample vertices spread over [0, n) (one block; par must be
-// compressed, so par[v] is v's root): the giant component's root when there is one.
+// The root most frequently pointed at among kGiantSample vertices spread over [0, n) (one block; par is
+// compressed, so nearly every vertex points at its root): the giant component's when there is one.
 constexpr int kGiantSample = 1024;
 
 __global__ void __launch_bounds__(kGiantSample) k_giant(const int32_t *__restrict__ par, int32_t n,
@@ -269,7 +282,15 @@ __global__ void __launch_bounds__(kGiantSample) k_giant(const int32_t *__restric
     if (slot >= 0)
         atomicMax(&best, (static_cast<unsigned long long>(cnt[slot]) << 32) | uint32_t(~uint32_t(r)));
     __syncthreads();
-    if (i == 0) *giant = best ? int32_t(~uint32_t(best & 0xffffffffu)) : -1;
+    if (i == 0) {  // k_hook takes it for a root, so it has to be one
+        int32_t r = best ? int32_t(~uint32_t(best & 0xffffffffu)) : 0;
+        for (int64_t budget = kFindCap; budget > 0; --budget) {
+            const int32_t p = __ldcg(par + r);
+            if (p == r) break;
+            r = p;
+        }
+        *giant = r;
+    }
 }
 
 // next[a] = the half-edge pushed onto its tail's list before a (-1: none). Half-edges of one tail in a
@@ -602,7 +623,7 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
         for (int64_t c0 = 0; c0 < nchunks;) {
             const int64_t c1 = (C.doubling || c0 == 0) ? (c0 + w < nchunks ? c0 + w : nchunks) : nchunks;
             if (c0 > 0) {
-                launch(k_compress, gn, 256, 0, s, n, par, st);
+                launch(k_compress<false>, gn, 256, 0, s, n, par, st);
                 note_launch();
                 if (C.giant) {
                     launch(k_giant, 1, kGiantSample, 0, s, par, n, giant);
@@ -789,7 +810,7 @@ extern "C" etl_status two_edge_cc(const int32_t *edges, int64_t m, int32_t n, in
         launch(k_hook, hook_grid(hook_positions(m)), kHookChunk, 0, s, edges, edges_aligned(edges), m, 0,
                hook_positions(m), hook_ilp(hook_positions(m)), false, n, label, nullptr, is_bridge, nullptr, nullptr, nullptr, nullptr, st);
         note_launch();
-        launch(k_compress, gn, 256, 0, s, n, label, st);
+        launch(k_compress<true>, gn, 256, 0, s, n, label, st);
         note_launch();
     }
     launch(k_labels_on_error, gn, 256, 0, s, n, st, label);
