@@ -698,7 +698,8 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
     // ---- upper levels until one CTA can finish the reduced list
     while (lv[nl - 1].cap > kTopCap) {
         Level &L = lv[nl - 1];
-        const uint32_t most = splitters(L.cap, P.k_log2);
+        uint32_t most = splitters(L.cap, P.k_log2);
+        if (most >= uint32_t(kTopCap)) --most;  // with the head's sublist, a power of two again
         L.loc = alloc.template get<int4>(L.cap);
         int4 *up = alloc.template get<int4>(int64_t(most) + 1);
         if (!L.loc || !up || nl >= 32) return ETL_ENOMEM;

@@ -128,20 +128,85 @@ __global__ void k_block_scan(typename Op::T *__restrict__ x, int64_t n, int64_t 
     }
 }
 
-// levels l .. l + count - 1 of the top table from level l - 1 (rows nblk apart, count <= 3)
+// The top table (rows of nblk entries; level l: op over 2^l entries from i) in few launches, each building
+// up to kLowLevels or kHighLevels levels from the one below in shared memory. Three levels a launch,
+// reading the shifted entries from L2, took seven launches and 64 us over 2^19 entries (20 levels), and
+// on small tables the launches were all of it: 2^11 entries 23 us.
+//
+// First levels: a block holds kLowTile entries and the kLowTile after them, thread t the entries t, t +
+// 1024, ...; the entries past the last whole range at each level are not used any more.
+constexpr int kTopThreads = 1024;
+constexpr int kLowLevels = 11, kLowTile = 1 << kLowLevels;
+
 template <class Op>
-__global__ void k_top_levels(typename Op::T *__restrict__ top, int64_t nblk, int l, int count) {
+__global__ void __launch_bounds__(kTopThreads) k_top_low(typename Op::T *__restrict__ top, int64_t nblk, int levels) {
     pdl_prologue();
     using T = typename Op::T;
-    const T *p = top + int64_t(l - 1) * nblk;
-    const int64_t h = int64_t(1) << (l - 1);
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < nblk; i += int64_t(gridDim.x) * blockDim.x) {
-        T m = Op::f(p[i], i + h < nblk ? p[i + h] : Op::id());
-        top[int64_t(l) * nblk + i] = m;
-        for (int c = 1; c < count; ++c) {
-            const int64_t w = h << c;  // the next level adds the 2^c shifted entries w .. 2w - 1 (steps of h)
-            for (int64_t j = w; j < 2 * w; j += h) m = Op::f(m, i + j < nblk ? p[i + j] : Op::id());
-            top[int64_t(l + c) * nblk + i] = m;
+    constexpr int kPer = 2 * kLowTile / kTopThreads;
+    __shared__ T sm[2 * kLowTile];
+    const int64_t base = int64_t(blockIdx.x) * kLowTile;
+    T v[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int64_t i = base + threadIdx.x + j * kTopThreads;
+        v[j] = i < nblk ? top[i] : Op::id();
+        sm[threadIdx.x + j * kTopThreads] = v[j];
+    }
+    for (int l = 1; l <= levels; ++l) {
+        const int h = 1 << (l - 1);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int i = threadIdx.x + j * kTopThreads + h;
+            if (i < 2 * kLowTile) v[j] = Op::f(v[j], sm[i]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int i = threadIdx.x + j * kTopThreads;
+            sm[i] = v[j];
+            if (i < kLowTile && base + i < nblk) top[int64_t(l) * nblk + base + i] = v[j];
+        }
+    }
+}
+
+// Further levels l0 + 1 .. l0 + levels: level l0's row read as a matrix with 2^l0 columns; a level is a
+// shift by whole matrix rows. A block takes 128 bytes of columns and kHighTile matrix rows, and the
+// 2^kHighLevels rows after them.
+constexpr int kHighLevels = 8, kHighTile = 128, kHighRows = kHighTile + (1 << kHighLevels);
+
+template <class Op>
+__global__ void __launch_bounds__(kTopThreads)
+    k_top_high(typename Op::T *__restrict__ top, int64_t nblk, int l0, int levels) {
+    pdl_prologue();
+    using T = typename Op::T;
+    constexpr int kCols = 128 / sizeof(T), kLanes = kTopThreads / kCols, kPer = kHighRows / kLanes;
+    __shared__ T sm[kHighRows][kCols];
+    const int c = threadIdx.x % kCols, y = threadIdx.x / kCols;
+    const int64_t col = int64_t(blockIdx.x) * kCols + c, row0 = int64_t(blockIdx.y) * kHighTile;
+    const T *p = top + int64_t(l0) * nblk;
+    T v[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int64_t i = ((row0 + y + j * kLanes) << l0) + col;
+        v[j] = i < nblk ? p[i] : Op::id();
+        sm[y + j * kLanes][c] = v[j];
+    }
+    for (int l = 1; l <= levels; ++l) {
+        const int h = 1 << (l - 1);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int r = y + j * kLanes + h;
+            if (r < kHighRows) v[j] = Op::f(v[j], sm[r][c]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int r = y + j * kLanes;
+            sm[r][c] = v[j];
+            const int64_t i = ((row0 + r) << l0) + col;
+            if (r < kHighTile && i < nblk) top[int64_t(l0 + l) * nblk + i] = v[j];
         }
     }
 }
@@ -177,12 +242,18 @@ etl_status blocked_build(typename Op::T *base, int64_t n, const BlockedLayout &L
         note_launch();
     }
     etl_status st = last_launch();
-    for (int l = 1; !st && l < L.tlevels;) {
-        const int count = L.tlevels - l >= 3 ? 3 : L.tlevels - l;
-        int blocks = int(ceil_div(L.nblk, 256));
-        if (blocks > grid_cap) blocks = grid_cap;
+    for (int l = 0; !st && l + 1 < L.tlevels;) {  // levels up to l are built
+        const int most = l == 0 ? kLowLevels : kHighLevels;
+        const int count = L.tlevels - 1 - l < most ? L.tlevels - 1 - l : most;
         PhaseTimer pt("rmq.top", s);
-        launch(k_top_levels<Op>, blocks, 256, 0, s, top, L.nblk, l, count);
+        if (l == 0) {
+            launch(k_top_low<Op>, unsigned(ceil_div(L.nblk, kLowTile)), kTopThreads, 0, s, top, L.nblk, count);
+        } else {
+            const int64_t cols = (int64_t(1) << l) / (128 / int64_t(sizeof(T)));
+            const int64_t rows = ceil_div(L.nblk, int64_t(1) << l);
+            launch(k_top_high<Op>, dim3(unsigned(cols), unsigned(ceil_div(rows, kHighTile))), kTopThreads, 0, s, top,
+                   L.nblk, l, count);
+        }
         note_launch();
         st = last_launch();
         l += count;
