@@ -49,35 +49,12 @@
 #include <mutex>
 #include <type_traits>
 
-#include "etl_internal.cuh"
+#include "rank_top.cuh"
 
 namespace etl {
 namespace {
 
 constexpr int32_t kLcap = 4096;  // longest sublist of 8-byte records (< 2^15)
-constexpr int kTopThreads = 1024;
-constexpr int kTopCap = 15360;   // entries one CTA ranks in shared memory (12 bytes each)
-constexpr int kTopSub = 2 * kTopThreads;
-constexpr int32_t kEndT = 0x7fffffff;  // "no successor" in a reduced list's entry
-constexpr int32_t kVisited = int32_t(0x80000000u);
-constexpr uint32_t kMul = 0x9E3779B1u;  // odd, so multiplication is a bijection mod 2^b
-
-constexpr uint32_t inverse_mod_2_32(uint32_t a) {  // Newton iteration for a^-1 mod 2^32 (a odd)
-    uint32_t x = a;
-    for (int i = 0; i < 5; ++i) x *= 2u - a * x;
-    return x;
-}
-
-struct Hash {
-    uint32_t mask, S0;  // elements [0, mask], splitters hash below S0
-    __device__ __forceinline__ bool split(uint32_t e) const { return ((e * kMul) & mask) < S0; }
-    __device__ __forceinline__ int32_t sid(uint32_t e) const { return int32_t((e * kMul) & mask); }
-    __device__ __forceinline__ uint32_t elem(uint32_t s) const {
-        constexpr uint32_t kInv = inverse_mod_2_32(kMul);
-        return (s * kInv) & mask;
-    }
-};
-
 // candidate w >= 1 of a list of len elements: floor(frac(w * golden ratio) * len). The distance of any
 // two of the first W multiples is above 0.38 / W, so W <= len / 3 candidates are distinct elements.
 __device__ __forceinline__ int64_t candidate(uint32_t w, int64_t len) {
@@ -369,12 +346,8 @@ __global__ void k_walk(const int4 *__restrict__ T, int64_t base, const int32_t *
 // ------------------------------------------------------------ top level: one CTA, shared memory
 
 // FROM_LIST: the list itself instead of a reduced list; each element on it becomes its own sublist in
-// the result. Shared memory holds the entries (three words each); at most kTopSub - 1 splitters and the
-// head cut them into sublists, and those are ranked by pointer jumping: Q = predecessor, V1 / V2 = sums
-// over the segment (Q, e], F = first sublist of that segment. A round replaces Q by Q[Q] and adds the
-// predecessor's segment; after ceil(log2 kTopSub) rounds every Q is -1 and V is the inclusive prefix
-// from the list head, F the head's sublist. One SM issues all of it, so the steps are kept to a few
-// instructions (claims as in the in-place walk, tried here, took twice the time).
+// the result. One SM issues all of it, so the steps are kept to a few instructions (claims as in the
+// in-place walk, tried here, took twice the time; pointer jumping over all entries three times).
 constexpr int kTopBatch = 5;  // entries per thread whose loads are in flight together
 
 template <class S, bool DUAL, bool FROM_LIST>
@@ -384,18 +357,10 @@ __global__ void __launch_bounds__(kTopThreads)
           int32_t head_value, int64_t expect_total, int32_t *__restrict__ status) {
     pdl_prologue();
     extern __shared__ int32_t sm[];
-    __shared__ int found;
-    int32_t *Q = sm, *V1 = sm + kTopSub, *V2 = sm + 2 * kTopSub, *F = sm + 3 * kTopSub, *SN = sm + 4 * kTopSub;
+    __shared__ TopShared sh;
     const int len = int(level_len(base, d_add, cap));
-    int32_t *nx = sm + 5 * kTopSub, *a1 = nx + len, *a2 = a1 + len;
+    int32_t *nx = sm, *a1 = nx + len, *a2 = a1 + len;
     const int32_t head = d_head ? *d_head : head_value;
-    Hash H;
-    const int b = len <= 1 ? 0 : 32 - __clz(len - 1);
-    H.mask = (1u << b) - 1u;
-    H.S0 = min((H.mask + 1u) >> 1, uint32_t(kTopSub - 1));
-    const bool head_split = H.split(uint32_t(head));
-    const int32_t head_sub = head_split ? H.sid(uint32_t(head)) : int32_t(H.S0);
-    if (threadIdx.x == 0) found = 0;
     for (int i = threadIdx.x; i < len; i += kTopBatch * kTopThreads) {
         int4 t[kTopBatch];
         uint32_t v[kTopBatch];
@@ -422,118 +387,34 @@ __global__ void __launch_bounds__(kTopThreads)
                 // anything that is no element ends the list (the total is checked)
                 nx[e] = (nxt < 0 || nxt >= len) ? kEndT : nxt;
                 a1[e] = w1;
-                a2[e] = (DUAL && (e & 1) == 0) ? 1 : 0;
+                if (DUAL) a2[e] = (e & 1) == 0 ? 1 : 0;
                 if (nxt != ETL_END && nxt >= len && v[j] != Slot4::kOff) set_status(status, ETL_EBADTREE);
                 if (!DUAL && nxt < ETL_END) set_status(status, ETL_EBADTREE);
                 if (!DUAL && expect_total >= 0 && v[j] == Slot4::kOff) set_status(status, ETL_EBADTREE);
             } else {
                 nx[e] = t[j].z;
                 a1[e] = t[j].x;
-                a2[e] = t[j].y;
+                if (DUAL) a2[e] = t[j].y;
             }
         }
     }
     __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int w = threadIdx.x + k * kTopThreads;
-        const int32_t e0 = w < int(H.S0) ? int32_t(H.elem(uint32_t(w))) : w == int(H.S0) && !head_split ? head : len;
-        int32_t e = e0, x1 = 0, x2 = 0, link = kEndT;
-        while (e >= 0 && e < len) {
-            const int32_t z = nx[e], y1 = a1[e], y2 = a2[e];
-            if (z < 0) {  // visited before: no list
-                set_status(status, ETL_EBADTREE);
-                break;
-            }
-            nx[e] = kVisited | w;
-            a1[e] = x1;
-            a2[e] = x2;
-            x1 += y1;
-            x2 += y2;
-            e = z;
-            if (z < len && H.split(uint32_t(z))) {
-                link = H.sid(uint32_t(z));
-                break;
-            }
-        }
-        Q[w] = -1;
-        V1[w] = x1;
-        V2[w] = x2;
-        F[w] = w;
-        SN[w] = link;
-    }
-    __syncthreads();
-    int32_t s1[2], s2[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int w = threadIdx.x + k * kTopThreads;
-        s1[k] = V1[w];
-        s2[k] = V2[w];
-        const int32_t s = SN[w];
-        if (s != kEndT) Q[s] = w;  // a link is a sublist id below kTopSub
-    }
-    __syncthreads();
-    int rounds = 0;
-    while (true) {
-        int32_t nq[2], n1[2], n2[2], nf[2];
-        int any = 0;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int w = threadIdx.x + k * kTopThreads;
-            const int32_t q = Q[w];
-            if (q >= 0) {
-                nq[k] = Q[q];
-                n1[k] = V1[w] + V1[q];
-                n2[k] = V2[w] + V2[q];
-                nf[k] = F[q];
-                any = 1;
-            } else {
-                nq[k] = -1;
-                n1[k] = V1[w];
-                n2[k] = V2[w];
-                nf[k] = F[w];
-            }
-        }
-        any = __syncthreads_or(any);
-        if (!any) break;
-        if (++rounds > 40) {  // a cycle: cannot happen on a valid list
-            if (threadIdx.x == 0) set_status(status, ETL_EBADTREE);
-            break;
-        }
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int w = threadIdx.x + k * kTopThreads;
-            Q[w] = nq[k];
-            V1[w] = n1[k];
-            V2[w] = n2[k];
-            F[w] = nf[k];
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int w = threadIdx.x + k * kTopThreads;
-        if (expect_total >= 0 && SN[w] == kEndT && F[w] == head_sub && int64_t(V1[w]) == expect_total) found = 1;
-        V1[w] -= s1[k];  // exclusive
-        V2[w] -= s2[k];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && expect_total >= 0 && !found) set_status(status, ETL_EBADTREE);
+    rank_in_shared<DUAL>(len, head, expect_total, sh, nx, a1, a2, status);
     for (int e = threadIdx.x; e < len; e += kTopThreads) {
         const int32_t z = nx[e];
         if (z >= 0) continue;  // on no walk
-        const int32_t s = z & ~kVisited;
+        const int32_t s = z & ~kVisited, r = sh.V1[s] + a1[e], o = DUAL ? sh.V2[s] + a2[e] : 0;
         if (FROM_LIST) {
-            T[e] = make_int4(V1[s] + a1[e], V2[s] + a2[e], 0, 0);
+            T[e] = make_int4(r, o, 0, 0);
             const bool leaf = DUAL && int32_t(succ[e]) < ETL_END;
             recs[e] = S::rec(e, 0, leaf ? 0x8000u : 0u, lb);
         } else {
-            *reinterpret_cast<int2 *>(T + e) = make_int2(V1[s] + a1[e], V2[s] + a2[e]);
+            *reinterpret_cast<int2 *>(T + e) = make_int2(r, o);
         }
     }
 }
 
-size_t top_smem(int64_t len) { return size_t(5 * kTopSub + 3 * len) * sizeof(int32_t); }
+size_t top_smem(int64_t len, bool dual) { return size_t((dual ? 3 : 2) * len) * sizeof(int32_t); }
 
 // an entry's weights give way to the prefix over the whole list
 __global__ void k_expand(int4 *__restrict__ T, const int4 *__restrict__ loc, int64_t base,
@@ -609,8 +490,8 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
     if (!recs) return ETL_ENOMEM;
     out->recs = recs;
     const uint32_t *succ = static_cast<const uint32_t *>(list);
-    cudaFuncSetAttribute(k_top<S, DUAL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap)));
-    cudaFuncSetAttribute(k_top<S, DUAL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap)));
+    cudaFuncSetAttribute(k_top<S, DUAL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap, DUAL)));
+    cudaFuncSetAttribute(k_top<S, DUAL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap, DUAL)));
     etl_status st;
     if (len <= kTopCap) {
         int4 *T = alloc.template get<int4>(len);
@@ -618,7 +499,7 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         out->T = T;
         out->rcap = len;
         PhaseTimer pt("rank.top", s);
-        launch(k_top<S, DUAL, true>, 1, kTopThreads, top_smem(len), s, succ, static_cast<R *>(recs), out->lb, T, len,
+        launch(k_top<S, DUAL, true>, 1, kTopThreads, top_smem(len, DUAL), s, succ, static_cast<R *>(recs), out->lb, T, len,
                nullptr, len, d_head, head, expect_len, status);
         note_launch();
         return last_launch();
@@ -720,7 +601,7 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
     {
         const Level &L = lv[nl - 1];
         PhaseTimer ptp("rank.top", s);
-        launch(k_top<S, DUAL, false>, 1, kTopThreads, top_smem(L.cap), s, nullptr, nullptr, 0, L.T, L.base, L.d_add,
+        launch(k_top<S, DUAL, false>, 1, kTopThreads, top_smem(L.cap, DUAL), s, nullptr, nullptr, 0, L.T, L.base, L.d_add,
                L.cap, L.d_head, 0, expect_len, status);
         note_launch();
         st = last_launch();
