@@ -64,8 +64,10 @@ cudaError_t dev_alloc(void **p, size_t bytes, cudaStream_t s);
 cudaError_t memset_async(void *p, int value, size_t bytes, cudaStream_t s);
 cudaError_t copy_d2d_async(void *dst, const void *src, size_t bytes, cudaStream_t s);
 
-// Stream-ordered scratch: every buffer taken here is released with
-// cudaFreeAsync on the same stream when the Workspace goes out of scope.
+// Stream-ordered scratch: released with cudaFreeAsync on the same stream when the Workspace goes out of
+// scope. Small buffers are cut from chunks, so that a call on a small input asks the allocator for memory
+// once or twice and not for each of its dozen buffers (1 us of host time for each pair of calls); buffers
+// in a caller's arena are cut from that one by one.
 class Workspace {
   public:
     explicit Workspace(cudaStream_t s) : s_(s), arena_(current_arena() != nullptr) {}
@@ -74,27 +76,44 @@ class Workspace {
     Workspace &operator=(const Workspace &) = delete;
     template <class T>
     T *get(size_t count) {
-        void *p = nullptr;
         size_t bytes = count * sizeof(T);
         if (bytes == 0) bytes = 16;
-        if (dev_alloc(&p, bytes, s_) != cudaSuccess) {
-            ok_ = false;
-            return nullptr;
+        if (arena_ || bytes > kSmall) return static_cast<T *>(take(bytes));
+        bytes = (bytes + 255) & ~size_t(255);
+        if (bytes > left_) {
+            at_ = static_cast<char *>(take(kChunk));
+            left_ = at_ ? kChunk : 0;
+            if (!at_) return nullptr;
         }
-        bufs_.push_back(p);
-        return static_cast<T *>(p);
+        char *p = at_;
+        at_ += bytes;
+        left_ -= bytes;
+        return reinterpret_cast<T *>(p);
     }
     bool ok() const { return ok_; }
     void release() {
         if (!arena_)
             for (void *p : bufs_) cudaFreeAsync(p, s_);
         bufs_.clear();
+        left_ = 0;
     }
     cudaStream_t stream() const { return s_; }
 
   private:
+    static constexpr size_t kChunk = size_t(4) << 20, kSmall = size_t(1) << 20;
+    void *take(size_t bytes) {
+        void *p = nullptr;
+        if (dev_alloc(&p, bytes, s_) != cudaSuccess) {
+            ok_ = false;
+            return nullptr;
+        }
+        bufs_.push_back(p);
+        return p;
+    }
     cudaStream_t s_;
     std::vector<void *> bufs_;
+    char *at_ = nullptr;  // rest of the current chunk
+    size_t left_ = 0;
     bool ok_ = true;
     bool arena_;  // buffers come from a caller-owned arena: nothing to free
 };
@@ -451,5 +470,13 @@ struct etl_lca_s {
     void *tour_table = nullptr;  // Euler-tour RMQ: blocked table of (depth << 32 | node) keys over 2n positions
     int32_t *tpos = nullptr;     // Euler-tour RMQ: tour position of each node's opening bracket
     etl::BlockedLayout tbl{};
+    void *block = nullptr;       // the allocation that pre .. order, table, nrec, status and node_off are cut from
     bool arena = false;          // device arrays live in a caller-owned workspace: lca_free frees none of them
 };
+
+namespace etl {
+// Single trees of up to kTinyNodes nodes with the blocked table (or none): all of the preprocessing in one
+// launch (tiny.cu).
+constexpr int kTinyNodes = 4096;
+etl_status build_tiny_tree(const int32_t *parent, etl_lca_s *h, cudaStream_t s);
+}  // namespace etl

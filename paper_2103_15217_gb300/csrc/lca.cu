@@ -344,9 +344,7 @@ void free_handle(etl_lca_s *h) {
         return;
     }
     cudaStream_t s = h->stream;
-    for (int32_t *p : {h->pre, h->depth, h->size, h->order, h->table, h->status, h->node_off})
-        if (p) cudaFreeAsync(p, s);
-    for (void *p : {h->inrec, h->inpath, h->tour_table, static_cast<void *>(h->tpos), h->nrec})
+    for (void *p : {h->block, h->inrec, h->inpath, h->tour_table, static_cast<void *>(h->tpos)})
         if (p) cudaFreeAsync(p, s);
     delete h;
 }
@@ -366,21 +364,38 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
     h->blocked = rmq_params().blocked;
     h->bl = blocked_layout(n, max_n);
     const size_t table_bytes = (h->blocked ? size_t(h->bl.elems()) : size_t(h->ld) * size_t(h->levels)) * 4;
+    // one allocation for all arrays of the handle, each 256-byte aligned in it
     const size_t nb = size_t(n) * sizeof(int32_t);
-    bool ok = dev_alloc((void **)&h->pre, nb, s) == cudaSuccess;
-    ok = ok && dev_alloc((void **)&h->depth, nb, s) == cudaSuccess;
-    ok = ok && dev_alloc((void **)&h->size, nb, s) == cudaSuccess;
-    ok = ok && dev_alloc((void **)&h->order, nb, s) == cudaSuccess;
-    if (with_table)
-        ok = ok && dev_alloc((void **)&h->table, table_bytes, s) == cudaSuccess;
-    if (with_table && h->blocked)
-        ok = ok && dev_alloc((void **)&h->nrec, size_t(n) * sizeof(int4), s) == cudaSuccess;
-    ok = ok && dev_alloc((void **)&h->status, sizeof(int32_t), s) == cudaSuccess;
-    if (ok && batch)
-        ok = dev_alloc((void **)&h->node_off, size_t(k + 1) * sizeof(int32_t), s) == cudaSuccess;
-    if (!ok) {
+    const size_t bytes[8] = {nb, nb, nb, nb, sizeof(int32_t), with_table ? table_bytes : 0,
+                             with_table && h->blocked ? size_t(n) * sizeof(int4) : 0,
+                             batch ? size_t(k + 1) * sizeof(int32_t) : 0};
+    size_t at[8], total = 0;
+    for (int i = 0; i < 8; ++i) {
+        at[i] = total;
+        total += (bytes[i] + 255) & ~size_t(255);
+    }
+    if (dev_alloc(&h->block, total, s) != cudaSuccess) {
+        h->block = nullptr;
         free_handle(h);
         return ETL_ENOMEM;
+    }
+    auto part = [&](int i) { return bytes[i] ? reinterpret_cast<int32_t *>(static_cast<char *>(h->block) + at[i]) : nullptr; };
+    h->pre = part(0);
+    h->depth = part(1);
+    h->size = part(2);
+    h->order = part(3);
+    h->status = part(4);
+    h->table = part(5);
+    h->nrec = part(6);
+    h->node_off = part(7);
+    if (!batch && n <= kTinyNodes && (h->blocked || !with_table)) {
+        const etl_status st = build_tiny_tree(parent, h, s);
+        if (st) {
+            free_handle(h);
+            return st;
+        }
+        *out = h;
+        return ETL_OK;
     }
     memset_async(h->status, 0, sizeof(int32_t), s);
     if (batch) copy_d2d_async(h->node_off, node_off, size_t(k + 1) * sizeof(int32_t), s);
