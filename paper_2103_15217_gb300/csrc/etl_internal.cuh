@@ -381,11 +381,6 @@ struct OpMin {
     __device__ static __forceinline__ T id() { return INT32_MAX; }
     __device__ static __forceinline__ T f(T a, T b) { return min(a, b); }
 };
-struct OpMax {
-    using T = int32_t;
-    __device__ static __forceinline__ T id() { return INT32_MIN; }
-    __device__ static __forceinline__ T f(T a, T b) { return max(a, b); }
-};
 struct OpMinKey {  // 64-bit keys: a value in the high half, a payload it carries in the low half
     using T = long long;
     __device__ static __forceinline__ T id() { return INT64_MAX; }
@@ -407,12 +402,13 @@ struct BlockedLayout {
 };
 // a table over n entries answering ranges of up to max_len entries
 BlockedLayout blocked_layout(int64_t n, int64_t max_len);
-// x (first n entries of base) must be filled; builds pad, pm, sm and top. pairs (int32 entries only):
-// pm and sm interleaved as (pm[i], sm[i]) pairs in the 2N entries after x (then blocked_query, which
-// reads them as separate arrays, must not be used on the table; x and top are unchanged)
+// x (first n entries of base) must be filled; builds pad, pm, sm and top
 template <class Op>
-etl_status blocked_build(typename Op::T *base, int64_t n, const BlockedLayout &L, cudaStream_t s,
-                         bool pairs = false);
+etl_status blocked_build(typename Op::T *base, int64_t n, const BlockedLayout &L, cudaStream_t s);
+// the top table from its first row. (A handle's table has pm and sm interleaved as (pm[i], sm[i]) pairs in
+// the 2N entries after x, built in lca.cu: blocked_query, which reads them as separate arrays, is not for it.)
+template <class Op>
+etl_status blocked_top(typename Op::T *top, const BlockedLayout &L, cudaStream_t s);
 
 template <class Op>
 struct BlockedView {

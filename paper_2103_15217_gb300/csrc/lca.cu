@@ -19,12 +19,10 @@
 //      prefix sum of Sec. 2); size = (rank(2v+1) - rank(2v) + 1) / 2. In a
 //      chained batch, tree i occupies preorder positions node_off[i] ..
 //      node_off[i+1]-1 and depth / size come out per tree.
-//   6. k_parent_pre: Q[i] = pre(parent(order[i])), level 0 of the range-minimum
-//      table, written in preorder (a separate pass: gathering pre[] is cheaper
-//      than re-deriving the parent's preorder from its bracket record).
-//   7. range-minimum table over Q (rmq.cu): by default the blocked two-level
-//      table (in-block prefix / suffix minima plus a sparse table over blocks
-//      of 32), else a full sparse table; sized for the largest tree.
+//   6. k_parent_pre: Q[i] = pre(parent(order[i])), level 0 of the range-minimum table, in preorder, with
+//      the in-block prefix / suffix minima of the blocked table.
+//   7. the rest of the range-minimum table over Q (rmq.cu): by default the sparse table over blocks of
+//      32 (the blocked two-level table), else a full sparse table; sized for the largest tree.
 //
 // Query: for u != v with i = min(pre u, pre v), j = max(...), every node with
 // preorder in (i, j] is a proper descendant of LCA(u, v), and the child of the
@@ -77,7 +75,8 @@ __global__ void k_tour_assemble(const int32_t *__restrict__ par, const int32_t *
     pdl_prologue();
     for (int64_t t = gtid(); t < n; t += gstride()) {
         const int32_t p = __ldcs(par + t), h = __ldcs(head + t), x = __ldcs(next + t);
-        const int32_t c = x >= 0 ? 2 * x : p >= 0 ? 2 * p + 1 : ETL_END;  // leave t -> enter next sibling, or leave p
+        // leave t -> enter next sibling, or leave p; leave a root -> enter the next root
+        const int32_t c = x >= 0 ? 2 * x : p >= 0 ? 2 * p + 1 : x < -1 ? 2 * (-2 - x) : ETL_END;
         const bool one = h < 0 && p >= 0;                                 // a leaf, and no root
         const int32_t a = one ? int32_t(uint32_t(c) | 0x80000000u) : h >= 0 ? 2 * h : 2 * int32_t(t) + 1;
         if constexpr (std::is_same<S, Slot8>::value)
@@ -101,7 +100,7 @@ __global__ void k_link_roots(const int32_t *__restrict__ root_cnt, const int32_t
         const int32_t r = root_of[i];
         if (r < 0 || r >= n) continue;
         const int32_t nr = (i + 1 < k) ? root_of[i + 1] : -1;
-        next[r] = (nr >= 0 && nr < n) ? nr : -1;
+        next[r] = (nr >= 0 && nr < n) ? -2 - nr : -1;  // told apart from a sibling by its sign
     }
 }
 
@@ -134,9 +133,12 @@ __device__ __forceinline__ NodeRecs node_recs(uint2 q) {
     return r;
 }
 
+// next (null: plain node ids): order[] entries carry what k_parent_pre needs to know of the node in their
+// top bits, 0: it has children, 1: a leaf with a next sibling, 2: a leaf without
 template <class Q>
-__global__ void k_node_stats(RankResult rr, int32_t n, int32_t *__restrict__ pre, int32_t *__restrict__ depth,
-                             int32_t *__restrict__ size, int32_t *__restrict__ order, int32_t *__restrict__ status) {
+__global__ void k_node_stats(RankResult rr, int32_t n, const int32_t *__restrict__ next, int32_t *__restrict__ pre,
+                             int32_t *__restrict__ depth, int32_t *__restrict__ size, int32_t *__restrict__ order,
+                             int32_t *__restrict__ status) {
     pdl_prologue();
     const Q *recs = static_cast<const Q *>(rr.recs);
     for (int64_t t = gtid(); t < n; t += gstride()) {
@@ -152,33 +154,86 @@ __global__ void k_node_stats(RankResult rr, int32_t n, int32_t *__restrict__ pre
         const int32_t p = A.y + r.oa;
         __stcs(pre + t, p);
         __stcs(depth + t, 2 * p - r0);
-        __stcs(size + t, (r1 - r0 + 1) >> 1);
-        if (p >= 0 && p < n) order[p] = int32_t(t);
+        const int32_t sz = (r1 - r0 + 1) >> 1;
+        __stcs(size + t, sz);
+        uint32_t kind = 0;
+        if (next) {
+            const int32_t x = __ldcs(next + t);
+            kind = sz > 1 ? 0u : x >= 0 ? 1u : 2u;
+        }
+        if (p >= 0 && p < n) order[p] = int32_t(uint32_t(t) | kind << 30);
     }
 }
 
-// Q in preorder: position i holds pre(parent(order[i])); two gathers and a coalesced write (a
-// scatter to pre(v) would cost a read-for-fill and a write-back per random sector). The root is
-// never inside a query range.
-constexpr int kGatherIlp = 4;  // positions per thread per step whose dependent gathers are in flight together
-
-__global__ void k_parent_pre(const int32_t *__restrict__ parent, const int32_t *__restrict__ pre,
-                             const int32_t *__restrict__ order, int32_t n, int32_t *__restrict__ q0) {
+// Q in preorder: position i holds pre(parent(order[i])). If the node before i has children, it is i's
+// parent: Q[i] = i - 1. If it is a leaf with a next sibling, i is that sibling: Q[i] = Q[i - 1]. Only after
+// a leaf that is a last child (the rest: 30% of a random tree's positions, none of a path's) parent[] and
+// pre[] have to be read at random places. A warp takes a block of 32 positions, kIlp blocks at a time, and
+// leaves the block's prefix / suffix minima and its result, too (table: x, (pm, sm) pairs, top row 0 of the
+// blocked layout; BLOCKED false: x only). tagged = order as k_node_stats left it, order = without tags.
+// 2^24 nodes: random TODO us, path TODO, with two gathers per position and a pass of its own for the
+// blocks 307 and 379.
+template <bool BLOCKED>
+__global__ void __launch_bounds__(256)
+    k_parent_pre(const int32_t *__restrict__ parent, const int32_t *__restrict__ pre,
+                 const int32_t *__restrict__ tagged, int32_t n, int64_t nblk, int32_t *__restrict__ order,
+                 int32_t *__restrict__ table) {
     pdl_prologue();
-    const int64_t step = gstride() * kGatherIlp;
-    for (int64_t base = blockIdx.x * int64_t(blockDim.x) * kGatherIlp + threadIdx.x; base < n; base += step) {
-        int32_t v[kGatherIlp], p[kGatherIlp];
+    constexpr int kIlp = 4;
+    const int64_t N = nblk * kRmqBlock, warps = gstride() / kWarp, warp = gtid() / kWarp;
+    const int lane = threadIdx.x & 31;
+    int32_t *top = table + 3 * N;
+    for (int64_t b0 = warp * kIlp; b0 < nblk; b0 += warps * kIlp) {
+        int32_t w[kIlp], before[kIlp], q[kIlp];
 #pragma unroll
-        for (int j = 0; j < kGatherIlp; ++j) {
-            const int64_t i = base + int64_t(j) * blockDim.x;
-            v[j] = i < n ? __ldcs(order + i) : -1;
+        for (int j = 0; j < kIlp; ++j) {
+            const int64_t i = (b0 + j) * kRmqBlock + lane;
+            w[j] = b0 + j < nblk && i < n ? __ldg(tagged + i) : -1;
+            before[j] = lane == 0 && b0 + j < nblk && i > 0 ? __ldg(tagged + i - 1) : -1;
         }
 #pragma unroll
-        for (int j = 0; j < kGatherIlp; ++j) p[j] = (v[j] >= 0 && v[j] < n) ? __ldg(parent + v[j]) : -1;
+        for (int j = 0; j < kIlp; ++j) {
+            const int32_t up = __shfl_up_sync(kFull, w[j], 1);
+            if (lane) before[j] = up;
+            uint32_t kind = uint32_t(before[j]) >> 30;  // 3: no node before
+            if (lane == 0 && kind == 1) kind = 2;       // the sibling's Q is another warp's
+            before[j] = int32_t(kind);
+            q[j] = -1;
+            const int64_t i = (b0 + j) * kRmqBlock + lane;
+            if (kind == 0) {
+                q[j] = int32_t(i - 1);
+            } else if (kind >= 2 && b0 + j < nblk && i < n) {
+                const int32_t v = w[j] & 0x3fffffff;
+                q[j] = v < n ? __ldg(parent + v) : -1;
+            }
+        }
 #pragma unroll
-        for (int j = 0; j < kGatherIlp; ++j) {
-            const int64_t i = base + int64_t(j) * blockDim.x;
-            if (i < n) __stcs(q0 + i, (p[j] >= 0 && p[j] < n) ? __ldg(pre + p[j]) : -1);
+        for (int j = 0; j < kIlp; ++j)
+            if (before[j] >= 2) q[j] = (q[j] >= 0 && q[j] < n) ? __ldg(pre + q[j]) : -1;  // a root's is never asked for
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j) {
+            if (b0 + j >= nblk) break;
+            const int64_t i = (b0 + j) * kRmqBlock + lane;
+            const unsigned known = __ballot_sync(kFull, before[j] != 1) & (lanemask_lt() | (1u << lane));
+            int32_t x = __shfl_sync(kFull, q[j], 31 - __clz(known));  // lane 0 is always known
+            if (i < n) {
+                __stcs(order + i, w[j] & 0x3fffffff);
+                __stcs(table + i, x);
+            } else if (BLOCKED) {
+                x = INT_MAX;
+                table[i] = x;
+            }
+            if (BLOCKED) {
+                int32_t a = x, c = x;
+#pragma unroll
+                for (int d = 1; d < kRmqBlock; d <<= 1) {
+                    const int32_t ua = __shfl_up_sync(kFull, a, d), dc = __shfl_down_sync(kFull, c, d);
+                    if (lane >= d) a = min(a, ua);
+                    if (lane + d < kRmqBlock) c = min(c, dc);
+                }
+                __stcs(reinterpret_cast<int2 *>(table + N) + i, make_int2(a, c));
+                if (lane == kRmqBlock - 1) top[b0 + j] = a;
+            }
         }
     }
 }
@@ -405,6 +460,7 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         const RankForm form = rank_form(2 * int64_t(n), true);
         void *list = form == RankForm::kSlots8 ? static_cast<void *>(ws.get<ulonglong2>(n)) : ws.get<int2>(n);  // 2n elements
         int32_t *head = ws.get<int32_t>(n), *next = ws.get<int32_t>(n);
+        int32_t *tagged = head;  // order[] with tags; the first children are not needed once the list is built
         int32_t *misc = ws.get<int32_t>(2 + 2 * int64_t(k));  // list head, offsets invalid, roots per tree, a root
         int32_t *root_cnt = misc + 2, *root_of = root_cnt + k;
         int32_t *inst_of = batch ? ws.get<int32_t>(n) : nullptr;
@@ -438,8 +494,8 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         if (!st) st = list_rank(list, 2 * int64_t(n), misc, 0, true, 2 * int64_t(n), h->status, ws, &rr);
         if (!st) {
             PhaseTimer pt("lca.node_stats", s);
-            launch(rr.wide ? k_node_stats<ulonglong2> : k_node_stats<uint2>, grid_for(n, 256), 256, 0, s, rr, n, h->pre, h->depth,
-                   h->size, h->order, h->status);
+            launch(rr.wide ? k_node_stats<ulonglong2> : k_node_stats<uint2>, grid_for(n, 256), 256, 0, s, rr, n,
+                   with_table ? next : nullptr, h->pre, h->depth, h->size, with_table ? tagged : h->order, h->status);
             note_launch();
             launch(k_check_instances, grid_for(k, 256), 256, 0, s, root_of, batch ? h->node_off : nullptr, k, n, h->pre,
                    h->size, h->status);
@@ -448,12 +504,13 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         }
         if (!st && with_table) {
             PhaseTimer pt("lca.parent_pre", s);
-            launch(k_parent_pre, grid_for(n, 256), 256, 0, s, par, h->pre, h->order, n, h->table);
+            launch(h->blocked ? k_parent_pre<true> : k_parent_pre<false>, grid_for(n, 256 * 4), 256, 0, s, par, h->pre,
+                   tagged, n, h->bl.nblk, h->order, h->table);
             note_launch();
             st = last_launch();
         }
         if (!st && with_table)
-            st = h->blocked ? blocked_build<OpMin>(h->table, n, h->bl, s, /*pairs=*/true)
+            st = h->blocked ? blocked_top<OpMin>(h->table + 3 * h->bl.nblk * kRmqBlock, h->bl, s)
                             : sparse_table_build<false>(h->table, n, h->levels, s);
         if (!st && with_table && h->blocked) {
             PhaseTimer pt("lca.node_rec", s);

@@ -16,7 +16,6 @@
 // 129 MB L2 for the sizes used here. Rows are padded to a multiple of four
 // entries with the identity.
 #include <climits>
-#include <type_traits>
 
 #include "etl_internal.cuh"
 
@@ -93,9 +92,8 @@ __device__ __forceinline__ int2 shfl_down(int2 v, int d) {
 }
 
 // one warp per block of 32 entries: prefix and suffix op by shuffles, block result -> top level 0;
-// entries in [n, nblk * 32) are set to the identity first. PAIRS (int32 entries only): pm and sm are
-// stored interleaved, (pm[i], sm[i]) as one 8-byte pair at position i of the 2N entries after x
-template <class Op, bool PAIRS>
+// entries in [n, nblk * 32) are set to the identity first
+template <class Op>
 __global__ void k_block_scan(typename Op::T *__restrict__ x, int64_t n, int64_t nblk, typename Op::T *__restrict__ pm,
                              typename Op::T *__restrict__ sm, typename Op::T *__restrict__ top0) {
     pdl_prologue();
@@ -118,12 +116,8 @@ __global__ void k_block_scan(typename Op::T *__restrict__ x, int64_t n, int64_t 
             if (lane >= d) p = Op::f(p, up);
             if (lane + d < kRmqBlock) q = Op::f(q, dn);
         }
-        if constexpr (PAIRS) {
-            reinterpret_cast<int2 *>(pm)[i] = make_int2(p, q);
-        } else {
-            pm[i] = p;
-            sm[i] = q;
-        }
+        pm[i] = p;
+        sm[i] = q;
         if (lane == kRmqBlock - 1) top0[b] = p;
     }
 }
@@ -222,26 +216,24 @@ BlockedLayout blocked_layout(int64_t n, int64_t max_len) {
 }
 
 template <class Op>
-etl_status blocked_build(typename Op::T *base, int64_t n, const BlockedLayout &L, cudaStream_t s, bool pairs) {
-    using T = typename Op::T;
+etl_status blocked_build(typename Op::T *base, int64_t n, const BlockedLayout &L, cudaStream_t s) {
     const int64_t N = L.nblk * kRmqBlock;
-    T *top = base + 3 * N;
-    const int grid_cap = num_sms() * 8;
+    typename Op::T *top = base + 3 * N;
     {
         PhaseTimer pt("rmq.blocks", s);
-        int blocks = int(ceil_div(N, 256));
-        if (blocks > grid_cap) blocks = grid_cap;
-        bool launched = false;
-        if constexpr (std::is_same<T, int32_t>::value) {
-            if (pairs) {
-                launch(k_block_scan<Op, true>, blocks, 256, 0, s, base, n, L.nblk, base + N, base + 2 * N, top);
-                launched = true;
-            }
-        }
-        if (!launched) launch(k_block_scan<Op, false>, blocks, 256, 0, s, base, n, L.nblk, base + N, base + 2 * N, top);
+        const int64_t blocks = ceil_div(N, 256), most = int64_t(num_sms()) * 8;
+        launch(k_block_scan<Op>, int(blocks < most ? blocks : most), 256, 0, s, base, n, L.nblk, base + N, base + 2 * N,
+               top);
         note_launch();
     }
-    etl_status st = last_launch();
+    const etl_status st = last_launch();
+    return st ? st : blocked_top<Op>(top, L, s);
+}
+
+template <class Op>
+etl_status blocked_top(typename Op::T *top, const BlockedLayout &L, cudaStream_t s) {
+    using T = typename Op::T;
+    etl_status st = ETL_OK;
     for (int l = 0; !st && l + 1 < L.tlevels;) {  // levels up to l are built
         const int most = l == 0 ? kLowLevels : kHighLevels;
         const int count = L.tlevels - 1 - l < most ? L.tlevels - 1 - l : most;
@@ -261,10 +253,9 @@ etl_status blocked_build(typename Op::T *base, int64_t n, const BlockedLayout &L
     return st;
 }
 
-template etl_status blocked_build<OpMin>(int32_t *, int64_t, const BlockedLayout &, cudaStream_t, bool);
-template etl_status blocked_build<OpMax>(int32_t *, int64_t, const BlockedLayout &, cudaStream_t, bool);
-template etl_status blocked_build<OpMinMax>(int2 *, int64_t, const BlockedLayout &, cudaStream_t, bool);
-template etl_status blocked_build<OpMinKey>(long long *, int64_t, const BlockedLayout &, cudaStream_t, bool);
+template etl_status blocked_top<OpMin>(int32_t *, const BlockedLayout &, cudaStream_t);
+template etl_status blocked_build<OpMinMax>(int2 *, int64_t, const BlockedLayout &, cudaStream_t);
+template etl_status blocked_build<OpMinKey>(long long *, int64_t, const BlockedLayout &, cudaStream_t);
 
 RmqParams &rmq_params() {
     static RmqParams p;
