@@ -269,7 +269,7 @@ etl_status find_bridges(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
  * not while calls are being enqueued from another thread.
  *   ETL_TUNE_RANK_K0_LOG2   level-0 density of the list ranker, k in [1, 8]
  *                           (default 5): lists ranked in place (longer than
- *                           L2 holds) start one walk per 2^(k+2) elements at
+ *                           L2 holds) start one walk per 2^(k+1) elements at
  *                           most; shorter ones (bound by the latency of their
  *                           longest sublist) take one splitter in 8 elements
  *                           up to 2^20, one in 16 beyond, or one in 2^k where
@@ -278,7 +278,8 @@ etl_status find_bridges(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
  *   ETL_TUNE_RANK_BLOCK     threads per block of the walk kernels, one of
  *                           64, 128, 256, 512, 1024 (128)
  *   ETL_TUNE_RANK_BLOCKS_PER_SM  resident walk blocks per SM on lists ranked
- *                           in place, block * value <= 2048 (10)
+ *                           in place, block * value <= 2048 (10; two thirds of
+ *                           it on those whose slots fit L2)
  *   ETL_TUNE_RMQ_LEVELS_PER_PASS sparse-table levels built per streaming
  *                           pass, 1..3 (3)
  *   ETL_TUNE_RMQ_BLOCK      threads per block of the sparse-table build,

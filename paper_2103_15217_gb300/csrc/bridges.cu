@@ -716,31 +716,33 @@ __global__ void k_check_batch(const int32_t *__restrict__ eoff, const int32_t *_
     }
 }
 
-__global__ void k_globalize(const int32_t *__restrict__ edges, int64_t m, const int32_t *__restrict__ eoff,
-                            const int32_t *__restrict__ noff, int32_t k, const int32_t *__restrict__ bad,
-                            int32_t *__restrict__ gedges, int32_t *__restrict__ status) {
+// A block takes kGlobalTile consecutive edges and looks up the instances of the first and the last, a
+// thread its edge's between the two (19M edges of 512 graphs: 124 us with a search over all instances per
+// edge, 67 now).
+constexpr int kGlobalTile = 2048;
+
+__global__ void __launch_bounds__(256)
+    k_globalize(const int32_t *__restrict__ edges, bool aligned, int64_t m, const int32_t *__restrict__ eoff,
+                const int32_t *__restrict__ noff, int32_t k, const int32_t *__restrict__ bad, int2 *__restrict__ gedges,
+                int32_t *__restrict__ status) {
     pdl_prologue();
+    __shared__ int32_t span[2];
     const bool unusable = *bad != 0;
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < m; e += int64_t(gridDim.x) * blockDim.x) {
-        int32_t gu = -1, gv = -1;
-        if (!unusable) {
-            int32_t lo = 0, hi = k;  // largest i with eoff[i] <= e (offsets checked monotone above)
-            while (lo < hi) {
-                const int32_t mid = (lo + hi + 1) >> 1;
-                if (__ldg(eoff + mid) <= e) lo = mid; else hi = mid - 1;
-            }
-            if (lo < k) {
-                const int32_t base = __ldg(noff + lo), size = __ldg(noff + lo + 1) - base;
-                const int32_t a = edges[2 * e], b = edges[2 * e + 1];
-                if (a >= 0 && a < size && b >= 0 && b < size) {
-                    gu = a + base;
-                    gv = b + base;
-                }
-            }
-            if (gu < 0) set_status(status, ETL_EBADGRAPH);
+    const int64_t base = int64_t(blockIdx.x) * kGlobalTile, end = min(base + kGlobalTile, m);
+    if (threadIdx.x < 2 && !unusable) span[threadIdx.x] = last_at_or_before(eoff, 0, k - 1, threadIdx.x == 0 ? base : end - 1);
+    __syncthreads();
+    for (int64_t e = base + threadIdx.x; e < end; e += blockDim.x) {
+        int2 g = make_int2(-1, -1);
+        if (!unusable) {  // offsets are monotone, from 0 to m: checked before
+            const int32_t i = last_at_or_before(eoff, span[0], span[1], e);
+            const int32_t from = __ldg(noff + i), size = __ldg(noff + i + 1) - from;
+            const int2 ab = load_edge(edges, e, aligned);
+            if (ab.x >= 0 && ab.x < size && ab.y >= 0 && ab.y < size)
+                g = make_int2(ab.x + from, ab.y + from);
+            else
+                set_status(status, ETL_EBADGRAPH);
         }
-        gedges[2 * e] = gu;
-        gedges[2 * e + 1] = gv;
+        gedges[e] = g;
     }
 }
 
@@ -782,7 +784,8 @@ extern "C" etl_status find_bridges_batch(const int32_t *edges, const int32_t *ed
         PhaseTimer pt("br.globalize", s);
         launch(k_check_batch, grid_for(k, 256), 256, 0, s, edge_off, node_off, k, total_m, total_n, bad, st);
         note_launch();
-        launch(k_globalize, grid_for(total_m, 256), 256, 0, s, edges, total_m, edge_off, node_off, k, bad, gedges, st);
+        launch(k_globalize, unsigned(ceil_div(total_m, kGlobalTile)), 256, 0, s, edges, edges_aligned(edges), total_m,
+               edge_off, node_off, k, bad, reinterpret_cast<int2 *>(gedges), st);
         note_launch();
     }
     etl_status rc = last_launch();

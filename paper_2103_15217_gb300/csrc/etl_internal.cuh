@@ -188,6 +188,16 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
+// largest i in [lo, hi] with off[i] <= x (off ascending, off[lo] <= x)
+__device__ __forceinline__ int32_t last_at_or_before(const int32_t *__restrict__ off, int32_t lo, int32_t hi, int64_t x) {
+    while (lo < hi) {
+        const int32_t mid = lo + ((hi - lo + 1) >> 1);
+        if (__ldg(off + mid) <= x) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
 // ----------------------------------------------------------------- primitives
 
 // Exclusive scan of in[0..n) into out[0..n], out[n] = total. If d_n is not
@@ -197,11 +207,10 @@ etl_status scan_exclusive_u8(const uint8_t *in, int32_t *out, int64_t n, Workspa
 
 // Children of every node in ascending label order: head[v] = first child or -1, next[c] = next sibling
 // or -1 (-1 for roots too). parent: ids in [0, n), -1 at roots; anything else is dropped and sets the
-// status. For a batch, off / inst_of / bad say which instance a node belongs to (*bad: drop all), ids
-// are local to it, and gparent receives the global ones (-1 at roots, -2: dropped). root_cnt / root_of
-// (zeroed by the caller): roots per instance and the last one seen.
-etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, const int32_t *inst_of,
-                         const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
+// status. For a batch of k instances, off (k + 1 offsets; *bad: unusable, drop all nodes) says which one a
+// node belongs to, ids are local to it, and gparent receives the global ones (-1 at roots, -2: dropped).
+// root_cnt / root_of (zeroed by the caller): roots per instance and the last one seen.
+etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, int32_t k, const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
                          int32_t *root_of, int32_t *status, Workspace &ws);
 
 // ----------------------------------------------------------------- list ranking

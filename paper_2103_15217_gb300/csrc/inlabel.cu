@@ -70,10 +70,11 @@ __global__ void k_inlabel_heads(const int32_t *__restrict__ parent, const int32_
         const bool head = p < 0 || p >= n || inl[p] != iv;
         const int64_t open = 2 * int64_t(pre[v]) - depth[v], close = open + 2 * int64_t(size[v]) - 1;
         if (open < 0 || close >= 2 * int64_t(n) || open >= close) continue;
-        const int32_t w = head ? int32_t(lowbit(iv)) : 0;
+        if (!head) continue;  // the tour's values are zero elsewhere
+        const int32_t w = int32_t(lowbit(iv));
         tourval[open] = w;
         tourval[close] = -w;
-        if (head && iv <= uint32_t(n)) pathrec[iv] = (p >= 0 && p < n) ? make_int2(p, depth[p]) : make_int2(-1, -1);
+        if (iv <= uint32_t(n)) pathrec[iv] = (p >= 0 && p < n) ? make_int2(p, depth[p]) : make_int2(-1, -1);
     }
 }
 
@@ -176,6 +177,7 @@ etl_status lca_build_inlabel_impl(etl_lca_t h, const int32_t *parent, cudaStream
     int32_t *excl = ws.get<int32_t>(2 * int64_t(n) + 1);
     if (!ws.ok()) return ETL_ENOMEM;
     const int g = grid_for(n, 256);
+    memset_async(tourval, 0, size_t(2) * n * sizeof(int32_t), s);
     {
         PhaseTimer pt("inlabel.build", s);
         launch(k_inlabel, g, 256, 0, s, h->pre, h->size, n, inl);

@@ -54,17 +54,6 @@ __global__ void k_check_offsets(const int32_t *__restrict__ off, int32_t k, int3
     }
 }
 
-// inst_of[v] = instance of node v; one block per instance, coalesced writes
-__global__ void k_fill_inst(const int32_t *__restrict__ off, int32_t k, const int32_t *__restrict__ bad,
-                            int32_t *__restrict__ inst_of) {
-    pdl_prologue();
-    if (*bad) return;
-    for (int64_t i = blockIdx.x; i < k; i += gridDim.x) {
-        const int32_t b = off[i], e = off[i + 1];
-        for (int32_t v = b + threadIdx.x; v < e; v += blockDim.x) inst_of[v] = int32_t(i);
-    }
-}
-
 // One store per node. A leaf v's brackets are adjacent in the tour: 2v jumps straight to the successor of
 // 2v+1 with weight 2 (top bit set), and 2v+1 is off the list. Roots are never contracted. All accesses
 // are coalesced (the closing brackets' successors were scattered to random places before, which made
@@ -171,7 +160,7 @@ __global__ void k_node_stats(RankResult rr, int32_t n, const int32_t *__restrict
 // pre[] have to be read at random places. A warp takes a block of 32 positions, kIlp blocks at a time, and
 // leaves the block's prefix / suffix minima and its result, too (table: x, (pm, sm) pairs, top row 0 of the
 // blocked layout; BLOCKED false: x only). tagged = order as k_node_stats left it, order = without tags.
-// 2^24 nodes: random TODO us, path TODO, with two gathers per position and a pass of its own for the
+// 2^24 nodes: random 153 us, path 72, with two gathers per position and a pass of its own for the
 // blocks 307 and 379.
 template <bool BLOCKED>
 __global__ void __launch_bounds__(256)
@@ -463,7 +452,6 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         int32_t *tagged = head;  // order[] with tags; the first children are not needed once the list is built
         int32_t *misc = ws.get<int32_t>(2 + 2 * int64_t(k));  // list head, offsets invalid, roots per tree, a root
         int32_t *root_cnt = misc + 2, *root_of = root_cnt + k;
-        int32_t *inst_of = batch ? ws.get<int32_t>(n) : nullptr;
         int32_t *gparent = batch ? ws.get<int32_t>(n) : nullptr;
         if (!ws.ok()) st = ETL_ENOMEM;
         const int32_t *par = batch ? gparent : parent;
@@ -473,10 +461,8 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
                 PhaseTimer pt("lca.inst", s);
                 launch(k_check_offsets, grid_for(k, 256), 256, 0, s, h->node_off, k, n, misc + 1, h->status);
                 note_launch();
-                launch(k_fill_inst, k < 8192 ? k : 8192, 256, 0, s, h->node_off, k, misc + 1, inst_of);
-                note_launch();
             }
-            st = link_children(parent, n, h->node_off, inst_of, misc + 1, gparent, head, next, root_cnt, root_of,
+            st = link_children(parent, n, h->node_off, k, misc + 1, gparent, head, next, root_cnt, root_of,
                                h->status, ws);
         }
         if (!st) {

@@ -452,10 +452,13 @@ RankParams &rank_params() {
     return p;
 }
 
-// Successors and records (8 bytes per element, 12 in dual mode) of up to 96 of the 129 MB L2 are kept in
-// separate arrays; longer lists are ranked in place, in 4-byte slots where the records fit them.
+// Shorter lists keep successors and records in separate arrays, longer ones are ranked in place, in 4-byte
+// slots where the records fit them. Tours of random trees, whole ranking: 2^21 brackets 139 us apart, 139
+// in place, 2^22 183 and 182, 2^23 250 and 226. Other lists: 2^22 elements 173 and 182, 2^23 251 and 233,
+// but a caller's list has to be copied into the slots first, so the line lies where successors and records
+// (8 bytes per element) exceed 96 of the 129 MB of L2.
 RankForm rank_form(int64_t len, bool dual) {
-    if (len * (dual ? 12 : 8) <= (int64_t(96) << 20)) return RankForm::kSeparate;
+    if (dual ? len <= (int64_t(1) << 22) : len * 8 <= (int64_t(96) << 20)) return RankForm::kSeparate;
     if (dual) return len <= (int64_t(1) << 26) ? RankForm::kSlots4 : RankForm::kSlots8;
     return wide_slots(len) ? RankForm::kSlots8 : RankForm::kSlots4;
 }
@@ -520,8 +523,10 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         w.len = len;
         w.d_head = d_head;
         w.head = head;
-        const int64_t per_lane = int64_t(4) << P.k0_log2;
-        const int grid = grid_of(len / per_lane, P.blocks_per_sm, P);
+        const int64_t per_lane = int64_t(2) << P.k0_log2;
+        // two thirds of the walkers where the slots fit L2: 2^24 random brackets 304 us, 320 with all of them
+        const bool fits = len * int64_t(sizeof(R)) <= (int64_t(96) << 20);
+        const int grid = grid_of(len / per_lane, fits ? std::max(1, P.blocks_per_sm * 2 / 3) : P.blocks_per_sm, P);
         const int64_t lanes = int64_t(grid) * P.block;
         w.nclaims = uint32_t(std::min(16 * lanes, len / 3) + 1);
         w.start = int32_t(lanes / kWarp * SidPool::kFirst);

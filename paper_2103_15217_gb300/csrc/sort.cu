@@ -27,16 +27,24 @@ constexpr int kLinkThreads = 256;
 constexpr int kLinkIlp = 2;  // labels per thread, from the highest down (1: 0.16 ms, 4: more siblings in flight together)
 constexpr int kLight = 32;   // children of a family that one thread sorts
 
-// off / inst_of / bad (batches): ids are local to the node's instance, gparent receives global ones
+// off / k / bad (batches): ids are local to the node's instance, gparent receives global ones. A block
+// looks up the instances of its first and last label, a thread its own between the two.
 template <bool BATCH>
 __global__ void __launch_bounds__(kLinkThreads)
     k_link_children(const int32_t *__restrict__ parent, int32_t n, const int32_t *__restrict__ off,
-                    const int32_t *__restrict__ inst_of, const int32_t *__restrict__ bad,
-                    int32_t *__restrict__ gparent, int32_t *__restrict__ head, int32_t *__restrict__ next,
-                    int32_t *__restrict__ root_cnt, int32_t *__restrict__ root_of, int32_t *__restrict__ status) {
+                    int32_t k, const int32_t *__restrict__ bad, int32_t *__restrict__ gparent, int32_t *__restrict__ head,
+                    int32_t *__restrict__ next, int32_t *__restrict__ root_cnt, int32_t *__restrict__ root_of,
+                    int32_t *__restrict__ status) {
     pdl_prologue();
     const bool bad_offsets = BATCH && *bad;
     const int64_t top = int64_t(gridDim.x - blockIdx.x) * (kLinkThreads * kLinkIlp);
+    __shared__ int32_t span[2];
+    if (BATCH) {
+        if (threadIdx.x < 2 && !bad_offsets)
+            span[threadIdx.x] = last_at_or_before(
+                off, 0, k - 1, threadIdx.x == 0 ? top - kLinkThreads * kLinkIlp : min(top, int64_t(n)) - 1);
+        __syncthreads();
+    }
     int32_t par[kLinkIlp];
 #pragma unroll
     for (int j = 0; j < kLinkIlp; ++j) {
@@ -51,7 +59,7 @@ __global__ void __launch_bounds__(kLinkThreads)
         if (t < n && !bad_offsets) {
             int32_t inst = 0, base = 0, size = n;
             if (BATCH) {
-                inst = inst_of[v];
+                inst = last_at_or_before(off, span[0], span[1], v);
                 base = off[inst];
                 size = off[inst + 1] - base;
             }
@@ -379,8 +387,7 @@ SortParams &sort_params() {
     return p;
 }
 
-etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, const int32_t *inst_of,
-                         const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
+etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, int32_t k, const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
                          int32_t *root_of, int32_t *status, Workspace &ws) {
     cudaStream_t s = ws.stream();
     const int64_t mask_words = ceil_div(n, 32);
@@ -394,7 +401,7 @@ etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, c
     {
         PhaseTimer pt("lca.link", s);
         const int blocks = int(ceil_div(n, kLinkThreads * kLinkIlp));
-        launch(off ? k_link_children<true> : k_link_children<false>, blocks, kLinkThreads, 0, s, parent, n, off, inst_of,
+        launch(off ? k_link_children<true> : k_link_children<false>, blocks, kLinkThreads, 0, s, parent, n, off, k,
                bad, gparent, head, next, root_cnt, root_of, status);
         note_launch();
     }

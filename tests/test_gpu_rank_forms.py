@@ -1,7 +1,6 @@
 """The list ranker's forms at the sizes where one gives way to the next: one CTA (up to 15360
-elements), separate records with one and with two upper levels, records in place (beyond 96 MB of
-successors and records: 12,582,912 elements, 2^22 tree nodes), for trees in 4-byte slots up to 2^25
-nodes. A list built from a permutation has rank[perm[i]] = i, so the results are compared exactly."""
+elements), separate records with one and with two upper levels, records in place (beyond 12,582,912
+elements, 2^21 tree nodes), for trees in 4-byte slots up to 2^25 nodes. A list built from a permutation has rank[perm[i]] = i, so the results are compared exactly."""
 
 import ctypes
 
@@ -67,7 +66,7 @@ def test_malformed_lists_end_with_a_status(n, fault):
     assert int(st) != 0
 
 
-@pytest.mark.parametrize("n,grasp", [(n, g) for n in (TOP // 2, TOP // 2 + 1, (1 << 20) + 3, 1 << 22, (1 << 22) + 1)
+@pytest.mark.parametrize("n,grasp", [(n, g) for n in (TOP // 2, TOP // 2 + 1, (1 << 20) + 3, 1 << 21, (1 << 21) + 1, (1 << 22) + 1)
                                      for g in (1, 3, 1024)] + [((1 << 25) + 1, 3)])
 def test_trees(n, grasp):
     # the tour of a tree by the grasp model: depth, size and preorder from the definition
