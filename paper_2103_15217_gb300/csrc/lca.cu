@@ -130,27 +130,45 @@ __global__ void k_node_stats(RankResult rr, int32_t n, const int32_t *__restrict
                              int32_t *__restrict__ status) {
     pdl_prologue();
     const Q *recs = static_cast<const Q *>(rr.recs);
-    for (int64_t t = gtid(); t < n; t += gstride()) {
-        const NodeRecs r = node_recs(__ldcs(recs + t));
-        if (!r.ok || r.sa < 0 || r.sa >= rr.rcap || r.sb < 0 || r.sb >= rr.rcap) {
-            set_status(status, ETL_EBADTREE);  // not on the list from the root: malformed input
-            pre[t] = depth[t] = size[t] = -1;
-            continue;
+    constexpr int kIlp = 2;  // nodes per thread and step, their gathers in flight together (2^24 nodes: 268 us; one 275, four 312)
+    for (int64_t base = blockIdx.x * int64_t(blockDim.x) * kIlp + threadIdx.x; base < n; base += gstride() * kIlp) {
+        NodeRecs r[kIlp];
+        int2 A[kIlp];
+        int32_t rb[kIlp];
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j) {
+            const int64_t t = base + int64_t(j) * blockDim.x;
+            r[j].ok = false;
+            if (t < n) r[j] = node_recs(__ldcs(recs + t));
+            r[j].ok = r[j].ok && r[j].sa >= 0 && r[j].sa < rr.rcap && r[j].sb >= 0 && r[j].sb < rr.rcap;
         }
-        const int2 A = __ldg(reinterpret_cast<const int2 *>(rr.T + r.sa));
-        const int32_t r0 = A.x + r.ra;
-        const int32_t r1 = r.leaf ? r0 + 1 : __ldg(&rr.T[r.sb].x) + r.rb;
-        const int32_t p = A.y + r.oa;
-        __stcs(pre + t, p);
-        __stcs(depth + t, 2 * p - r0);
-        const int32_t sz = (r1 - r0 + 1) >> 1;
-        __stcs(size + t, sz);
-        uint32_t kind = 0;
-        if (next) {
-            const int32_t x = __ldcs(next + t);
-            kind = sz > 1 ? 0u : x >= 0 ? 1u : 2u;
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j)
+            if (r[j].ok) {
+                A[j] = __ldg(reinterpret_cast<const int2 *>(rr.T + r[j].sa));
+                rb[j] = r[j].leaf ? 0 : __ldg(&rr.T[r[j].sb].x);
+            }
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j) {
+            const int64_t t = base + int64_t(j) * blockDim.x;
+            if (t >= n) continue;
+            if (!r[j].ok) {
+                set_status(status, ETL_EBADTREE);  // not on the list from the root: malformed input
+                pre[t] = depth[t] = size[t] = -1;
+                continue;
+            }
+            const int32_t r0 = A[j].x + r[j].ra, r1 = r[j].leaf ? r0 + 1 : rb[j] + r[j].rb;
+            const int32_t p = A[j].y + r[j].oa, sz = (r1 - r0 + 1) >> 1;
+            __stcs(pre + t, p);
+            __stcs(depth + t, 2 * p - r0);
+            __stcs(size + t, sz);
+            uint32_t kind = 0;
+            if (next) {
+                const int32_t x = __ldcs(next + t);
+                kind = sz > 1 ? 0u : x >= 0 ? 1u : 2u;
+            }
+            if (p >= 0 && p < n) order[p] = int32_t(uint32_t(t) | kind << 30);
         }
-        if (p >= 0 && p < n) order[p] = int32_t(uint32_t(t) | kind << 30);
     }
 }
 
