@@ -123,14 +123,14 @@ __device__ __forceinline__ NodeRecs node_recs(uint2 q) {
 }
 
 // next (null: plain node ids): order[] entries carry what k_parent_pre needs to know of the node in their
-// top bits, 0: it has children, 1: a leaf with a next sibling, 2: a leaf without
-template <class Q>
+// top bits, 0: it has children, 1: a leaf with a next sibling, 2: a leaf without. kIlp nodes per thread and
+// step (2^24 nodes: two 268 us, one 275, four 312).
+template <class Q, int kIlp>
 __global__ void k_node_stats(RankResult rr, int32_t n, const int32_t *__restrict__ next, int32_t *__restrict__ pre,
                              int32_t *__restrict__ depth, int32_t *__restrict__ size, int32_t *__restrict__ order,
                              int32_t *__restrict__ status) {
     pdl_prologue();
     const Q *recs = static_cast<const Q *>(rr.recs);
-    constexpr int kIlp = 2;  // nodes per thread and step, their gathers in flight together (2^24 nodes: 268 us; one 275, four 312)
     for (int64_t base = blockIdx.x * int64_t(blockDim.x) * kIlp + threadIdx.x; base < n; base += gstride() * kIlp) {
         NodeRecs r[kIlp];
         int2 A[kIlp];
@@ -172,6 +172,8 @@ __global__ void k_node_stats(RankResult rr, int32_t n, const int32_t *__restrict
     }
 }
 
+constexpr int32_t kFewNodes = 1 << 21;
+
 // Q in preorder: position i holds pre(parent(order[i])). If the node before i has children, it is i's
 // parent: Q[i] = i - 1. If it is a leaf with a next sibling, i is that sibling: Q[i] = Q[i - 1]. Only after
 // a leaf that is a last child (the rest: 30% of a random tree's positions, none of a path's) parent[] and
@@ -180,13 +182,12 @@ __global__ void k_node_stats(RankResult rr, int32_t n, const int32_t *__restrict
 // blocked layout; BLOCKED false: x only). tagged = order as k_node_stats left it, order = without tags.
 // 2^24 nodes: random 153 us, path 72, with two gathers per position and a pass of its own for the
 // blocks 307 and 379.
-template <bool BLOCKED>
+template <bool BLOCKED, int kIlp>
 __global__ void __launch_bounds__(256)
     k_parent_pre(const int32_t *__restrict__ parent, const int32_t *__restrict__ pre,
                  const int32_t *__restrict__ tagged, int32_t n, int64_t nblk, int32_t *__restrict__ order,
                  int32_t *__restrict__ table) {
     pdl_prologue();
-    constexpr int kIlp = 4;
     const int64_t N = nblk * kRmqBlock, warps = gstride() / kWarp, warp = gtid() / kWarp;
     const int lane = threadIdx.x & 31;
     int32_t *top = table + 3 * N;
@@ -270,10 +271,10 @@ struct LcaView {
 // from w's side, pm[p] (w has the larger preorder number) and sm[p] (the smaller one), with p and
 // size(w), so that a query reads two 16-byte records instead of pre[] twice, then pm and sm. The
 // table stores (pm, sm) pairs, so this is one 8-byte gather per node.
+template <int kIlp>  // nodes per thread per step, their gathers in flight together
 __global__ void k_node_rec(const int32_t *__restrict__ pre, const int32_t *__restrict__ size,
                            const int2 *__restrict__ pmsm, int32_t n, int4 *__restrict__ nrec) {
     pdl_prologue();
-    constexpr int kIlp = 4;  // nodes per thread per step, their gathers in flight together
     const int64_t step = gstride() * kIlp;
     for (int64_t base = blockIdx.x * int64_t(blockDim.x) * kIlp + threadIdx.x; base < n; base += step) {
         int32_t p[kIlp];
@@ -292,7 +293,11 @@ __global__ void k_node_rec(const int32_t *__restrict__ pre, const int32_t *__res
     }
 }
 
+// Queries per thread and step. Up to kQueryFew the memory behind them fits L2 or they are too few to fill
+// the GPU four to a thread: 2^20 queries of a 2^22-node tree 22.1 us with four, 19.1 with one, 2^14 5.4 and
+// 2.5; 2^22 69 and 69; 2^24 queries of a 2^24-node tree, bound by DRAM, 564 and 583.
 constexpr int kQueryIlp = 4;
+constexpr int64_t kQueryFew = int64_t(1) << 22;
 
 // min of x[lo..hi], a range inside one block of the blocked table (at most 32 entries, one line)
 __device__ __forceinline__ int32_t inblock_min(const int32_t *__restrict__ x, int32_t lo, int32_t hi) {
@@ -301,21 +306,21 @@ __device__ __forceinline__ int32_t inblock_min(const int32_t *__restrict__ x, in
     return m;
 }
 
-// Each thread answers kQueryIlp queries at once so that their dependent
-// gathers (pre, table, order) overlap in flight. BATCH: ids are local to the
+// Each thread answers ILP queries at once so that their dependent gathers
+// (pre, table, order) overlap in flight. BATCH: ids are local to the
 // instance inst[i] and so is the answer.
-template <bool BATCH, bool BLOCKED>
+template <bool BATCH, bool BLOCKED, int ILP>
 __global__ void __launch_bounds__(256)
     k_lca_query(LcaView h, const int32_t *__restrict__ inst, const int32_t *__restrict__ u,
                 const int32_t *__restrict__ v, int64_t q, int32_t *__restrict__ out, int32_t *__restrict__ status) {
     pdl_prologue();
     const bool bad_tree = *h.hstatus != 0;
     const int64_t stride = gstride();
-    for (int64_t base = gtid(); base < q; base += stride * kQueryIlp) {
-        int32_t a[kQueryIlp], b[kQueryIlp], lo[kQueryIlp], hi[kQueryIlp], res[kQueryIlp], ofs[kQueryIlp];
-        bool need[kQueryIlp], ok[kQueryIlp];
+    for (int64_t base = gtid(); base < q; base += stride * ILP) {
+        int32_t a[ILP], b[ILP], lo[ILP], hi[ILP], res[ILP], ofs[ILP];
+        bool need[ILP], ok[ILP];
 #pragma unroll
-        for (int k = 0; k < kQueryIlp; ++k) {
+        for (int k = 0; k < ILP; ++k) {
             const int64_t i = base + k * stride;
             need[k] = false;
             ok[k] = false;
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(256)
             }
         }
 #pragma unroll
-        for (int k = 0; k < kQueryIlp; ++k) {
+        for (int k = 0; k < ILP; ++k) {
             if (!ok[k] || bad_tree) continue;
             if (a[k] == b[k]) {
                 res[k] = a[k];
@@ -379,11 +384,11 @@ __global__ void __launch_bounds__(256)
             }
         }
 #pragma unroll
-        for (int k = 0; k < kQueryIlp; ++k)
+        for (int k = 0; k < ILP; ++k)
             if (need[k] && hi[k] >= 0)  // in one block (blocked table), or the full table
                 lo[k] = BLOCKED ? inblock_min(h.bv.x, lo[k], hi[k]) : sparse_query<false>(h.table, h.ld, lo[k], hi[k]);
 #pragma unroll
-        for (int k = 0; k < kQueryIlp; ++k) {
+        for (int k = 0; k < ILP; ++k) {
             const int64_t i = base + k * stride;
             if (i >= q) continue;
             if (need[k]) res[k] = __ldg(h.order + lo[k]) - ofs[k];
@@ -465,6 +470,7 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
     {
         Workspace ws(s);
         const RankForm form = rank_form(2 * int64_t(n), true);
+        const bool few = n <= kFewNodes;  // one node per thread and step fills the GPU better
         void *list = form == RankForm::kSlots8 ? static_cast<void *>(ws.get<ulonglong2>(n)) : ws.get<int2>(n);  // 2n elements
         int32_t *head = ws.get<int32_t>(n), *next = ws.get<int32_t>(n);
         int32_t *tagged = head;  // order[] with tags; the first children are not needed once the list is built
@@ -498,7 +504,8 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         if (!st) st = list_rank(list, 2 * int64_t(n), misc, 0, true, 2 * int64_t(n), h->status, ws, &rr);
         if (!st) {
             PhaseTimer pt("lca.node_stats", s);
-            launch(rr.wide ? k_node_stats<ulonglong2> : k_node_stats<uint2>, grid_for(n, 256), 256, 0, s, rr, n,
+            launch(rr.wide ? (few ? k_node_stats<ulonglong2, 1> : k_node_stats<ulonglong2, 2>) : k_node_stats<uint2, 2>,
+                   grid_for(n, 256), 256, 0, s, rr, n,
                    with_table ? next : nullptr, h->pre, h->depth, h->size, with_table ? tagged : h->order, h->status);
             note_launch();
             launch(k_check_instances, grid_for(k, 256), 256, 0, s, root_of, batch ? h->node_off : nullptr, k, n, h->pre,
@@ -508,8 +515,8 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         }
         if (!st && with_table) {
             PhaseTimer pt("lca.parent_pre", s);
-            launch(h->blocked ? k_parent_pre<true> : k_parent_pre<false>, grid_for(n, 256 * 4), 256, 0, s, par, h->pre,
-                   tagged, n, h->bl.nblk, h->order, h->table);
+            launch(h->blocked ? (few ? k_parent_pre<true, 1> : k_parent_pre<true, 4>) : k_parent_pre<false, 4>,
+                   grid_for(n, few ? 256 : 256 * 4), 256, 0, s, par, h->pre, tagged, n, h->bl.nblk, h->order, h->table);
             note_launch();
             st = last_launch();
         }
@@ -518,7 +525,7 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
                             : sparse_table_build<false>(h->table, n, h->levels, s);
         if (!st && with_table && h->blocked) {
             PhaseTimer pt("lca.node_rec", s);
-            launch(k_node_rec, grid_for(n, 256), 256, 0, s, h->pre, h->size,
+            launch(few ? k_node_rec<1> : k_node_rec<4>, grid_for(n, 256), 256, 0, s, h->pre, h->size,
                    reinterpret_cast<const int2 *>(h->table + h->bl.nblk * kRmqBlock), n, static_cast<int4 *>(h->nrec));
             note_launch();
             st = last_launch();
@@ -540,18 +547,13 @@ etl_status query_launch(etl_lca_t h, const int32_t *inst, const int32_t *u, cons
                  h->blocked ? blocked_max_len(h->bl) : (int64_t(1) << h->levels) - 1,
                  static_cast<const int4 *>(h->nrec)};
     PhaseTimer pt("lca.query", s);
-    const int grid = grid_for(ceil_div(q, kQueryIlp), 256);
-    if (h->blocked) {
-        if (inst)
-            launch(k_lca_query<true, true>, grid, 256, 0, s, view, inst, u, v, q, out, status);
-        else
-            launch(k_lca_query<false, true>, grid, 256, 0, s, view, nullptr, u, v, q, out, status);
-    } else {
-        if (inst)
-            launch(k_lca_query<true, false>, grid, 256, 0, s, view, inst, u, v, q, out, status);
-        else
-            launch(k_lca_query<false, false>, grid, 256, 0, s, view, nullptr, u, v, q, out, status);
-    }
+    const bool few = q <= kQueryFew;
+    const int grid = grid_for(few ? q : ceil_div(q, kQueryIlp), 256);
+    auto kernel = h->blocked ? (inst ? (few ? k_lca_query<true, true, 1> : k_lca_query<true, true, kQueryIlp>)
+                                     : (few ? k_lca_query<false, true, 1> : k_lca_query<false, true, kQueryIlp>))
+                             : (inst ? (few ? k_lca_query<true, false, 1> : k_lca_query<true, false, kQueryIlp>)
+                                     : (few ? k_lca_query<false, false, 1> : k_lca_query<false, false, kQueryIlp>));
+    launch(kernel, grid, 256, 0, s, view, inst, u, v, q, out, status);
     note_launch();
     return last_launch();
 }
