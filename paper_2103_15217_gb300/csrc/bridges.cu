@@ -38,13 +38,14 @@ namespace {
 
 constexpr int64_t kFindCap = int64_t(1) << 26;  // bound on pointer-chasing steps of one edge
 
-// forest: [0] edges found, [1] first half-edge of the component list (the ranked list's head)
+// forest: [0] edges found, [1] first half-edge of the component list (the ranked list's head), [2] zero
 __global__ void k_init(int32_t n, int32_t *__restrict__ par, int32_t *__restrict__ head, int32_t *__restrict__ tin,
                        int32_t *__restrict__ forest) {
     pdl_prologue();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         forest[0] = 0;
         forest[1] = ETL_END;
+        forest[2] = 0;
     }
     for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n; v += int64_t(gridDim.x) * blockDim.x) {
         par[v] = int32_t(v);
@@ -130,11 +131,11 @@ __device__ __forceinline__ bool hook_above(int32_t a, int32_t b, int32_t giant) 
 // over 1 us); the two loads per edge of its 31.4M later edges alone take 210 us. Batch of 512 graphs: 1430
 // -> 580 us. Graphs of up to kHookAtOnce edges skip the first slice: 2^14 vertices, 2^16 edges 65 -> 50 us.
 // skip (may be null): edges to leave out; is_tree (may be null): 1 for edges whose hook succeeded, and
-// then forest_count, tuv (both ends of forest edge t) and tedge (its edge) are written too
+// then is_bridge is cleared and forest_count, tuv (both ends of forest edge t) and tedge (its edge) are written too
 __global__ void __launch_bounds__(kHookChunk)
     k_hook(const int32_t *__restrict__ edges, bool aligned, int64_t m, int64_t c0, int64_t c1, int ilp, bool spread,
-           int32_t n, int32_t *__restrict__ par, uint8_t *__restrict__ is_tree, const uint8_t *__restrict__ skip,
-           const int32_t *__restrict__ d_giant, int32_t *__restrict__ forest_count, int2 *__restrict__ tuv,
+           int32_t n, int32_t *__restrict__ par, uint8_t *__restrict__ is_tree, uint8_t *__restrict__ is_bridge,
+           const uint8_t *__restrict__ skip, const int32_t *__restrict__ d_giant, int32_t *__restrict__ forest_count, int2 *__restrict__ tuv,
            int32_t *__restrict__ tedge, int32_t *__restrict__ status) {
     pdl_prologue();
     __shared__ int32_t qa[kHookChunk * (kHookIlp + 1)], qb[kHookChunk * (kHookIlp + 1)], qe[kHookChunk * (kHookIlp + 1)];
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(kHookChunk)
 #pragma unroll
         for (int j = 0; j < kHookIlp; ++j) {
             if (!ok[j]) continue;
-            if (is_tree) is_tree[e[j]] = 0;
+            if (is_tree) is_tree[e[j]] = is_bridge[e[j]] = 0;
             if (skip && skip[e[j]]) {
                 ok[j] = false;
             } else if (ab[j].x < 0 || ab[j].x >= n || ab[j].y < 0 || ab[j].y >= n) {
@@ -593,7 +594,7 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
     int2 *tuv = ws.get<int2>(n);
     int32_t *arcs = reinterpret_cast<int32_t *>(tuv), *next = ws.get<int32_t>(N + 1);  // tail of / half-edge after each
     int32_t *tedge = ws.get<int32_t>(n);
-    int32_t *forest = ws.get<int32_t>(2), *giant = ws.get<int32_t>(1);
+    int32_t *forest = ws.get<int32_t>(3), *giant = ws.get<int32_t>(1);
     const bool wide = wide_slots(N);
     void *list = wide ? static_cast<void *>(ws.get<Slot8::T>(N)) : static_cast<void *>(ws.get<Slot4::T>(N));  // slots or successors
     int32_t *child = hybrid ? ws.get<int32_t>(n) : nullptr;
@@ -604,7 +605,6 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
     if (!ws.ok()) return ETL_ENOMEM;
     etl_status rc = ETL_OK;
     const int gn = grid_for(n, 256), gm = grid_for(m, 256), gA = grid_for(N, 256);
-    memset_async(is_bridge, 0, size_t(m), s);
     {
         PhaseTimer pt("br.init", s);
         launch(k_init, gn, 256, 0, s, n, par, head, tin, forest);
@@ -631,7 +631,8 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
                 }
             }
             launch(k_hook, hook_grid(c1 - c0), kHookChunk, 0, s, edges, aligned, m, c0, c1,
-                   hook_ilp(c1 - c0), spread, n, par, is_tree, nullptr, (c0 > 0 && C.giant) ? giant : nullptr, forest, tuv, tedge, st);
+                   hook_ilp(c1 - c0), spread, n, par, is_tree, is_bridge, nullptr, (c0 > 0 && C.giant) ? giant : nullptr, forest,
+                   tuv, tedge, st);
             note_launch();
             c0 = c1;
             w *= 2;
@@ -650,7 +651,7 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
         rc = last_launch();
     }
     RankResult rr{};
-    if (!rc) rc = list_rank(list, N, forest + 1, 0, false, -1, st, ws, &rr);
+    if (!rc) rc = list_rank(list, N, forest + 1, 0, false, -1, forest + 2, st, ws, &rr);
     if (!rc) {
         PhaseTimer pt("br.tin", s);
         launch(k_forest_tin, gn, 256, 0, s, rr, forest, n, tuv, par, head, tin, child, etin, etout);
@@ -811,7 +812,8 @@ extern "C" etl_status two_edge_cc(const int32_t *edges, int64_t m, int32_t n, in
     note_launch();
     if (m > 0) {  // connected components of the graph without its bridges; labels = smallest vertex
         launch(k_hook, hook_grid(hook_positions(m)), kHookChunk, 0, s, edges, edges_aligned(edges), m, 0,
-               hook_positions(m), hook_ilp(hook_positions(m)), false, n, label, nullptr, is_bridge, nullptr, nullptr, nullptr, nullptr, st);
+               hook_positions(m), hook_ilp(hook_positions(m)), false, n, label, nullptr,
+               nullptr, is_bridge, nullptr, nullptr, nullptr, nullptr, st);
         note_launch();
         launch(k_compress<true>, gn, 256, 0, s, n, label, st);
         note_launch();

@@ -209,9 +209,11 @@ etl_status scan_exclusive_u8(const uint8_t *in, int32_t *out, int64_t n, Workspa
 // or -1 (-1 for roots too). parent: ids in [0, n), -1 at roots; anything else is dropped and sets the
 // status. For a batch of k instances, off (k + 1 offsets; *bad: unusable, drop all nodes) says which one a
 // node belongs to, ids are local to it, and gparent receives the global ones (-1 at roots, -2: dropped).
-// root_cnt / root_of (zeroed by the caller): roots per instance and the last one seen.
+// The caller has set head to -1 and cleared root_cnt, root_of (roots per instance and the last one seen) and
+// words (link_words(n) of them, scratch).
+inline int64_t link_words(int64_t n) { return 2 * ((n + 31) / 32) + 2; }
 etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, int32_t k, const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
-                         int32_t *root_of, int32_t *status, Workspace &ws);
+                         int32_t *root_of, int32_t *words, int32_t *status, Workspace &ws);
 
 // ----------------------------------------------------------------- list ranking
 
@@ -345,9 +347,10 @@ RankForm rank_form(int64_t len, bool dual);
 // Ranks a list of len elements in that form, from *d_head, or from `head` if d_head is null. An element
 // that is on no list holds off_list() in a slot, Slot4::kOff as a successor; a contracted leaf's second
 // element off_list() in a slot, -1 as a successor. dual: also counts even-indexed elements (the opening
-// brackets of a tour). expect_len: the total weight the list must have (-1: not checked).
+// brackets of a tour). expect_len: the total weight the list must have (-1: not checked). zero: a device
+// word that is zero when this runs and is not used afterwards (or null: the call clears one itself).
 etl_status list_rank(void *list, int64_t len, const int32_t *d_head, int32_t head, bool dual, int64_t expect_len,
-                     int32_t *status, Workspace &ws, RankResult *out);
+                     int32_t *zero, int32_t *status, Workspace &ws, RankResult *out);
 
 // ----------------------------------------------------------------- sparse tables
 

@@ -54,14 +54,29 @@ __global__ void k_check_offsets(const int32_t *__restrict__ off, int32_t k, int3
     }
 }
 
+// everything a build starts from: no children, cleared counters and status, the batch's offsets
+__global__ void k_lca_init(int32_t n, int32_t *__restrict__ head, int64_t zeros, int32_t *__restrict__ zero,
+                           int32_t *__restrict__ status) {
+    pdl_prologue();
+    if (gtid() == 0) *status = 0;
+    for (int64_t i = gtid(); i < n; i += gstride()) head[i] = -1;
+    for (int64_t i = gtid(); i < zeros; i += gstride()) zero[i] = 0;
+}
+
 // One store per node. A leaf v's brackets are adjacent in the tour: 2v jumps straight to the successor of
 // 2v+1 with weight 2 (top bit set), and 2v+1 is off the list. Roots are never contracted. All accesses
 // are coalesced (the closing brackets' successors were scattered to random places before, which made
-// this step 0.26 ms for 2^24 nodes; now 0.08).
+// this step 0.26 ms for 2^24 nodes; now 0.07).
 template <class S>  // void: successors
 __global__ void k_tour_assemble(const int32_t *__restrict__ par, const int32_t *__restrict__ head,
-                                const int32_t *__restrict__ next, int32_t n, void *__restrict__ list) {
+                                const int32_t *__restrict__ next, int32_t n, const int32_t *__restrict__ roots,
+                                const int32_t *__restrict__ root_of, int32_t *__restrict__ list_head,
+                                void *__restrict__ list, int32_t *__restrict__ status) {
     pdl_prologue();
+    if (roots && gtid() == 0) {  // one tree; k_link_roots does it for a batch
+        *list_head = 2 * *root_of;
+        if (*roots != 1) set_status(status, ETL_EBADTREE);
+    }
     for (int64_t t = gtid(); t < n; t += gstride()) {
         const int32_t p = __ldcs(par + t), h = __ldcs(head + t), x = __ldcs(next + t);
         // leave t -> enter next sibling, or leave p; leave a root -> enter the next root
@@ -186,8 +201,13 @@ template <bool BLOCKED, int kIlp>
 __global__ void __launch_bounds__(256)
     k_parent_pre(const int32_t *__restrict__ parent, const int32_t *__restrict__ pre,
                  const int32_t *__restrict__ tagged, int32_t n, int64_t nblk, int32_t *__restrict__ order,
-                 int32_t *__restrict__ table) {
+                 int32_t *__restrict__ table, const int32_t *__restrict__ root_of, const int32_t *__restrict__ size,
+                 int32_t *__restrict__ status) {
     pdl_prologue();
+    if (root_of && gtid() == 0) {  // a single tree's root opens its tour and spans the tree
+        const int32_t r = *root_of;
+        if (r < 0 || r >= n || pre[r] != 0 || size[r] != n) set_status(status, ETL_EBADTREE);
+    }
     const int64_t N = nblk * kRmqBlock, warps = gstride() / kWarp, warp = gtid() / kWarp;
     const int lane = threadIdx.x & 31;
     int32_t *top = table + 3 * N;
@@ -464,7 +484,6 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         *out = h;
         return ETL_OK;
     }
-    memset_async(h->status, 0, sizeof(int32_t), s);
     if (batch) copy_d2d_async(h->node_off, node_off, size_t(k + 1) * sizeof(int32_t), s);
     etl_status st = ETL_OK;
     {
@@ -474,49 +493,60 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         void *list = form == RankForm::kSlots8 ? static_cast<void *>(ws.get<ulonglong2>(n)) : ws.get<int2>(n);  // 2n elements
         int32_t *head = ws.get<int32_t>(n), *next = ws.get<int32_t>(n);
         int32_t *tagged = head;  // order[] with tags; the first children are not needed once the list is built
-        int32_t *misc = ws.get<int32_t>(2 + 2 * int64_t(k));  // list head, offsets invalid, roots per tree, a root
-        int32_t *root_cnt = misc + 2, *root_of = root_cnt + k;
+        // cleared: offsets invalid, the ranking's counter, roots per tree, a root of each, link_children's words
+        const int64_t zeros = 2 + 2 * int64_t(k) + link_words(n);
+        int32_t *zero = ws.get<int32_t>(zeros + 1), *list_head = zero + zeros;
+        int32_t *bad = zero, *rank_zero = zero + 1, *root_cnt = zero + 2, *root_of = root_cnt + k, *words = root_of + k;
         int32_t *gparent = batch ? ws.get<int32_t>(n) : nullptr;
         if (!ws.ok()) st = ETL_ENOMEM;
         const int32_t *par = batch ? gparent : parent;
         if (!st) {
-            memset_async(misc, 0, (2 + 2 * size_t(k)) * sizeof(int32_t), s);
-            if (batch) {
-                PhaseTimer pt("lca.inst", s);
-                launch(k_check_offsets, grid_for(k, 256), 256, 0, s, h->node_off, k, n, misc + 1, h->status);
+            {
+                PhaseTimer pt("lca.init", s);
+                launch(k_lca_init, grid_for(n, 256), 256, 0, s, n, head, zeros, zero, h->status);
                 note_launch();
+                if (batch) {
+                    launch(k_check_offsets, grid_for(k, 256), 256, 0, s, h->node_off, k, n, bad, h->status);
+                    note_launch();
+                }
             }
-            st = link_children(parent, n, h->node_off, k, misc + 1, gparent, head, next, root_cnt, root_of,
-                               h->status, ws);
+            st = link_children(parent, n, h->node_off, k, bad, gparent, head, next, root_cnt, root_of, words, h->status,
+                               ws);
         }
         if (!st) {
             PhaseTimer pt("lca.succ", s);
-            launch(k_link_roots, grid_for(k, 256), 256, 0, s, root_cnt, root_of, k, n, next, misc, h->status);
-            note_launch();
+            if (batch) {
+                launch(k_link_roots, grid_for(k, 256), 256, 0, s, root_cnt, root_of, k, n, next, list_head, h->status);
+                note_launch();
+            }
             launch(form == RankForm::kSlots8   ? k_tour_assemble<Slot8>
                    : form == RankForm::kSlots4 ? k_tour_assemble<Slot4d>
                                                : k_tour_assemble<void>,
-                   grid_for(n, 256), 256, 0, s, par, head, next, n, list);
+                   grid_for(n, 256), 256, 0, s, par, head, next, n, batch ? nullptr : root_cnt, root_of, list_head, list,
+                   h->status);
             note_launch();
             st = last_launch();
         }
         RankResult rr{};
-        if (!st) st = list_rank(list, 2 * int64_t(n), misc, 0, true, 2 * int64_t(n), h->status, ws, &rr);
+        if (!st) st = list_rank(list, 2 * int64_t(n), list_head, 0, true, 2 * int64_t(n), rank_zero, h->status, ws, &rr);
         if (!st) {
             PhaseTimer pt("lca.node_stats", s);
             launch(rr.wide ? (few ? k_node_stats<ulonglong2, 1> : k_node_stats<ulonglong2, 2>) : k_node_stats<uint2, 2>,
                    grid_for(n, 256), 256, 0, s, rr, n,
                    with_table ? next : nullptr, h->pre, h->depth, h->size, with_table ? tagged : h->order, h->status);
             note_launch();
-            launch(k_check_instances, grid_for(k, 256), 256, 0, s, root_of, batch ? h->node_off : nullptr, k, n, h->pre,
-                   h->size, h->status);
-            note_launch();
+            if (batch || !with_table) {  // k_parent_pre looks at a single tree's root
+                launch(k_check_instances, grid_for(k, 256), 256, 0, s, root_of, batch ? h->node_off : nullptr, k, n,
+                       h->pre, h->size, h->status);
+                note_launch();
+            }
             st = last_launch();
         }
         if (!st && with_table) {
             PhaseTimer pt("lca.parent_pre", s);
             launch(h->blocked ? (few ? k_parent_pre<true, 1> : k_parent_pre<true, 4>) : k_parent_pre<false, 4>,
-                   grid_for(n, few ? 256 : 256 * 4), 256, 0, s, par, h->pre, tagged, n, h->bl.nblk, h->order, h->table);
+                   grid_for(n, few ? 256 : 256 * 4), 256, 0, s, par, h->pre, tagged, n, h->bl.nblk, h->order, h->table,
+                   batch ? nullptr : root_of, h->size, h->status);
             note_launch();
             st = last_launch();
         }

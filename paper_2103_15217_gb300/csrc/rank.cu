@@ -479,10 +479,11 @@ uint32_t splitters(int64_t len, int k) {
 }
 
 // A: where scratch comes from (get<T>(count); a null pointer when there is none). list: len 4-byte
-// successors, recs: room for len records (or null: taken from alloc); in place: list = slots S::T
+// successors, recs: room for len records (or null: taken from alloc); in place: list = slots S::T. zero: a
+// device word that is zero (or null)
 template <class S, bool DUAL, class A>
 etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head, int32_t head, int64_t expect_len,
-                     int32_t *status, const RankParams &P, A &alloc, cudaStream_t s, RankResult *out) {
+                     int32_t *zero, int32_t *status, const RankParams &P, A &alloc, cudaStream_t s, RankResult *out) {
     using R = typename S::T;
     const bool in_place = rank_form(len, DUAL) != RankForm::kSeparate;
     constexpr bool kNarrow = std::is_same<S, Slot4d>::value;
@@ -517,7 +518,10 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
     int nl = 0;
     int32_t *words = alloc.template get<int32_t>(64);  // per level: [2 i] entry count, [2 i + 1] head
     if (!words) return ETL_ENOMEM;
-    memset_async(words, 0, sizeof(int32_t), s);
+    if (!zero) {
+        zero = words;
+        memset_async(zero, 0, sizeof(int32_t), s);
+    }
     if (in_place) {
         Walk0 w{};
         w.len = len;
@@ -549,9 +553,9 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         out->lb = w.lb;
         int4 *T = alloc.template get<int4>(w.cap);
         if (!T) return ETL_ENOMEM;
-        lv[nl++] = Level{T, nullptr, w.start, w.cap, words, words + 1};
+        lv[nl++] = Level{T, nullptr, w.start, w.cap, zero, words + 1};
         PhaseTimer pt0("rank.walk0", s);
-        launch(k_walk0_in_place<S, DUAL>, grid, P.block, 0, s, static_cast<R *>(recs), w, T, words, words + 1, status);
+        launch(k_walk0_in_place<S, DUAL>, grid, P.block, 0, s, static_cast<R *>(recs), w, T, zero, words + 1, status);
         note_launch();
         st = last_launch();
     } else {
@@ -572,10 +576,10 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         }
         int4 *T = alloc.template get<int4>(cap);
         if (!T) return ETL_ENOMEM;
-        lv[nl++] = Level{T, nullptr, int64_t(H.S0) + 1, cap, words, words + 1};
+        lv[nl++] = Level{T, nullptr, int64_t(H.S0) + 1, cap, zero, words + 1};
         PhaseTimer pt0("rank.walk0", s);
         launch(k_walk0<S, DUAL>, grid_of(int64_t(H.S0) + 1, 2048 / P.block, P), P.block, 0, s, succ, len, d_head, head,
-               H, static_cast<R *>(recs), out->lb, lcap, T, words, cap, words + 1, status);
+               H, static_cast<R *>(recs), out->lb, lcap, T, zero, cap, words + 1, status);
         note_launch();
         st = last_launch();
     }
@@ -652,8 +656,8 @@ etl_status rank_plain_list(const int32_t *succ, int64_t len, int32_t head, int32
     etl_status rc = last_launch();
     RankResult rr{};
     if (!rc)
-        rc = wide ? rank_impl<Slot8, false>(list, recs, len, nullptr, head, len, status, P, alloc, s, &rr)
-                  : rank_impl<Slot4, false>(list, recs, len, nullptr, head, len, status, P, alloc, s, &rr);
+        rc = wide ? rank_impl<Slot8, false>(list, recs, len, nullptr, head, len, nullptr, status, P, alloc, s, &rr)
+                  : rank_impl<Slot4, false>(list, recs, len, nullptr, head, len, nullptr, status, P, alloc, s, &rr);
     if (rc) return rc;
     PhaseTimer pt("rank.final", s);
     launch(k_final_rank, blocks, 256, 0, s, rr, len, rank);
@@ -664,15 +668,15 @@ etl_status rank_plain_list(const int32_t *succ, int64_t len, int32_t head, int32
 }  // namespace
 
 etl_status list_rank(void *list, int64_t len, const int32_t *d_head, int32_t head, bool dual, int64_t expect_len,
-                     int32_t *status, Workspace &ws, RankResult *out) {
+                     int32_t *zero, int32_t *status, Workspace &ws, RankResult *out) {
     cudaStream_t s = ws.stream();
     const RankParams &P = rank_params();
     if (dual && rank_form(len, true) == RankForm::kSlots4)
-        return rank_impl<Slot4d, true>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
-    if (dual) return rank_impl<Slot8, true>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
+        return rank_impl<Slot4d, true>(list, nullptr, len, d_head, head, expect_len, zero, status, P, ws, s, out);
+    if (dual) return rank_impl<Slot8, true>(list, nullptr, len, d_head, head, expect_len, zero, status, P, ws, s, out);
     if (wide_slots(len))
-        return rank_impl<Slot8, false>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
-    return rank_impl<Slot4, false>(list, nullptr, len, d_head, head, expect_len, status, P, ws, s, out);
+        return rank_impl<Slot8, false>(list, nullptr, len, d_head, head, expect_len, zero, status, P, ws, s, out);
+    return rank_impl<Slot4, false>(list, nullptr, len, d_head, head, expect_len, zero, status, P, ws, s, out);
 }
 
 }  // namespace etl

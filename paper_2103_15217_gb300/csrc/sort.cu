@@ -392,15 +392,11 @@ SortParams &sort_params() {
 }
 
 etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, int32_t k, const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
-                         int32_t *root_of, int32_t *status, Workspace &ws) {
+                         int32_t *root_of, int32_t *words, int32_t *status, Workspace &ws) {
     cudaStream_t s = ws.stream();
-    const int64_t mask_words = ceil_div(n, 32);
-    uint32_t *words = ws.get<uint32_t>(2 * mask_words + 2);  // seen, heavy, heavy families, barrier
-    if (!ws.ok()) return ETL_ENOMEM;
-    uint32_t *heavy = words + mask_words, *bar = words + 2 * mask_words + 1;
-    int32_t *heavy_count = reinterpret_cast<int32_t *>(words + 2 * mask_words);
-    memset_async(words, 0, size_t(2 * mask_words + 2) * 4, s);
-    memset_async(head, 0xff, size_t(n) * 4, s);
+    const int64_t mask_words = ceil_div(n, 32);  // words: seen, heavy, heavy families, barrier
+    uint32_t *seen = reinterpret_cast<uint32_t *>(words), *heavy = seen + mask_words, *bar = seen + 2 * mask_words + 1;
+    int32_t *heavy_count = words + 2 * mask_words;
     const int32_t *par = off ? gparent : parent;
     {
         PhaseTimer pt("lca.link", s);
@@ -413,7 +409,7 @@ etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, i
         PhaseTimer pt("lca.check", s);
         const bool small = n <= kCheckSmall;
         const int64_t blocks = ceil_div(n, kCheckThreads * (small ? 1 : 4)), most = int64_t(num_sms()) * 8;
-        launch(small ? k_check_children<1> : k_check_children<4>, int(blocks < most ? blocks : most), kCheckThreads, 0, s, par, n, head, next, words, heavy,
+        launch(small ? k_check_children<1> : k_check_children<4>, int(blocks < most ? blocks : most), kCheckThreads, 0, s, par, n, head, next, seen, heavy,
                heavy_count);
         note_launch();
     }
