@@ -61,27 +61,19 @@ __device__ __forceinline__ int2 load_edge(const int32_t *__restrict__ edges, int
 }
 inline bool edges_aligned(const int32_t *edges) { return (reinterpret_cast<uintptr_t>(edges) & 7) == 0; }
 
-// Root of x with path halving; -1 if the step budget runs out. giant (or -1): a root that stays one while
-// this runs, so that pointing at it ends the walk without another load. A node's pointer is read from
-// L2, its parent's through L1 unless `fresh`: parents are few and popular (a large component's root is on
-// every other path, and reads of one address are served one after another by its L2 slice). A stale
-// pointer does no harm: it still leads to an ancestor, a root that is none any more makes the hook's CAS
-// fail or lets it point at an inner node of higher rank; after a failed hook the pointers are read fresh.
-// MIN (only where ancestors have smaller ids): pointers never move down again, whatever order the writes
-// of several lanes come in.
-template <bool MIN = false>
-__device__ __forceinline__ int32_t find_root(int32_t *par, int32_t x, int64_t &budget, int32_t giant = -1,
-                                             bool fresh = true) {
+// Root of x with path halving; -1 if the step budget runs out. MIN (only where ancestors have smaller ids):
+// pointers never move down again, whatever order the writes of several lanes come in.
+template <bool MIN>
+__device__ __forceinline__ int32_t find_root(int32_t *par, int32_t x, int64_t &budget) {
     while (budget-- > 0) {
         const int32_t p = __ldcg(par + x);
-        if (p == x || p == giant) return p;
-        const int32_t gp = fresh ? __ldcg(par + p) : __ldca(par + p);
+        if (p == x) return p;
+        const int32_t gp = __ldcg(par + p);
         if (gp == p) return p;
         if (MIN)
             atomicMin(par + x, gp);
         else
             atomicExch(par + x, gp);  // only non-roots are rewritten, always to an ancestor
-        if (gp == giant) return gp;
         x = gp;
     }
     return -1;
@@ -99,7 +91,13 @@ __device__ __forceinline__ int32_t find_root(int32_t *par, int32_t x, int64_t &b
 // contiguous order, which measured faster on it (0.7 against 1.3 ms on 2^25 shuffled edges).
 constexpr int kHookChunk = 256;
 constexpr int kHookIlp = 4;
-constexpr int64_t kHookAtOnce = 98304;  // edges hooked in one launch, without a first slice
+// Hook launches, us (random graphs; hard ones, of long paths, in brackets). Up to kHookAtOnce edges go in one
+// launch: 32770 edges on 16385 vertices 27 against 30 in two (20, 34), 32768 on 8192 33 against 29 (21, 32),
+// 65536 on 8192 72 against 31, on 16385 50 against 31 (22, 35). Half as many edges again in the first slice
+// up to kHookMoreFirst vertices: 2^15.3 vertices, 4 edges each 59 -> 38, 2^17 77 -> 59 (57 -> 53), 2^18
+// 74 -> 78, 2^20 123 -> 175; there the slice itself is the dearer part.
+constexpr int64_t kHookAtOnce = 49152;
+constexpr int32_t kHookMoreFirst = 1 << 17;
 constexpr int kHookSuper = 32;
 
 // number of positions of the chunk sequence over m edges (whole superchunks)
@@ -123,13 +121,17 @@ __device__ __forceinline__ bool hook_above(int32_t a, int32_t b, int32_t giant) 
 }
 
 // Most edges join two vertices that already point at the same node; those cost two loads, all of a
-// block step's in flight together. The others go to a queue in shared memory, and the block finds and
-// hooks them 256 at a time with every lane busy (one lane's walk to a root held up the other 31 before).
-// The edges that join two trees are appended to the forest's list, one counter update per round. Easy
-// graph of 2^22 vertices and 2^25 edges: 735 us before, 680 with the queue, 530 with the giant root known
-// to find_root, 500 with the halving done by exchanges (a plain store to a sector that others read takes
-// over 1 us); the two loads per edge of its 31.4M later edges alone take 210 us. Batch of 512 graphs: 1430
-// -> 580 us. Graphs of up to kHookAtOnce edges skip the first slice: 2^14 vertices, 2^16 edges 65 -> 50 us.
+// block step's in flight together. The others go to a queue in shared memory, and the block hooks them
+// 256 at a time with every lane busy (one lane's walk to a root held up the other 31 before). A lane walks
+// up from both ends of its edge at once, halving both paths, until they meet (usually well below the root)
+// or both end at roots. Halving is done by exchanges: a plain store to a sector that others read takes over
+// 1 us. A node's pointer is read from L2, its parent's through L1: parents are few and popular (reads of
+// one address are served one after another by its L2 slice). A stale one does no harm: it still leads to
+// an ancestor, what is no root any more makes the CAS fail, and the walk goes on from its own pointer. The
+// edges that join two trees are appended to the forest's list, one counter update per round. Easy graph of
+// 2^22 vertices and 2^25 edges, whole pass: 735 us without the queue, 680 with it, 530 with the giant root
+// known to the walks, 500 with exchanges, 478 with both walks at once (hard graph 557 -> 470, 512 graphs
+// 588 -> 456); the two loads per edge of its 31.4M later edges alone take 210 us.
 // skip (may be null): edges to leave out; is_tree (may be null): 1 for edges whose hook succeeded, and
 // then is_bridge is cleared and forest_count, tuv (both ends of forest edge t) and tedge (its edge) are written too
 __global__ void __launch_bounds__(kHookChunk)
@@ -187,23 +189,28 @@ __global__ void __launch_bounds__(kHookChunk)
             if (i < have) {
                 int32_t a = qa[i], b = qb[i];
                 int64_t budget = kFindCap;
-                bool fresh = false;
-                while (true) {
-                    const int32_t ra = find_root(par, a, budget, giant, fresh), rb = find_root(par, b, budget, giant, fresh);
-                    if (ra < 0 || rb < 0) {
+                while (true) {  // both walks at once, up to a node on both
+                    if (budget-- <= 0) {
                         set_status(status, ETL_ETIMEOUT);
                         break;
                     }
-                    if (ra == rb) break;
-                    const bool a_up = hook_above(ra, rb, giant);
-                    const int32_t hi = a_up ? rb : ra, lo = a_up ? ra : rb;  // hi goes under lo
+                    const int32_t pa = a == giant ? a : __ldcg(par + a), pb = b == giant ? b : __ldcg(par + b);
+                    if (pa == pb) break;
+                    const bool ta = pa == a || pa == giant, tb = pb == b || pb == giant;
+                    const int32_t ga = ta ? pa : __ldca(par + pa);
+                    const int32_t gb = tb ? pb : __ldca(par + pb);
+                    if (ga != pa) atomicExch(par + a, ga);  // only non-roots are rewritten, always to an ancestor
+                    if (gb != pb) atomicExch(par + b, gb);
+                    if (ga == gb) break;
+                    a = ga;
+                    b = gb;
+                    if ((ga != pa && ga != giant) || (gb != pb && gb != giant)) continue;
+                    const bool a_up = hook_above(a, b, giant);
+                    const int32_t hi = a_up ? b : a, lo = a_up ? a : b;  // hi goes under lo
                     if (atomicCAS(par + hi, hi, lo) == hi) {
                         won = true;
                         break;
-                    }
-                    a = ra;  // someone hooked one of the roots meanwhile: retry from them
-                    b = rb;
-                    fresh = true;
+                    }  // someone hooked one of the roots meanwhile: on from them
                 }
             }
             if (!is_tree) continue;
@@ -230,12 +237,78 @@ __global__ void __launch_bounds__(kHookChunk)
     }
 }
 
+// The root most often reached from kGiantSample vertices spread over [0, n): the giant component's when
+// there is one. k_hook takes it for a root, so every walk goes on to a true one. One block
+constexpr int kGiantSample = 1024;
+
+__device__ void sample_giant(const int32_t *__restrict__ par, int32_t n, int32_t *__restrict__ giant) {
+    constexpr int kSlots = 2 * kGiantSample;  // open-addressing table of (root, count)
+    __shared__ int32_t key[kSlots], cnt[kSlots];
+    __shared__ unsigned long long best;
+    for (int j = threadIdx.x; j < kSlots; j += blockDim.x) {
+        key[j] = -1;
+        cnt[j] = 0;
+    }
+    if (threadIdx.x == 0) best = 0;
+    __syncthreads();
+    for (int i0 = threadIdx.x; i0 < kGiantSample; i0 += 4 * blockDim.x) {
+        int32_t r[4], p[4];
+        int64_t budget = kFindCap;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            r[j] = int32_t((uint64_t(i0 + j * int(blockDim.x)) * 2654435761u + 12345u) % uint64_t(n));
+        bool more = true;
+        while (more && budget-- > 0) {
+            more = false;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) p[j] = __ldcg(par + r[j]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                more |= p[j] != r[j];
+                r[j] = p[j];
+            }
+        }
+        for (int j = 0; j < 4; ++j) {
+            if (i0 + j * int(blockDim.x) >= kGiantSample) break;
+            uint32_t h = (uint32_t(r[j]) * 2654435761u) >> 21;  // 11 bits: kSlots = 2048
+            for (int probe = 0; probe < kSlots; ++probe, h = (h + 1) & (kSlots - 1)) {
+                const int32_t prev = atomicCAS(&key[h], -1, r[j]);
+                if (prev == -1 || prev == r[j]) {
+                    atomicAdd(&cnt[h], 1);
+                    break;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    // largest count, then smallest root id: pack (count, ~root) and take the maximum
+    for (int j = threadIdx.x; j < kSlots; j += blockDim.x)
+        if (cnt[j]) atomicMax(&best, (static_cast<unsigned long long>(cnt[j]) << 32) | uint32_t(~uint32_t(key[j])));
+    __syncthreads();
+    if (threadIdx.x == 0) *giant = int32_t(~uint32_t(best & 0xffffffffu));
+}
+
+// Up to kGiantBeside vertices the giant is found by an extra block of the compression (2^14 vertices 36 ->
+// 31 us for both hook launches), beyond by a launch after it, when its walks are one step: the table in
+// shared memory takes L1 from all blocks of the compression and of what runs next (hard graph of 2^22
+// vertices 518 us against 470).
+constexpr int32_t kGiantBeside = 1 << 18;
+
 // Points every vertex at its root. EXACT: at the root itself in the end (the labels of components hooked in
-// id order); otherwise a lane that halves a path late may leave a vertex at an inner node.
-template <bool EXACT>
-__global__ void k_compress(int32_t n, int32_t *__restrict__ par, int32_t *__restrict__ status) {
+// id order); otherwise a lane that halves a path late may leave a vertex at an inner node, and the last
+// block finds the giant root meanwhile
+template <bool EXACT, bool GIANT>
+__global__ void k_compress(int32_t n, int32_t *__restrict__ par, int32_t *__restrict__ giant, int32_t *__restrict__ status) {
     pdl_prologue();
-    for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n; v += int64_t(gridDim.x) * blockDim.x) {
+    int64_t blocks = gridDim.x;
+    if (GIANT) {
+        --blocks;
+        if (blockIdx.x == blocks) {
+            sample_giant(par, n, giant);
+            return;
+        }
+    }
+    for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < n; v += blocks * blockDim.x) {
         int64_t budget = kFindCap;
         const int32_t p = __ldcg(par + v), r = find_root<EXACT>(par, p, budget);
         if (r < 0) {
@@ -249,49 +322,9 @@ __global__ void k_compress(int32_t n, int32_t *__restrict__ par, int32_t *__rest
     }
 }
 
-// The root most frequently pointed at among kGiantSample vertices spread over [0, n) (one block; par is
-// compressed, so nearly every vertex points at its root): the giant component's when there is one.
-constexpr int kGiantSample = 1024;
-
-__global__ void __launch_bounds__(kGiantSample) k_giant(const int32_t *__restrict__ par, int32_t n,
-                                                         int32_t *__restrict__ giant) {
+__global__ void k_giant(const int32_t *__restrict__ par, int32_t n, int32_t *__restrict__ giant) {
     pdl_prologue();
-    constexpr int kSlots = 2 * kGiantSample;  // open-addressing table of (root, count)
-    __shared__ int32_t key[kSlots], cnt[kSlots];
-    __shared__ unsigned long long best;
-    const int i = threadIdx.x;
-    for (int j = i; j < kSlots; j += kGiantSample) {
-        key[j] = -1;
-        cnt[j] = 0;
-    }
-    if (i == 0) best = 0;
-    __syncthreads();
-    const int32_t v = int32_t((uint64_t(i) * 2654435761u + 12345u) % uint64_t(n));
-    const int32_t r = __ldcg(par + v);
-    int slot = -1;
-    uint32_t h = (uint32_t(r) * 2654435761u) >> 21;  // 11 bits: kSlots = 2048
-    for (int probe = 0; probe < kSlots; ++probe, h = (h + 1) & (kSlots - 1)) {
-        const int32_t prev = atomicCAS(&key[h], -1, r);
-        if (prev == -1 || prev == r) {
-            slot = int(h);
-            atomicAdd(&cnt[h], 1);
-            break;
-        }
-    }
-    __syncthreads();
-    // largest count, then smallest root id: pack (count, ~root) and take the maximum
-    if (slot >= 0)
-        atomicMax(&best, (static_cast<unsigned long long>(cnt[slot]) << 32) | uint32_t(~uint32_t(r)));
-    __syncthreads();
-    if (i == 0) {  // k_hook takes it for a root, so it has to be one
-        int32_t r = best ? int32_t(~uint32_t(best & 0xffffffffu)) : 0;
-        for (int64_t budget = kFindCap; budget > 0; --budget) {
-            const int32_t p = __ldcg(par + r);
-            if (p == r) break;
-            r = p;
-        }
-        *giant = r;
-    }
+    sample_giant(par, n, giant);
 }
 
 // next[a] = the half-edge pushed onto its tail's list before a (-1: none). Half-edges of one tail in a
@@ -617,15 +650,20 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
         // compression, so that no phase builds long paths in a fresh part of the forest.
         const CcParams &C = cc_params();
         const int64_t nchunks = hook_positions(m);
-        const int64_t slice = int64_t(C.first_slice_quarters) * n / 4;
+        int64_t slice = int64_t(C.first_slice_quarters) * n / 4;
+        if (n <= kHookMoreFirst) slice += slice / 2;
         int64_t w = m <= kHookAtOnce ? nchunks : ceil_div(slice > 0 ? slice : 1, kHookChunk);  // chunks in the current slice
         PhaseTimer pt("br.hook", s);
         for (int64_t c0 = 0; c0 < nchunks;) {
             const int64_t c1 = (C.doubling || c0 == 0) ? (c0 + w < nchunks ? c0 + w : nchunks) : nchunks;
             if (c0 > 0) {
-                launch(k_compress<false>, gn, 256, 0, s, n, par, st);
+                const bool beside = C.giant && n <= kGiantBeside;
+                if (beside)
+                    launch(k_compress<false, true>, gn + 1, 256, 0, s, n, par, giant, st);
+                else
+                    launch(k_compress<false, false>, gn, 256, 0, s, n, par, nullptr, st);
                 note_launch();
-                if (C.giant) {
+                if (C.giant && !beside) {
                     launch(k_giant, 1, kGiantSample, 0, s, par, n, giant);
                     note_launch();
                 }
@@ -815,7 +853,7 @@ extern "C" etl_status two_edge_cc(const int32_t *edges, int64_t m, int32_t n, in
                hook_positions(m), hook_ilp(hook_positions(m)), false, n, label, nullptr,
                nullptr, is_bridge, nullptr, nullptr, nullptr, nullptr, st);
         note_launch();
-        launch(k_compress<true>, gn, 256, 0, s, n, label, st);
+        launch(k_compress<true, false>, gn, 256, 0, s, n, label, nullptr, st);
         note_launch();
     }
     launch(k_labels_on_error, gn, 256, 0, s, n, st, label);

@@ -1,7 +1,8 @@
 """Bridges at the places where the connectivity pass and the forest's tour change form: graphs hooked in
-one launch (up to 98304 edges) and in slices, edge arrays that are and are not 8-byte aligned, forests of
-many components (each starts a tour of its own in one list), stars (one tail for every half-edge),
-isolated vertices and loops. Masks and 2-edge-connected labels are unique, so they are compared exactly."""
+one launch (up to 49152 edges) and in slices (the giant component's root found beside the compression or
+after it), edge arrays that are and are not 8-byte aligned, forests of many components (each starts a tour
+of its own in one list), stars (one tail for every half-edge), isolated vertices and loops. Masks and
+2-edge-connected labels are unique, so they are compared exactly."""
 
 import numpy as np
 import pytest
@@ -32,7 +33,9 @@ def star(n, seed):
     return rng.permutation(np.concatenate([e, extra])).astype(np.int32)
 
 
-CASES = [(f"easy {m}", lambda m=m: (20000, synth.easy_graph(20000, m, seed=m))) for m in (AT_ONCE - 1, AT_ONCE, AT_ONCE + 1)] + \
+CASES = [(f"easy {m}", lambda m=m: (20000, synth.easy_graph(20000, m, seed=m))) for a in (AT_ONCE // 2, AT_ONCE) for m in (a - 1, a, a + 1)] + \
+        [(f"random {n}", lambda n=n: (n, synth.easy_graph(n, 2 * n, seed=n))) for n in (1 << 17, (1 << 17) + 1, 1 << 18, (1 << 18) + 1)] + \
+        [(f"paths {n}", lambda n=n: (n, synth.hard_graph(n, n, n // 100, seed=n))) for n in (1 << 17, (1 << 18) + 1)] + \
         [(f"groups of {s}", lambda s=s: (50001, many_components(50001, 60000, s, s))) for s in (1, 2, 3, 33, 1000)] + \
         [("large groups", lambda: (300000, many_components(300000, 500000, 5, 7))),
          ("star", lambda: (40001, star(40001, 1))), ("large star", lambda: (200000, star(200000, 2))),
