@@ -188,21 +188,25 @@ __global__ void k_node_stats(RankResult rr, int32_t n, const int32_t *__restrict
 }
 
 constexpr int32_t kFewNodes = 1 << 21;
+constexpr int32_t kRecsHere = 1 << 20;
 
 // Q in preorder: position i holds pre(parent(order[i])). If the node before i has children, it is i's
 // parent: Q[i] = i - 1. If it is a leaf with a next sibling, i is that sibling: Q[i] = Q[i - 1]. Only after
 // a leaf that is a last child (the rest: 30% of a random tree's positions, none of a path's) parent[] and
 // pre[] have to be read at random places. A warp takes a block of 32 positions, kIlp blocks at a time, and
 // leaves the block's prefix / suffix minima and its result, too (table: x, (pm, sm) pairs, top row 0 of the
-// blocked layout; BLOCKED false: x only). tagged = order as k_node_stats left it, order = without tags.
+// blocked layout; BLOCKED false: x only). RECS: the nodes' query records (below) instead of the pairs, in
+// random order: up to kRecsHere nodes, whose records fit L2 well, that beats a launch of its own that
+// gathers the pairs (whole preprocessing and n / 4 queries, us: 2^16 nodes 78.2 -> 76.9, 2^20 193.6 -> 189.1,
+// 2^21 293.8 -> 302.2, 2^24 1775 -> 2380). tagged = order as k_node_stats left it, order = without tags.
 // 2^24 nodes: random 153 us, path 72, with two gathers per position and a pass of its own for the
 // blocks 307 and 379.
-template <bool BLOCKED, int kIlp>
+template <bool BLOCKED, bool RECS, int kIlp>
 __global__ void __launch_bounds__(256)
     k_parent_pre(const int32_t *__restrict__ parent, const int32_t *__restrict__ pre,
                  const int32_t *__restrict__ tagged, int32_t n, int64_t nblk, int32_t *__restrict__ order,
-                 int32_t *__restrict__ table, const int32_t *__restrict__ root_of, const int32_t *__restrict__ size,
-                 int32_t *__restrict__ status) {
+                 int32_t *__restrict__ table, int4 *__restrict__ nrec, const int32_t *__restrict__ root_of,
+                 const int32_t *__restrict__ size, int32_t *__restrict__ status) {
     pdl_prologue();
     if (root_of && gtid() == 0) {  // a single tree's root opens its tour and spans the tree
         const int32_t r = *root_of;
@@ -212,12 +216,19 @@ __global__ void __launch_bounds__(256)
     const int lane = threadIdx.x & 31;
     int32_t *top = table + 3 * N;
     for (int64_t b0 = warp * kIlp; b0 < nblk; b0 += warps * kIlp) {
-        int32_t w[kIlp], before[kIlp], q[kIlp];
+        int32_t w[kIlp], before[kIlp], q[kIlp], sz[kIlp];
 #pragma unroll
         for (int j = 0; j < kIlp; ++j) {
             const int64_t i = (b0 + j) * kRmqBlock + lane;
             w[j] = b0 + j < nblk && i < n ? __ldg(tagged + i) : -1;
             before[j] = lane == 0 && b0 + j < nblk && i > 0 ? __ldg(tagged + i - 1) : -1;
+        }
+        if (RECS) {
+#pragma unroll
+            for (int j = 0; j < kIlp; ++j) {
+                const int32_t v = w[j] & 0x3fffffff;
+                sz[j] = v < n ? __ldg(size + v) : 0;
+            }
         }
 #pragma unroll
         for (int j = 0; j < kIlp; ++j) {
@@ -259,7 +270,10 @@ __global__ void __launch_bounds__(256)
                     if (lane >= d) a = min(a, ua);
                     if (lane + d < kRmqBlock) c = min(c, dc);
                 }
-                __stcs(reinterpret_cast<int2 *>(table + N) + i, make_int2(a, c));
+                if (!RECS)
+                    __stcs(reinterpret_cast<int2 *>(table + N) + i, make_int2(a, c));
+                else if (i < n && (w[j] & 0x3fffffff) < n)
+                    nrec[w[j] & 0x3fffffff] = make_int4(int32_t(i), a, c, sz[j]);
                 if (lane == kRmqBlock - 1) top[b0 + j] = a;
             }
         }
@@ -489,6 +503,7 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
     {
         Workspace ws(s);
         const RankForm form = rank_form(2 * int64_t(n), true);
+        const bool recs_here = h->blocked && n <= kRecsHere;
         const bool few = n <= kFewNodes;  // one node per thread and step fills the GPU better
         void *list = form == RankForm::kSlots8 ? static_cast<void *>(ws.get<ulonglong2>(n)) : ws.get<int2>(n);  // 2n elements
         int32_t *head = ws.get<int32_t>(n), *next = ws.get<int32_t>(n);
@@ -544,16 +559,19 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         }
         if (!st && with_table) {
             PhaseTimer pt("lca.parent_pre", s);
-            launch(h->blocked ? (few ? k_parent_pre<true, 1> : k_parent_pre<true, 4>) : k_parent_pre<false, 4>,
+            launch(!h->blocked ? k_parent_pre<false, false, 4>
+                   : recs_here ? k_parent_pre<true, true, 1>
+                   : few       ? k_parent_pre<true, false, 1>
+                               : k_parent_pre<true, false, 4>,
                    grid_for(n, few ? 256 : 256 * 4), 256, 0, s, par, h->pre, tagged, n, h->bl.nblk, h->order, h->table,
-                   batch ? nullptr : root_of, h->size, h->status);
+                   static_cast<int4 *>(h->nrec), batch ? nullptr : root_of, h->size, h->status);
             note_launch();
             st = last_launch();
         }
         if (!st && with_table)
             st = h->blocked ? blocked_top<OpMin>(h->table + 3 * h->bl.nblk * kRmqBlock, h->bl, s)
                             : sparse_table_build<false>(h->table, n, h->levels, s);
-        if (!st && with_table && h->blocked) {
+        if (!st && with_table && h->blocked && !recs_here) {
             PhaseTimer pt("lca.node_rec", s);
             launch(few ? k_node_rec<1> : k_node_rec<4>, grid_for(n, 256), 256, 0, s, h->pre, h->size,
                    reinterpret_cast<const int2 *>(h->table + h->bl.nblk * kRmqBlock), n, static_cast<int4 *>(h->nrec));
