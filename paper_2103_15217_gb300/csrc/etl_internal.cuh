@@ -210,10 +210,10 @@ etl_status scan_exclusive_u8(const uint8_t *in, int32_t *out, int64_t n, Workspa
 // status. For a batch of k instances, off (k + 1 offsets; *bad: unusable, drop all nodes) says which one a
 // node belongs to, ids are local to it, and gparent receives the global ones (-1 at roots, -2: dropped).
 // The caller has set head to -1 and cleared root_cnt, root_of (roots per instance and the last one seen) and
-// words (link_words(n) of them, scratch).
+// words (link_words(n) of them, scratch). head and next may come back as other arrays of the workspace.
 inline int64_t link_words(int64_t n) { return 2 * ((n + 31) / 32) + 2; }
-etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, int32_t k, const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
-                         int32_t *root_of, int32_t *words, int32_t *status, Workspace &ws);
+etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, int32_t k, const int32_t *bad, int32_t *gparent,
+                         int32_t *&head, int32_t *&next, int32_t *root_cnt, int32_t *root_of, int32_t *words, int32_t *status, Workspace &ws);
 
 // ----------------------------------------------------------------- list ranking
 

@@ -507,7 +507,6 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
         const bool few = n <= kFewNodes;  // one node per thread and step fills the GPU better
         void *list = form == RankForm::kSlots8 ? static_cast<void *>(ws.get<ulonglong2>(n)) : ws.get<int2>(n);  // 2n elements
         int32_t *head = ws.get<int32_t>(n), *next = ws.get<int32_t>(n);
-        int32_t *tagged = head;  // order[] with tags; the first children are not needed once the list is built
         // cleared: offsets invalid, the ranking's counter, roots per tree, a root of each, link_children's words
         const int64_t zeros = 2 + 2 * int64_t(k) + link_words(n);
         int32_t *zero = ws.get<int32_t>(zeros + 1), *list_head = zero + zeros;
@@ -542,6 +541,7 @@ etl_status lca_build(const int32_t *parent, int32_t n, const int32_t *node_off, 
             note_launch();
             st = last_launch();
         }
+        int32_t *tagged = head;  // order[] with tags; the first children are not needed once the list is built
         RankResult rr{};
         if (!st) st = list_rank(list, 2 * int64_t(n), list_head, 0, true, 2 * int64_t(n), rank_zero, h->status, ws, &rr);
         if (!st) {

@@ -9,12 +9,14 @@
 //    scanning the counts and a stable 3-pass radix sort of (parent, child) pairs took 0.54 ms, and a
 //    random tree's successors another 0.17 ms of random writes that the lists do not need.
 //  * k_check_children finds every link that does not ascend and sorts that family's list on the spot
-//    (up to kLight children, by one thread).
+//    (up to kLight children, by one thread). k_sort_children takes its place on small inputs, where most do not.
 //  * k_sort_heavy does longer families that are out of order: a stable LSD radix sort of their
 //    (parent, child) pairs, 8 bits per pass, in one cooperative launch, which returns at once when
 //    there are none (3 us). Inside a tile each warp ranks its 32-element rounds (peers with the same
 //    digit by __match_any_sync or by eight ballots) with per-warp smem counters; the ranked tile is
 //    staged in shared memory in digit order and written out in runs.
+#include <climits>
+
 #include "etl_internal.cuh"
 
 namespace etl {
@@ -97,7 +99,7 @@ __global__ void __launch_bounds__(kLinkThreads)
 // `seen`) and puts it on its block's list; the block sorts those together (one thread each), so that
 // the few walks do not hold up warps that are checking: 2^24 nodes of a random tree 0.19 -> 0.06 ms.
 // Threads that check may read links being rewritten; whatever they see, they find the bit set. On a
-// small tree most families have to be sorted, by as many blocks as there are (ILP 1).
+// smaller tree many families have to be sorted, by as many blocks as there are (ILP 1).
 constexpr int kCheckThreads = 256;
 constexpr int64_t kCheckSmall = int64_t(1) << 19;
 
@@ -154,6 +156,41 @@ __global__ void __launch_bounds__(kCheckThreads)
             if (threadIdx.x == 0) count = 0;
         }
         __syncthreads();
+    }
+}
+
+// Up to kSortAll nodes nearly every family is pushed by threads that run together and has to be sorted, and
+// what counts is the chain of dependent steps. Every node walks its family's list itself: the least larger
+// label is its next sibling, and the least of all the first child. No marks, no second stage, and no
+// insertions one after another. Results go to arrays of their own, so that nothing read changes (and L1
+// serves the walks of siblings). Bound by the latency of the longest list: random tree of 2^16 nodes 8.7 us
+// (k_check_children 18.3), of 2^18 11 (20), families of 30 27 (62); a path, which has nothing to sort, 8.6
+// (6.2). Beyond, the work grows with the squares of the families: 2^20 random 23 (23), families of 30 119 (61).
+constexpr int32_t kSortAll = 1 << 18;
+
+__global__ void __launch_bounds__(kCheckThreads)
+    k_sort_children(const int32_t *__restrict__ par, int32_t n, const int32_t *__restrict__ head,
+                    const int32_t *__restrict__ next, int32_t *__restrict__ head2, int32_t *__restrict__ next2,
+                    uint32_t *__restrict__ heavy, int32_t *__restrict__ heavy_count) {
+    pdl_prologue();
+    const int64_t t = gtid();
+    if (t >= n) return;
+    if (head[t] < 0) head2[t] = -1;
+    const int32_t p = par[t], first = p >= 0 && p < n ? __ldg(head + p) : -1;
+    int32_t c = first, after = INT_MAX, least = INT_MAX;
+    for (int k = 0; c >= 0 && c < n && k < kLight; ++k) {
+        least = min(least, c);
+        if (c > t) after = min(after, c);
+        c = __ldg(next + c);
+    }
+    next2[t] = after < INT_MAX ? after : -1;
+    if (c >= 0) {  // too many for one thread: k_sort_heavy writes all of the family's links
+        if (first == t) {
+            atomicOr(heavy + (p >> 5), 1u << (p & 31));
+            atomicAdd(heavy_count, 1);
+        }
+    } else if (least == t) {
+        head2[p] = int32_t(t);
     }
 }
 
@@ -391,8 +428,8 @@ SortParams &sort_params() {
     return p;
 }
 
-etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, int32_t k, const int32_t *bad, int32_t *gparent, int32_t *head, int32_t *next, int32_t *root_cnt,
-                         int32_t *root_of, int32_t *words, int32_t *status, Workspace &ws) {
+etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, int32_t k, const int32_t *bad, int32_t *gparent,
+                         int32_t *&head, int32_t *&next, int32_t *root_cnt, int32_t *root_of, int32_t *words, int32_t *status, Workspace &ws) {
     cudaStream_t s = ws.stream();
     const int64_t mask_words = ceil_div(n, 32);  // words: seen, heavy, heavy families, barrier
     uint32_t *seen = reinterpret_cast<uint32_t *>(words), *heavy = seen + mask_words, *bar = seen + 2 * mask_words + 1;
@@ -407,10 +444,19 @@ etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, i
     }
     {
         PhaseTimer pt("lca.check", s);
-        const bool small = n <= kCheckSmall;
-        const int64_t blocks = ceil_div(n, kCheckThreads * (small ? 1 : 4)), most = int64_t(num_sms()) * 8;
-        launch(small ? k_check_children<1> : k_check_children<4>, int(blocks < most ? blocks : most), kCheckThreads, 0, s, par, n, head, next, seen, heavy,
-               heavy_count);
+        if (n <= kSortAll) {
+            int32_t *head2 = ws.get<int32_t>(n), *next2 = ws.get<int32_t>(n);
+            if (!ws.ok()) return ETL_ENOMEM;
+            launch(k_sort_children, int(ceil_div(n, kCheckThreads)), kCheckThreads, 0, s, par, n, head, next, head2, next2,
+                   heavy, heavy_count);
+            head = head2;
+            next = next2;
+        } else {
+            const bool small = n <= kCheckSmall;
+            const int64_t blocks = ceil_div(n, kCheckThreads * (small ? 1 : 4)), most = int64_t(num_sms()) * 8;
+            launch(small ? k_check_children<1> : k_check_children<4>, int(blocks < most ? blocks : most), kCheckThreads, 0,
+                   s, par, n, head, next, seen, heavy, heavy_count);
+        }
         note_launch();
     }
     etl_status st = last_launch();
