@@ -284,15 +284,16 @@ struct Slot4d {
 };
 inline bool wide_slots(int64_t len) { return len > (int64_t(1) << 30); }
 
-// Result of ranking one list: element e's record names its sublist; T[sid].x / T[sid].y are the number
-// of elements / of even-indexed elements before that sublist's first element. So rank(e) =
-// T[sid].x + lr and evens_before(e) = T[sid].y + lo.
+// Result of ranking one list: element e's record names its sublist; first[sid], or in dual mode
+// first2[sid].x / .y, are the number of elements / of even-indexed elements before that sublist's first
+// element. So rank(e) = first + lr and evens_before(e) = first2.y + lo.
 struct RankResult {
     const void *recs;  // Slot8 records if wide; else Slot4 or, in dual mode, Slot4d ones
     bool wide;
     int lb;
-    const int4 *T;
-    int64_t rcap;  // entries of T
+    const int32_t *first;
+    const int2 *first2;
+    int64_t rcap;  // sublists
 };
 
 // rank of element e of a list ranked without dual; -1 if its record shows that it is not on the list
@@ -309,7 +310,7 @@ __device__ __forceinline__ int32_t rank_at(const RankResult &r, int64_t e) {
         sid = Slot4::sid(v, r.lb);
         lr = int32_t(Slot4::lr(v, r.lb));
     }
-    return (sid >= 0 && sid < r.rcap) ? __ldg(&r.T[sid].x) + lr : -1;
+    return (sid >= 0 && sid < r.rcap) ? __ldg(r.first + sid) + lr : -1;
 }
 
 struct RankParams {

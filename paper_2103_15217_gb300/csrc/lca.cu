@@ -160,8 +160,8 @@ __global__ void k_node_stats(RankResult rr, int32_t n, const int32_t *__restrict
 #pragma unroll
         for (int j = 0; j < kIlp; ++j)
             if (r[j].ok) {
-                A[j] = __ldg(reinterpret_cast<const int2 *>(rr.T + r[j].sa));
-                rb[j] = r[j].leaf ? 0 : __ldg(&rr.T[r[j].sb].x);
+                A[j] = __ldg(rr.first2 + r[j].sa);
+                rb[j] = r[j].leaf ? 0 : __ldg(&rr.first2[r[j].sb].x);
             }
 #pragma unroll
         for (int j = 0; j < kIlp; ++j) {

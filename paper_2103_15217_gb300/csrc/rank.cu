@@ -345,6 +345,18 @@ __global__ void k_walk(const int4 *__restrict__ T, int64_t base, const int32_t *
 
 // ------------------------------------------------------------ top level: one CTA, shared memory
 
+// The sums before an entry. They have an array of their own, 8 or 4 bytes per entry, not the first half of
+// the 16-byte entries: the top writes half the sectors, and what is gathered from it later stays small.
+template <bool DUAL>
+using Prefix = std::conditional_t<DUAL, int2, int32_t>;
+template <bool DUAL>
+__device__ __forceinline__ Prefix<DUAL> prefix(int32_t x, int32_t y) {
+    if constexpr (DUAL)
+        return make_int2(x, y);
+    else
+        return x;
+}
+
 // FROM_LIST: the list itself instead of a reduced list; each element on it becomes its own sublist in
 // the result. One SM issues all of it, so the steps are kept to a few instructions (claims as in the
 // in-place walk, tried here, took twice the time; pointer jumping over all entries three times).
@@ -352,8 +364,8 @@ constexpr int kTopBatch = 5;  // entries per thread whose loads are in flight to
 
 template <class S, bool DUAL, bool FROM_LIST>
 __global__ void __launch_bounds__(kTopThreads)
-    k_top(const uint32_t *__restrict__ succ, typename S::T *__restrict__ recs, int lb, int4 *__restrict__ T,
-          int64_t base, const int32_t *__restrict__ d_add, int64_t cap, const int32_t *__restrict__ d_head,
+    k_top(const uint32_t *__restrict__ succ, typename S::T *__restrict__ recs, int lb, const int4 *__restrict__ T,
+          Prefix<DUAL> *__restrict__ out, int64_t base, const int32_t *__restrict__ d_add, int64_t cap, const int32_t *__restrict__ d_head,
           int32_t head_value, int64_t expect_total, int32_t *__restrict__ status) {
     pdl_prologue();
     extern __shared__ int32_t sm[];
@@ -401,31 +413,32 @@ __global__ void __launch_bounds__(kTopThreads)
     __syncthreads();
     rank_in_shared<DUAL>(len, head, expect_total, sh, nx, a1, a2, status);
     for (int e = threadIdx.x; e < len; e += kTopThreads) {
-        const int32_t z = nx[e];
-        if (z >= 0) continue;  // on no walk
-        const int32_t s = z & ~kVisited, r = sh.V1[s] + a1[e], o = DUAL ? sh.V2[s] + a2[e] : 0;
-        if (FROM_LIST) {
-            T[e] = make_int4(r, o, 0, 0);
+        const int32_t z = nx[e], w = z & (kTopSub - 1);
+        const bool on = z < 0;  // on a walk
+        out[e] = prefix<DUAL>(on ? sh.V1[w] + a1[e] : 0, DUAL && on ? sh.V2[w] + a2[e] : 0);
+        if (FROM_LIST && on) {
             const bool leaf = DUAL && int32_t(succ[e]) < ETL_END;
             recs[e] = S::rec(e, 0, leaf ? 0x8000u : 0u, lb);
-        } else {
-            *reinterpret_cast<int2 *>(T + e) = make_int2(r, o);
         }
     }
 }
 
 size_t top_smem(int64_t len, bool dual) { return size_t((dual ? 3 : 2) * len) * sizeof(int32_t); }
 
-// an entry's weights give way to the prefix over the whole list
-__global__ void k_expand(int4 *__restrict__ T, const int4 *__restrict__ loc, int64_t base,
-                         const int32_t *__restrict__ d_add, int64_t cap, const int4 *__restrict__ up, int64_t up_cap) {
+// an entry's prefix over the whole list: its sublist's and that in the sublist
+template <bool DUAL>
+__global__ void k_expand(const int4 *__restrict__ loc, int64_t base, const int32_t *__restrict__ d_add, int64_t cap,
+                         const Prefix<DUAL> *__restrict__ up, int64_t up_cap, Prefix<DUAL> *__restrict__ out) {
     pdl_prologue();
     const int64_t len = level_len(base, d_add, cap);
     for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < len; e += int64_t(gridDim.x) * blockDim.x) {
         const int4 l = __ldcs(loc + e);
-        if (l.z >= 0 && l.z < up_cap) {  // entries on no walk get whatever is there
-            const int2 u = __ldg(reinterpret_cast<const int2 *>(up + l.z));
-            *reinterpret_cast<int2 *>(T + e) = make_int2(u.x + l.x, u.y + l.y);
+        if (l.z < 0 || l.z >= up_cap) continue;  // entries on no walk get whatever is there
+        if constexpr (DUAL) {
+            const int2 u = __ldg(up + l.z);
+            out[e] = make_int2(u.x + l.x, u.y + l.y);
+        } else {
+            out[e] = __ldg(up + l.z) + l.x;
         }
     }
 }
@@ -497,20 +510,27 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
     cudaFuncSetAttribute(k_top<S, DUAL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap, DUAL)));
     cudaFuncSetAttribute(k_top<S, DUAL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap, DUAL)));
     etl_status st;
+    auto set_result = [&](Prefix<DUAL> *first, int64_t cap) {
+        if constexpr (DUAL)
+            out->first2 = first;
+        else
+            out->first = first;
+        out->rcap = cap;
+    };
     if (len <= kTopCap) {
-        int4 *T = alloc.template get<int4>(len);
-        if (!T) return ETL_ENOMEM;
-        out->T = T;
-        out->rcap = len;
+        Prefix<DUAL> *first = alloc.template get<Prefix<DUAL>>(len);
+        if (!first) return ETL_ENOMEM;
+        set_result(first, len);
         PhaseTimer pt("rank.top", s);
-        launch(k_top<S, DUAL, true>, 1, kTopThreads, top_smem(len, DUAL), s, succ, static_cast<R *>(recs), out->lb, T, len,
-               nullptr, len, d_head, head, expect_len, status);
+        launch(k_top<S, DUAL, true>, 1, kTopThreads, top_smem(len, DUAL), s, succ, static_cast<R *>(recs), out->lb, nullptr,
+               first, len, nullptr, len, d_head, head, expect_len, status);
         note_launch();
         return last_launch();
     }
 
     struct Level {
         int4 *T, *loc;
+        Prefix<DUAL> *first;
         int64_t base, cap;  // entries: base + *d_add, at most cap
         const int32_t *d_add, *d_head;
     };
@@ -553,7 +573,7 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         out->lb = w.lb;
         int4 *T = alloc.template get<int4>(w.cap);
         if (!T) return ETL_ENOMEM;
-        lv[nl++] = Level{T, nullptr, w.start, w.cap, zero, words + 1};
+        lv[nl++] = Level{T, nullptr, nullptr, w.start, w.cap, zero, words + 1};
         PhaseTimer pt0("rank.walk0", s);
         launch(k_walk0_in_place<S, DUAL>, grid, P.block, 0, s, static_cast<R *>(recs), w, T, zero, words + 1, status);
         note_launch();
@@ -576,7 +596,7 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         }
         int4 *T = alloc.template get<int4>(cap);
         if (!T) return ETL_ENOMEM;
-        lv[nl++] = Level{T, nullptr, int64_t(H.S0) + 1, cap, zero, words + 1};
+        lv[nl++] = Level{T, nullptr, nullptr, int64_t(H.S0) + 1, cap, zero, words + 1};
         PhaseTimer pt0("rank.walk0", s);
         launch(k_walk0<S, DUAL>, grid_of(int64_t(H.S0) + 1, 2048 / P.block, P), P.block, 0, s, succ, len, d_head, head,
                H, static_cast<R *>(recs), out->lb, lcap, T, zero, cap, words + 1, status);
@@ -602,16 +622,18 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
             st = last_launch();
         }
         if (st) return st;
-        lv[nl] = Level{up, nullptr, 0, int64_t(most) + 1, words + 2 * nl, words + 2 * nl + 1};
+        lv[nl] = Level{up, nullptr, nullptr, 0, int64_t(most) + 1, words + 2 * nl, words + 2 * nl + 1};
         ++nl;
     }
 
+    for (int i = 0; i < nl; ++i)
+        if (!(lv[i].first = alloc.template get<Prefix<DUAL>>(lv[i].cap))) return ETL_ENOMEM;
     // ---- top
     {
         const Level &L = lv[nl - 1];
         PhaseTimer ptp("rank.top", s);
-        launch(k_top<S, DUAL, false>, 1, kTopThreads, top_smem(L.cap, DUAL), s, nullptr, nullptr, 0, L.T, L.base, L.d_add,
-               L.cap, L.d_head, 0, expect_len, status);
+        launch(k_top<S, DUAL, false>, 1, kTopThreads, top_smem(L.cap, DUAL), s, nullptr, nullptr, 0, L.T, L.first, L.base,
+               L.d_add, L.cap, L.d_head, 0, expect_len, status);
         note_launch();
         st = last_launch();
         if (st) return st;
@@ -622,13 +644,12 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         int blocks = int(ceil_div(L.cap, 256));
         if (blocks > num_sms() * 32) blocks = num_sms() * 32;  // four waves of full occupancy
         PhaseTimer pte("rank.expand", s);
-        launch(k_expand, blocks, 256, 0, s, L.T, L.loc, L.base, L.d_add, L.cap, lv[i + 1].T, lv[i + 1].cap);
+        launch(k_expand<DUAL>, blocks, 256, 0, s, L.loc, L.base, L.d_add, L.cap, lv[i + 1].first, lv[i + 1].cap, L.first);
         note_launch();
         st = last_launch();
         if (st) return st;
     }
-    out->T = lv[0].T;
-    out->rcap = lv[0].cap;
+    set_result(lv[0].first, lv[0].cap);
     return ETL_OK;
 }
 
