@@ -50,3 +50,29 @@ def test_malformed_trees(n, fault):
     out = host(h.query(dev(np.zeros(5, np.int32)), dev(np.full(5, n - 1, np.int32))))
     assert h.status() == 4          # ETL_EBADTREE
     assert (out == -1).all()
+
+
+@pytest.mark.parametrize("n", [5000, 8191, 8192, 8193])
+@pytest.mark.parametrize("grasp", [1, 5, None, "star"])
+def test_largest_trees(n, grasp):
+    test_trees(n, grasp)
+
+
+@pytest.mark.parametrize("n", [257, 258, 4096, 8192])
+@pytest.mark.parametrize("family", [31, 64, 65, 300])
+def test_families(n, family):
+    """Every node has `family` children (as long as there are labels), labels permuted."""
+    import paper_2103_15217_gb300 as etl
+    perm = np.random.default_rng(n).permutation(n)
+    parent = np.full(n, -1, np.int32)
+    parent[perm[1:]] = perm[(np.arange(1, n) - 1) // family]
+    h = etl.lca_preprocess(dev(parent))
+    pre, depth, size, _ = oracle.tree_tour(parent)
+    arr = {k: host(t) for k, t in h.arrays().items()}
+    assert h.status() == 0
+    assert (arr["pre"] == pre).all() and (arr["depth"] == depth).all() and (arr["size"] == size).all()
+
+
+@pytest.mark.parametrize("fault", ["two roots", "no root", "cycle", "past the end", "below -1", "own parent"])
+def test_malformed_largest(fault):
+    test_malformed_trees(8192, fault)
