@@ -52,19 +52,17 @@ E2E_MIN_STEPS = 60  # steps of the end-to-end measurement (at least --steps)
 # algorithmic bytes per unit for each phase (what the method must read and write
 # once: int32 = 4 B); keys are (phase, part) where part is "tree" or "graph"
 ALGO = {
-    ("rank.walk0", "tree"): ("arc", 12),       # read succ 4, write (sublist, offsets) 8
+    ("rank.walk0", "tree"): ("arc", 12),       # read succ 4, write (sublist, offsets) 8 (in place: 4-byte slots, 8)
     ("rank.walk0", "graph"): ("arc", 12),
     ("rmq.level_min", "tree"): ("node", 8),    # read level l-1, write level l
     ("rmq.level_min", "graph"): ("pos", 8),
     ("rmq.level_max", "graph"): ("pos", 8),
     ("lca.query", "tree"): ("query", 32),      # u, v 8; pre of both 8; the two range entries 8; order 4; out 4
-    ("lca.succ", "tree"): ("node", 16),        # child offsets 8, grouped child 4, successor 4 (per node)
+    ("lca.link", "tree"): ("node", 16),        # parent 4, the list's head exchanged 8, link 4
+    ("lca.succ", "tree"): ("node", 20),        # parent, first child, next sibling 12, both successors 8
     ("lca.node_rec", "tree"): ("node", 24),    # pre 4, size 4, (pm, sm) 8, record 8 of it used
-    ("rmq.blocks", "tree"): ("node", 12),      # read Q, write pm and sm
-    ("sort.scatter", "tree"): ("node", 16),    # read key, value; write key, value
-    ("sort.scatter", "graph"): ("arc", 16),
-    ("lca.node_stats", "tree"): ("node", 32),  # 2 records 16, write pre/depth/size 12, order 4
-    ("lca.parent_pre", "tree"): ("node", 16),  # parent 4, pre 4, pre[parent] 4, Q 4
+    ("lca.node_stats", "tree"): ("node", 28),  # 2 records 8, next sibling 4, write pre/depth/size 12, order 4
+    ("lca.parent_pre", "tree"): ("node", 20),  # order 8, Q 4, write pm and sm 8
     ("br.hook", "graph"): ("edge", 17),        # edge 8, flag 1, two root lookups 8
     ("br.lowhigh_prep", "graph"): ("edge", 24),
 }
@@ -441,13 +439,13 @@ def run_ours(args):
 
 
 def random_access_ceiling(etl, dev, flush, n=1 << 25, reps=5):
-    """A measured ceiling for the ranking walk. The probe kernel performs the walk's accesses (a
-    random 4-byte successor read and an 8-byte record write at the same index) for every element of
-    a random permutation of 2^25 elements, all independent of one another; the library's ranker then
-    ranks the list that visits the elements in that same order, where each step's read depends on the
-    previous one. Both run with 512 MB flushed from L2 before each launch; the fraction is the probe's
-    time over the level-0 walk's (k_walk0) time on the same list: the same elements, the same random
-    addresses."""
+    """A measured mark for the ranking walk: a random 4-byte successor read and an 8-byte record write
+    at the same index for every element of a random permutation of 2^25 elements, all independent of one
+    another. The library's ranker then ranks the list that visits the elements in that same order, where
+    each step depends on the previous one. Both run with 512 MB flushed from L2 before each launch; the
+    fraction is the probe's time over the level-0 walk's on the same list: the same elements, the same
+    random addresses. A walk in place (one exchange per element instead of a read and a write in two
+    arrays) exceeds 1."""
     import torch
     order = torch.randperm(n, device=dev, dtype=torch.int32)
     succ = torch.empty(n, dtype=torch.int32, device=dev)

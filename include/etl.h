@@ -280,9 +280,9 @@ etl_status find_bridges(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
  *   ETL_TUNE_RANK_BLOCKS_PER_SM  resident walk blocks per SM on lists ranked
  *                           in place, block * value <= 2048 (10; two thirds of
  *                           it on those whose slots fit L2)
- *   ETL_TUNE_RMQ_LEVELS_PER_PASS sparse-table levels built per streaming
- *                           pass, 1..3 (3)
- *   ETL_TUNE_RMQ_BLOCK      threads per block of the sparse-table build,
+ *   ETL_TUNE_RMQ_LEVELS_PER_PASS levels of a full sparse table built per
+ *                           streaming pass, 1..3 (3)
+ *   ETL_TUNE_RMQ_BLOCK      threads per block of the full sparse table's build,
  *                           128, 256, 512 or 1024 (256)
  *   ETL_TUNE_CC_FIRST_SLICE edges hooked before the first compression of the
  *                           connected-components pass, in units of n/4,
@@ -296,9 +296,10 @@ etl_status find_bridges(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
  *                           O(n) memory); 0: full sparse tables (n log n
  *                           entries). Both answer every query exactly. (1)
  *                           Read when a handle or a bridge call is built.
- *   ETL_TUNE_SORT_ROUNDS    32-element rounds per warp in the radix-sort
- *                           passes that group children by parent: tiles of
- *                           256 * value elements, value 8 or 16 (8)
+ *   ETL_TUNE_SORT_ROUNDS    32-element rounds per warp in the radix sort of
+ *                           families of more than 32 children that are out of
+ *                           label order: tiles of 256 * value elements, value
+ *                           8 or 16 (8)
  *   ETL_TUNE_CC_DOUBLING    1: after the first slice the connected-components
  *                           pass hooks the edges in slices that double in
  *                           size, compressing the forest before each; 0: the
@@ -307,8 +308,8 @@ etl_status find_bridges(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
  *                           of a sample (the giant component's) outranks all
  *                           others when roots are hooked, so it never moves;
  *                           0: plain smaller-id order (1)
- *   ETL_TUNE_SORT_BALLOT    1: the radix scatter finds the lanes holding the
- *                           same digit with eight warp ballots; 0: with
+ *   ETL_TUNE_SORT_BALLOT    1: that sort finds the lanes holding the same
+ *                           digit with eight warp ballots; 0: with
  *                           __match_any_sync (1)
  *   ETL_TUNE_PDL            1: the library's kernels are launched with
  *                           programmatic dependent launch, so each one is

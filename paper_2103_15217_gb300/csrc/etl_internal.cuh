@@ -200,10 +200,8 @@ __device__ __forceinline__ int32_t last_at_or_before(const int32_t *__restrict__
 
 // ----------------------------------------------------------------- primitives
 
-// Exclusive scan of in[0..n) into out[0..n], out[n] = total. If d_n is not
-// null, only in[0..*d_n) is read (the rest counts as 0); n is the capacity.
+// Exclusive scan of in[0..n) into out[0..n], out[n] = total.
 etl_status scan_exclusive_i32(const int32_t *in, int32_t *out, int64_t n, Workspace &ws);
-etl_status scan_exclusive_u8(const uint8_t *in, int32_t *out, int64_t n, Workspace &ws);
 
 // Children of every node in ascending label order: head[v] = first child or -1, next[c] = next sibling
 // or -1 (-1 for roots too). parent: ids in [0, n), -1 at roots; anything else is dropped and sets the
@@ -470,7 +468,7 @@ struct etl_lca_s {
     int64_t ld = 0;             // row length of the sparse table
     int32_t *table = nullptr;   // levels * ld (full sparse table) or the blocked table's allocation
     bool blocked = false;       // table is a blocked two-level table (layout `bl`)
-    void *nrec = nullptr;       // blocked table: per node (pre, pm[pre], sm[pre + 1], 0), int4[n]
+    void *nrec = nullptr;       // blocked table: per node (pre, pm[pre], sm[pre], size), int4[n]
     etl::BlockedLayout bl{};
     int32_t *status = nullptr;  // device status word
     bool has_table = false;     // RMQ sparse table built (lca_query available)

@@ -3,7 +3,7 @@
 The knobs change no result, only speed (``etl_tune_set``): the list ranker's
 splitter densities and walk-kernel shape (threads per block and resident
 blocks per SM of the walks over lists larger than L2), the range tables'
-form and build shape, the radix passes' tile size and ranking, and the
+form and build shape, tile size and ranking of the sort of long families, the
 connectivity pass's hooking schedule, and whether kernels are launched as
 programmatic dependents of the one before. ``autotune`` times candidate settings
 with CUDA events on the caller's own work -- a callable that enqueues one
