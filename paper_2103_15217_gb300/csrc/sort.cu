@@ -15,6 +15,7 @@
 //    there are none (3 us). Inside a tile each warp ranks its 32-element rounds (peers with the same
 //    digit by __match_any_sync or by eight ballots) with per-warp smem counters; the ranked tile is
 //    staged in shared memory in digit order and written out in runs.
+#include <algorithm>
 #include <climits>
 
 #include "etl_internal.cuh"
@@ -29,17 +30,29 @@ constexpr int kLinkThreads = 256;
 constexpr int kLinkIlp = 2;  // labels per thread, from the highest down (1: 0.16 ms, 4: more siblings in flight together)
 constexpr int kLight = 32;   // children of a family that one thread sorts
 
+// Batches: blocks that run together take tiles of different parts of the list, each part from its end down, so
+// that fewer siblings are pushed at one time. A part's ends cut through a tree, whose halves come in the wrong
+// order, so a part holds at least 8 trees. 512 trees of 2^24 nodes in all, the check of the order: 174 us as
+// one part, 136 as 8, 118 to 121 as 16 to 48, 131 as 64, 156 as 128; the pushes take the same time.
+constexpr int kLinkGroups = 32;
+
 // off / k / bad (batches): ids are local to the node's instance, gparent receives global ones. A block
 // looks up the instances of its first and last label, a thread its own between the two.
 template <bool BATCH>
 __global__ void __launch_bounds__(kLinkThreads)
-    k_link_children(const int32_t *__restrict__ parent, int32_t n, const int32_t *__restrict__ off,
+    k_link_children(const int32_t *__restrict__ parent, int32_t n, int32_t groups, const int32_t *__restrict__ off,
                     int32_t k, const int32_t *__restrict__ bad, int32_t *__restrict__ gparent, int32_t *__restrict__ head,
                     int32_t *__restrict__ next, int32_t *__restrict__ root_cnt, int32_t *__restrict__ root_of,
                     int32_t *__restrict__ status) {
     pdl_prologue();
     const bool bad_offsets = BATCH && *bad;
-    const int64_t top = int64_t(gridDim.x - blockIdx.x) * (kLinkThreads * kLinkIlp);
+    int64_t tile = gridDim.x - 1 - blockIdx.x;
+    if (BATCH) {
+        const uint32_t each = gridDim.x / groups;
+        tile = int64_t(blockIdx.x % groups) * each + (each - 1 - blockIdx.x / groups);
+    }
+    const int64_t top = (tile + 1) * (kLinkThreads * kLinkIlp);
+    if (BATCH && tile * (kLinkThreads * kLinkIlp) >= n) return;
     __shared__ int32_t span[2];
     if (BATCH) {
         if (threadIdx.x < 2 && !bad_offsets)
@@ -437,8 +450,10 @@ etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, i
     const int32_t *par = off ? gparent : parent;
     {
         PhaseTimer pt("lca.link", s);
-        const int blocks = int(ceil_div(n, kLinkThreads * kLinkIlp));
-        launch(off ? k_link_children<true> : k_link_children<false>, blocks, kLinkThreads, 0, s, parent, n, off, k,
+        const int64_t tiles = ceil_div(n, kLinkThreads * kLinkIlp);
+        const int groups = off ? std::max(1, std::min(k / 8, kLinkGroups)) : 1;
+        const int blocks = int(ceil_div(tiles, groups) * groups);
+        launch(off ? k_link_children<true> : k_link_children<false>, blocks, kLinkThreads, 0, s, parent, n, groups, off, k,
                bad, gparent, head, next, root_cnt, root_of, status);
         note_launch();
     }

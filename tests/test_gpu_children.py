@@ -56,3 +56,19 @@ def test_hub_batches(rounds, ballot):
 @pytest.mark.parametrize("hubs", [30, 8000, 1 << 17])
 def test_where_families_change_hands(n, hubs):
     test_hub_trees(n, hubs)
+
+
+@pytest.mark.parametrize("k", [16, 41, 300])
+def test_batches_pushed_in_parts(k):
+    """From 16 trees on the labels are pushed in several parts of the list at a time."""
+    import paper_2103_15217_gb300 as etl
+    rng = np.random.default_rng(k)
+    sizes = rng.integers(1, 3000, k)
+    sizes[k // 2] = 40000
+    trees = [hub_tree(int(n), int(rng.integers(1, 400)), i) for i, n in enumerate(sizes)]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    h = etl.lca_preprocess_batch(dev(np.concatenate(trees)), dev(off), int(sizes.max()))
+    got = host(h.arrays()["pre"])
+    assert h.status() == 0
+    for i, t in enumerate(trees):
+        assert (got[off[i]:off[i + 1]] - off[i] == oracle.tree_tour(t)[0]).all()
