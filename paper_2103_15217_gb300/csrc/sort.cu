@@ -111,10 +111,9 @@ __global__ void __launch_bounds__(kLinkThreads)
 // Every link must ascend. The first to see one of a family that does not takes the family (its bit in
 // `seen`) and puts it on its block's list; the block sorts those together (one thread each), so that
 // the few walks do not hold up warps that are checking: 2^24 nodes of a random tree 0.19 -> 0.06 ms.
-// Threads that check may read links being rewritten; whatever they see, they find the bit set. On a
-// smaller tree many families have to be sorted, by as many blocks as there are (ILP 1).
+// Threads that check may read links being rewritten; whatever they see, they find the bit set.
 constexpr int kCheckThreads = 256;
-constexpr int64_t kCheckSmall = int64_t(1) << 19;
+constexpr int kCheckIlp = 4;
 
 __device__ void sort_family(int32_t p, int32_t n, int32_t *head, int32_t *next, uint32_t *heavy, int32_t *heavy_count) {
     int32_t kids[kLight];
@@ -135,26 +134,25 @@ __device__ void sort_family(int32_t p, int32_t n, int32_t *head, int32_t *next, 
     for (int i = 0; i < k; ++i) next[kids[i]] = i + 1 < k ? kids[i + 1] : -1;
 }
 
-template <int ILP>
 __global__ void __launch_bounds__(kCheckThreads)
     k_check_children(const int32_t *__restrict__ par, int32_t n, int32_t *head, int32_t *next,
                      uint32_t *__restrict__ seen, uint32_t *__restrict__ heavy, int32_t *__restrict__ heavy_count) {
     pdl_prologue();
-    constexpr int kTile = kCheckThreads * ILP;
+    constexpr int kTile = kCheckThreads * kCheckIlp;
     __shared__ int32_t todo[2 * kTile];
     __shared__ int count;
     if (threadIdx.x == 0) count = 0;
     __syncthreads();
     const int64_t step = int64_t(gridDim.x) * kTile;
     for (int64_t base = int64_t(blockIdx.x) * kTile; base < n; base += step) {
-        int32_t x[ILP];
+        int32_t x[kCheckIlp];
 #pragma unroll
-        for (int j = 0; j < ILP; ++j) {
+        for (int j = 0; j < kCheckIlp; ++j) {
             const int64_t t = base + j * kCheckThreads + threadIdx.x;
             x[j] = t < n ? __ldcg(next + t) : -1;
         }
 #pragma unroll
-        for (int j = 0; j < ILP; ++j) {
+        for (int j = 0; j < kCheckIlp; ++j) {
             const int64_t t = base + j * kCheckThreads + threadIdx.x;
             if (x[j] < 0 || x[j] > t) continue;
             const int32_t p = par[t];
@@ -177,9 +175,10 @@ __global__ void __launch_bounds__(kCheckThreads)
 // label is its next sibling, and the least of all the first child. No marks, no second stage, and no
 // insertions one after another. Results go to arrays of their own, so that nothing read changes (and L1
 // serves the walks of siblings). Bound by the latency of the longest list: random tree of 2^16 nodes 8.7 us
-// (k_check_children 18.3), of 2^18 11 (20), families of 30 27 (62); a path, which has nothing to sort, 8.6
-// (6.2). Beyond, the work grows with the squares of the families: 2^20 random 23 (23), families of 30 119 (61).
-constexpr int32_t kSortAll = 1 << 18;
+// (k_check_children 18.3), of 2^18 11 (20), of 2^19 14 (22), families of 30 27 and 58 (62, 72); a path, which
+// has nothing to sort, 8.6 and 10.4 (6.2, 6.0). Beyond, the work grows with the squares of the families: 2^20
+// random 23 (23), families of 30 119 (61).
+constexpr int32_t kSortAll = 1 << 19;
 
 __global__ void __launch_bounds__(kCheckThreads)
     k_sort_children(const int32_t *__restrict__ par, int32_t n, const int32_t *__restrict__ head,
@@ -467,10 +466,9 @@ etl_status link_children(const int32_t *parent, int32_t n, const int32_t *off, i
             head = head2;
             next = next2;
         } else {
-            const bool small = n <= kCheckSmall;
-            const int64_t blocks = ceil_div(n, kCheckThreads * (small ? 1 : 4)), most = int64_t(num_sms()) * 8;
-            launch(small ? k_check_children<1> : k_check_children<4>, int(blocks < most ? blocks : most), kCheckThreads, 0,
-                   s, par, n, head, next, seen, heavy, heavy_count);
+            const int64_t blocks = ceil_div(n, kCheckThreads * kCheckIlp), most = int64_t(num_sms()) * 8;
+            launch(k_check_children, int(blocks < most ? blocks : most), kCheckThreads, 0, s, par, n, head, next, seen, heavy,
+                   heavy_count);
         }
         note_launch();
     }

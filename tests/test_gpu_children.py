@@ -52,7 +52,7 @@ def test_hub_batches(rounds, ballot):
         etl.tune_set(sort_rounds=old["sort_rounds"], sort_ballot=old["sort_ballot"])
 
 
-@pytest.mark.parametrize("n", [(1 << 18) - 1, 1 << 18, (1 << 18) + 1])
+@pytest.mark.parametrize("n", [(1 << 18) - 1, 1 << 18, (1 << 18) + 1, (1 << 19) - 1, 1 << 19, (1 << 19) + 1])
 @pytest.mark.parametrize("hubs", [30, 8000, 1 << 17])
 def test_where_families_change_hands(n, hubs):
     test_hub_trees(n, hubs)
