@@ -1,4 +1,4 @@
-// Device-wide exclusive prefix sums (reduce-then-scan) over tour positions (Inlabel's path heads, the
+// Device-wide exclusive prefix sums (reduce-then-scan) over preorder or tour positions (Inlabel, the
 // hybrid method's levels). Loads are warp-striped, so every warp-wide load touches one contiguous
 // 128-byte line.
 #include "etl_internal.cuh"
