@@ -307,7 +307,7 @@ etl_status find_bridges(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
  *   ETL_TUNE_CC_GIANT       1: after each compression the most frequent root
  *                           of a sample (the giant component's) outranks all
  *                           others when roots are hooked, so it never moves;
- *                           0: plain smaller-id order (1)
+ *                           0: the fixed order of the mixed ids (1)
  *   ETL_TUNE_SORT_BALLOT    1: that sort finds the lanes holding the same
  *                           digit with eight warp ballots; 0: with
  *                           __match_any_sync (1)

@@ -2,8 +2,8 @@
 //
 // Phase 1, spanning forest: a lock-free hook-and-compress connected-components
 //   pass in the style the paper takes from Jaiganesh and Burtscher: every edge
-//   finds the roots of its two ends (with path halving) and hooks the larger
-//   root under the smaller one with a CAS. A CAS that succeeds joins two
+//   finds the roots of its two ends (with path halving) and hooks the one of
+//   lower priority under the other with a CAS. A CAS that succeeds joins two
 //   different trees, so its edge is a forest edge; exactly n - c succeed.
 //   The successful edges are appended to the forest's list as they are found.
 // Phase 2, Euler tour of the forest (Sec. 2.1): forest edge t owns half-edges
@@ -110,14 +110,27 @@ __device__ __forceinline__ int64_t hook_chunk(int64_t c, int64_t nsuper, bool sp
     return spread ? ((c / kHookSuper) * kP % nsuper) * kHookSuper + c % kHookSuper : c;
 }
 
-// Roots are hooked under roots of higher priority: a smaller id, except that the root named by
-// *giant (if any: the most frequent root after a compression, i.e. the giant component's) ranks above
-// all. Priorities are a strict total order, so the forest stays acyclic, and the giant root never
-// moves: once the giant component has formed, every later hook leaves the paths of its members as
-// they are (with plain smaller-id order the giant root moves whenever a smaller one joins, and every
-// member's path grows by a step).
+// Roots are hooked under roots of higher priority. Priorities are a strict total order, so the forest stays
+// acyclic. The root named by *giant (if any: the most frequent root after a compression, i.e. the giant
+// component's) ranks above all, so it never moves: once the giant component has formed, every later hook
+// leaves the paths of its members as they are (with a fixed order its root moves whenever a higher one joins,
+// and every member's path grows by a step). The others are ordered by a mixed id (MurmurHash3's 32-bit
+// finalizer, a bijection), or, where the component's label is to be its smallest vertex (BY_ID), by the id.
+// By ids a path whose vertices are numbered along it is hooked into one chain, and an edge that comes late
+// climbs it alone, 0.5 us for two steps. Whole calls, us, by ids and now: paths in order of 2^17 vertices 1170
+// to 2640 and 111, of 2^20 31700 and 254 (from their end 27700 and 257), a cycle of 2^14 4120 and 57. On the
+// easy graph of 2^22 vertices, whose labels are permuted, 1433 and 1442, on the hard one 1234 and 1196.
+template <bool BY_ID>
+__device__ __forceinline__ uint32_t hook_key(int32_t v) {
+    uint32_t h = uint32_t(v);
+    if (BY_ID) return h;
+    h = (h ^ (h >> 16)) * 0x85ebca6bu;
+    h = (h ^ (h >> 13)) * 0xc2b2ae35u;
+    return h ^ (h >> 16);
+}
+template <bool BY_ID>
 __device__ __forceinline__ bool hook_above(int32_t a, int32_t b, int32_t giant) {  // a ranks above b
-    return a == giant || (b != giant && a < b);
+    return a == giant || (b != giant && hook_key<BY_ID>(a) < hook_key<BY_ID>(b));
 }
 
 // Most edges join two vertices that already point at the same node; those cost two loads, all of a
@@ -134,6 +147,7 @@ __device__ __forceinline__ bool hook_above(int32_t a, int32_t b, int32_t giant) 
 // 588 -> 456); the two loads per edge of its 31.4M later edges alone take 210 us.
 // skip (may be null): edges to leave out; is_tree (may be null): 1 for edges whose hook succeeded, and
 // then is_bridge is cleared and forest_count, tuv (both ends of forest edge t) and tedge (its edge) are written too
+template <bool BY_ID>
 __global__ void __launch_bounds__(kHookChunk)
     k_hook(const int32_t *__restrict__ edges, bool aligned, int64_t m, int64_t c0, int64_t c1, int ilp, bool spread,
            int32_t n, int32_t *__restrict__ par, uint8_t *__restrict__ is_tree, uint8_t *__restrict__ is_bridge,
@@ -143,7 +157,7 @@ __global__ void __launch_bounds__(kHookChunk)
     __shared__ int32_t qa[kHookChunk * (kHookIlp + 1)], qb[kHookChunk * (kHookIlp + 1)], qe[kHookChunk * (kHookIlp + 1)];
     __shared__ int queued, wins[kHookChunk / 32], first;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int32_t giant = d_giant ? *d_giant : 0;  // vertex 0 ranks above all by its id
+    const int32_t giant = d_giant ? *d_giant : 0;  // vertex 0 ranks above all by its id, and by its key
     const int64_t nsuper = ((m + kHookChunk - 1) / kHookChunk + kHookSuper - 1) / kHookSuper;
     if (threadIdx.x == 0) queued = 0;
     __syncthreads();
@@ -205,7 +219,7 @@ __global__ void __launch_bounds__(kHookChunk)
                     a = ga;
                     b = gb;
                     if ((ga != pa && ga != giant) || (gb != pb && gb != giant)) continue;
-                    const bool a_up = hook_above(a, b, giant);
+                    const bool a_up = hook_above<BY_ID>(a, b, giant);
                     const int32_t hi = a_up ? b : a, lo = a_up ? a : b;  // hi goes under lo
                     if (atomicCAS(par + hi, hi, lo) == hi) {
                         won = true;
@@ -668,7 +682,7 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
                     note_launch();
                 }
             }
-            launch(k_hook, hook_grid(c1 - c0), kHookChunk, 0, s, edges, aligned, m, c0, c1,
+            launch(k_hook<false>, hook_grid(c1 - c0), kHookChunk, 0, s, edges, aligned, m, c0, c1,
                    hook_ilp(c1 - c0), spread, n, par, is_tree, is_bridge, nullptr, (c0 > 0 && C.giant) ? giant : nullptr, forest,
                    tuv, tedge, st);
             note_launch();
@@ -849,7 +863,7 @@ extern "C" etl_status two_edge_cc(const int32_t *edges, int64_t m, int32_t n, in
     launch(k_iota, gn, 256, 0, s, n, label);
     note_launch();
     if (m > 0) {  // connected components of the graph without its bridges; labels = smallest vertex
-        launch(k_hook, hook_grid(hook_positions(m)), kHookChunk, 0, s, edges, edges_aligned(edges), m, 0,
+        launch(k_hook<true>, hook_grid(hook_positions(m)), kHookChunk, 0, s, edges, edges_aligned(edges), m, 0,
                hook_positions(m), hook_ilp(hook_positions(m)), false, n, label, nullptr,
                nullptr, is_bridge, nullptr, nullptr, nullptr, nullptr, st);
         note_launch();
