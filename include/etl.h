@@ -288,8 +288,8 @@ etl_status find_bridges(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
  *                           connected-components pass, in units of n/4,
  *                           1..64 (2, i.e. n/2 edges: a random sample of that
  *                           size is still below the giant-component threshold;
- *                           half as many again up to 2^17 vertices, and one
- *                           launch without a slice up to 49152 edges)
+ *                           half as many again up to 2^18 vertices, and one
+ *                           launch without a slice up to 700 sqrt(n) edges)
  *   ETL_TUNE_RMQ_BLOCKED    1: range-min / max tables are blocked two-level
  *                           tables (prefix / suffix results inside blocks of
  *                           32 entries plus a sparse table over the blocks,

@@ -91,13 +91,18 @@ __device__ __forceinline__ int32_t find_root(int32_t *par, int32_t x, int64_t &b
 // contiguous order, which measured faster on it (0.7 against 1.3 ms on 2^25 shuffled edges).
 constexpr int kHookChunk = 256;
 constexpr int kHookIlp = 4;
-// Hook launches, us (random graphs; hard ones, of long paths, in brackets). Up to kHookAtOnce edges go in one
-// launch: 32770 edges on 16385 vertices 27 against 30 in two (20, 34), 32768 on 8192 33 against 29 (21, 32),
-// 65536 on 8192 72 against 31, on 16385 50 against 31 (22, 35). Half as many edges again in the first slice
-// up to kHookMoreFirst vertices: 2^15.3 vertices, 4 edges each 59 -> 38, 2^17 77 -> 59 (57 -> 53), 2^18
-// 74 -> 78, 2^20 123 -> 175; there the slice itself is the dearer part.
-constexpr int64_t kHookAtOnce = 49152;
-constexpr int32_t kHookMoreFirst = 1 << 17;
+// All edges go in one launch while their number is at most 700 sqrt(vertices), else a first slice, a compression
+// and the rest. One launch saves two others and the walk over all vertices between them; with more edges the
+// walks that meet no compressed path cost more. Hook launches of random graphs, us, in one and in slices, and
+// where the two are equal: 1025 vertices, 16 edges each 17 and 25, 32 32 and 30, equal at some 25000 edges; 4097,
+// 8 20 and 27, 16 29 and 28, 60000; 16385, 4 20 and 30, 8 29 and 31, 136000; 32769, 4 28 and 32, 8 54 and 36,
+// 160000; 65537, 2 24 and 35, 4 50 and 37, 180000; 92682, 2 31 and 37, 4 67 and 38, 250000. The line stays
+// below; hard graphs (long paths) gain from one launch at all of these sizes (16385, 4 each 20 and 34).
+// Half as many edges again in the first slice up to kHookMoreFirst vertices: 4 edges each on 2^15.3 vertices 42
+// -> 33, 2^17 63 -> 45 (hard 51 -> 49), 2^18 67 -> 63 (68 -> 65), 2^19 89 -> 92, 2^20 122 -> 144 (132 -> 134);
+// there the slice itself is the dearer part.
+inline bool hook_at_once(int64_t n, int64_t m) { return m * m <= 490000 * n; }
+constexpr int32_t kHookMoreFirst = 1 << 18;
 constexpr int kHookSuper = 32;
 
 // number of positions of the chunk sequence over m edges (whole superchunks)
@@ -666,7 +671,7 @@ etl_status bridges_core(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
         const int64_t nchunks = hook_positions(m);
         int64_t slice = int64_t(C.first_slice_quarters) * n / 4;
         if (n <= kHookMoreFirst) slice += slice / 2;
-        int64_t w = m <= kHookAtOnce ? nchunks : ceil_div(slice > 0 ? slice : 1, kHookChunk);  // chunks in the current slice
+        int64_t w = hook_at_once(n, m) ? nchunks : ceil_div(slice > 0 ? slice : 1, kHookChunk);  // chunks in the current slice
         PhaseTimer pt("br.hook", s);
         for (int64_t c0 = 0; c0 < nchunks;) {
             const int64_t c1 = (C.doubling || c0 == 0) ? (c0 + w < nchunks ? c0 + w : nchunks) : nchunks;
