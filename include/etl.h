@@ -67,6 +67,8 @@ const char *etl_status_string(int32_t status);
  * `status` (device int32, may be NULL) receives ETL_EBADTREE and the ranks of
  * the unreachable elements are unspecified. This is the ruling-set ranker
  * that the tree and bridge paths use internally, exposed for reuse.
+ * rank may be succ itself or overlap it in any other way (the successors in
+ * the shared part are then lost).
  * len in [1, 2^31 - 2]; head in [0, len).
  */
 etl_status etl_list_rank(const int32_t *succ, int64_t len, int32_t head, int32_t *rank, int32_t *status,

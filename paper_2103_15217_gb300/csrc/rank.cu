@@ -653,14 +653,16 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
     return ETL_OK;
 }
 
-// The records take the place of the ranks, unless the caller's two arrays overlap.
+// The records take the place of the ranks, unless the caller's two arrays overlap: then records apart from the
+// successors would overwrite them, and slots made from them in parallel would overwrite those of other threads
+// (but not where rank is succ itself, when a thread writes only over what it has read).
 template <class A>
 etl_status rank_plain_list(const int32_t *succ, int64_t len, int32_t head, int32_t *rank, int32_t *status,
                            const RankParams &P, A &alloc, cudaStream_t s) {
     const bool wide = wide_slots(len), in_place = rank_form(len, false) != RankForm::kSeparate;
-    const bool overlap = succ < rank + len && rank < succ + len;
+    const bool apart = succ < rank + len && rank < succ + len && !(in_place && succ == rank);
     void *recs = wide ? static_cast<void *>(alloc.template get<Slot8::T>(len))
-                      : (overlap && !in_place) ? static_cast<void *>(alloc.template get<Slot4::T>(len)) : rank;
+                      : apart ? static_cast<void *>(alloc.template get<Slot4::T>(len)) : rank;
     if (!recs) return ETL_ENOMEM;
     int blocks = int(ceil_div(len, 256));
     if (blocks > num_sms() * 16) blocks = num_sms() * 16;
