@@ -425,7 +425,10 @@ etl_status two_edge_cc(const int32_t *edges, int64_t m, int32_t n, int32_t *labe
  * graph and discarded unlaunched (nothing runs on the device and nothing is
  * allocated on it). Call it outside any stream capture on this thread.
  *   kind                      n            m_or_q
- *   ETL_WS_LIST_RANK          len          (unused)
+ *   ETL_WS_LIST_RANK          len          (unused)   enough also where rank
+ *                                                     overlaps succ; arrays apart
+ *                                                     take 4 len bytes less (up
+ *                                                     to 2^30 elements)
  *   ETL_WS_LCA_PREPROCESS     n            (unused)   includes the handle's tables
  *   ETL_WS_LCA_QUERY          n            q          always 0: lca_query,
  *                                                     lca_query_batch need no scratch

@@ -152,7 +152,8 @@ def _workspace(ws) -> tuple[int, int]:
 
 def workspace_size(kind: str, n: int, m_or_q: int = 0) -> int:
     """Bytes of caller-owned workspace a ``workspace=`` call of this kind needs (exact, for the tuning
-    parameters in force); kind is one of WS_KINDS."""
+    parameters in force; for "list_rank" as much as a C caller needs whose ranks overlap the list, 4 bytes
+    per element more than ``list_rank`` takes); kind is one of WS_KINDS."""
     b = ctypes.c_size_t(0)
     _check("etl_workspace_size", load_library().etl_workspace_size(WS_KINDS[kind], int(n), int(m_or_q),
                                                                    ctypes.byref(b)))

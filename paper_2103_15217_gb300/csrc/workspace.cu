@@ -9,7 +9,8 @@
 // addresses, the kernels that receive them are only recorded into a graph
 // that is destroyed without ever being launched, and the memset / copy helpers
 // skip their work. So the size is exact for the same sizes and tuning
-// parameters, and it cannot drift from the code that uses the memory.
+// parameters, and it cannot drift from the code that uses the memory. (List
+// ranking: exact for arrays that overlap, see etl.h.)
 #include "etl_internal.cuh"
 
 namespace etl {
@@ -68,8 +69,9 @@ extern "C" etl_status etl_workspace_size(int32_t kind, int64_t n, int64_t m_or_q
     switch (kind) {
         case ETL_WS_LIST_RANK:
             if (n < 1 || n > int64_t(INT32_MAX) - 1) return ETL_EINVAL;
+            // arrays that overlap take the most scratch: ranks one element after the list they are written over
             return measure([&](cudaStream_t s) {
-                return etl_list_rank(placeholder<const int32_t>(), n, 0, placeholder<int32_t>(), nullptr, s);
+                return etl_list_rank(placeholder<const int32_t>(), n, 0, placeholder<int32_t>() + (n > 1), nullptr, s);
             }, bytes);
         case ETL_WS_LCA_PREPROCESS:
             if (n < 1 || n > (1 << 30) - 1) return ETL_EINVAL;
