@@ -60,21 +60,25 @@ def test_shifted_ranks_without_allocation(n, shift):
 @pytest.mark.parametrize("n", [1, 1000, 15361, IN_PLACE, IN_PLACE + 1])
 @pytest.mark.parametrize("shift", [0, 1, -1000, None])
 def test_workspace_covers_every_overlap(n, shift):
-    # the reported size is enough however the arrays lie; where they overlap but are not the same it is
-    # needed to the byte (256 of it are room to align the buffer, which is aligned here)
+    # the reported size is enough however the arrays lie; where they overlap but are not the same, and the
+    # caller gives no status word, it is needed to the byte (256 of it are room to align the buffer, which is
+    # aligned here)
     import paper_2103_15217_gb300 as etl
     lib = etl.load_library()
     succ, rank, head, want = overlapping(n, n + 8 if shift is None else shift, n)
     need = etl.workspace_size("list_rank", n)
     ws = etl.new_workspace(need)
     assert ws.data_ptr() % 256 == 0
-    call = lambda size: lib.etl_list_rank_ws(pointer(succ), n, head, pointer(rank), pointer(st), pointer(ws), size, stream())
     st = etl.new_status()
+    call = lambda size, st: lib.etl_list_rank_ws(pointer(succ), n, head, pointer(rank), st, pointer(ws), size, stream())
     if shift and abs(shift) < n:
-        assert call(need - 257) == 2  # ETL_ENOMEM
+        assert call(need - 257, None) == 2  # ETL_ENOMEM
         succ, rank, head, want = overlapping(n, shift, n)
     a0 = etl.alloc_count()
-    assert call(need) == 0
+    assert call(need, None) == 0
+    assert torch.equal(rank, want)
+    succ, rank, head, want = overlapping(n, n + 8 if shift is None else shift, n + 1)
+    assert call(need, pointer(st)) == 0
     assert etl.alloc_count() == a0
     assert int(st) == 0
     assert torch.equal(rank, want)
