@@ -230,6 +230,11 @@ __device__ __forceinline__ unsigned digit_peers(int d, bool valid, int lane) {
     return valid ? peers : (1u << lane);
 }
 
+// A pass's histograms are 256 rows, one entry per block. Few blocks have many rows each, and short ones: there a
+// warp takes a row, else a block. All passes, us, by blocks and by warps: stars of 5000 nodes (3 blocks) 119 and
+// 37, 8193 (5) 70 and 35, 2^16 (32) 39 and 33, 2^18 (128) 46 and 48, 2^19 (257) 53 and 61.
+constexpr int kShortRow = 64;
+
 // all blocks of the cooperative grid; false (in every block that gets there) if the wait ran out
 __device__ bool grid_barrier(uint32_t *bar, uint32_t target, int32_t *status) {
     constexpr int kPolls = 1 << 24;  // about ten seconds
@@ -291,29 +296,48 @@ __global__ void __launch_bounds__(kThreads)
         arrivals += blocks;
         if (!grid_barrier(bar, arrivals, status)) return;
         // exclusive prefixes over the blocks, one digit's row at a time; its total goes to totals
-        for (int row = blk; row < kRadix; row += blocks) {
-            int32_t carry = 0;
-            for (int b0 = 0; b0 < blocks; b0 += kThreads) {
-                const int b = b0 + threadIdx.x;
-                int32_t *at = ghist + int64_t(row) * blocks + b;
-                const int32_t c = b < blocks ? __ldcg(at) : 0;
-                int32_t inc = c;
+        if (blocks <= kShortRow) {
+            for (int row = blk * kWarps + warp; row < kRadix; row += blocks * kWarps) {
+                int32_t carry = 0;
+                for (int b0 = 0; b0 < blocks; b0 += kWarp) {
+                    int32_t *at = ghist + int64_t(row) * blocks + b0 + lane;
+                    const int32_t c = b0 + lane < blocks ? __ldcg(at) : 0;
+                    int32_t inc = c;
 #pragma unroll
-                for (int o = 1; o < kWarp; o <<= 1) {
-                    const int32_t y = __shfl_up_sync(kFull, inc, o);
-                    if (lane >= o) inc += y;
+                    for (int o = 1; o < kWarp; o <<= 1) {
+                        const int32_t y = __shfl_up_sync(kFull, inc, o);
+                        if (lane >= o) inc += y;
+                    }
+                    if (b0 + lane < blocks) *at = carry + inc - c;
+                    carry += __shfl_sync(kFull, inc, kWarp - 1);
                 }
-                if (lane == kWarp - 1) wtot[warp] = inc;
-                __syncthreads();
-                int32_t wofs = carry;
-                for (int w = 0; w < kWarps; ++w) {
-                    if (w < warp) wofs += wtot[w];
-                    carry += wtot[w];
-                }
-                if (b < blocks) *at = wofs + inc - c;
-                __syncthreads();
+                if (lane == 0) totals[row] = carry;
             }
-            if (threadIdx.x == 0) totals[row] = carry;
+        } else {
+            for (int row = blk; row < kRadix; row += blocks) {
+                int32_t carry = 0;
+                for (int b0 = 0; b0 < blocks; b0 += kThreads) {
+                    const int b = b0 + threadIdx.x;
+                    int32_t *at = ghist + int64_t(row) * blocks + b;
+                    const int32_t c = b < blocks ? __ldcg(at) : 0;
+                    int32_t inc = c;
+#pragma unroll
+                    for (int o = 1; o < kWarp; o <<= 1) {
+                        const int32_t y = __shfl_up_sync(kFull, inc, o);
+                        if (lane >= o) inc += y;
+                    }
+                    if (lane == kWarp - 1) wtot[warp] = inc;
+                    __syncthreads();
+                    int32_t wofs = carry;
+                    for (int w = 0; w < kWarps; ++w) {
+                        if (w < warp) wofs += wtot[w];
+                        carry += wtot[w];
+                    }
+                    if (b < blocks) *at = wofs + inc - c;
+                    __syncthreads();
+                }
+                if (threadIdx.x == 0) totals[row] = carry;
+            }
         }
         arrivals += blocks;
         if (!grid_barrier(bar, arrivals, status)) return;
