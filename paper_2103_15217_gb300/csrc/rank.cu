@@ -500,6 +500,8 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
     using R = typename S::T;
     const bool in_place = rank_form(len, DUAL) != RankForm::kSeparate;
     constexpr bool kNarrow = std::is_same<S, Slot4d>::value;
+    // 4-byte slots of a tour and 8-byte ones of another list are only ever ranked in place
+    constexpr bool kApart = DUAL ? !kNarrow : std::is_same<S, Slot4>::value;
     out->wide = sizeof(R) == 8;
     out->lb = out->wide ? 16 : 12;
     if (in_place) recs = list;
@@ -507,9 +509,8 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
     if (!recs) return ETL_ENOMEM;
     out->recs = recs;
     const uint32_t *succ = static_cast<const uint32_t *>(list);
-    cudaFuncSetAttribute(k_top<S, DUAL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap, DUAL)));
     cudaFuncSetAttribute(k_top<S, DUAL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(top_smem(kTopCap, DUAL)));
-    etl_status st;
+    etl_status st = ETL_OK;
     auto set_result = [&](Prefix<DUAL> *first, int64_t cap) {
         if constexpr (DUAL)
             out->first2 = first;
@@ -517,15 +518,19 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
             out->first = first;
         out->rcap = cap;
     };
-    if (len <= kTopCap) {
-        Prefix<DUAL> *first = alloc.template get<Prefix<DUAL>>(len);
-        if (!first) return ETL_ENOMEM;
-        set_result(first, len);
-        PhaseTimer pt("rank.top", s);
-        launch(k_top<S, DUAL, true>, 1, kTopThreads, top_smem(len, DUAL), s, succ, static_cast<R *>(recs), out->lb, nullptr,
-               first, len, nullptr, len, d_head, head, expect_len, status);
-        note_launch();
-        return last_launch();
+    if constexpr (kApart) {
+        if (len <= kTopCap) {
+            cudaFuncSetAttribute(k_top<S, DUAL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(top_smem(kTopCap, DUAL)));
+            Prefix<DUAL> *first = alloc.template get<Prefix<DUAL>>(len);
+            if (!first) return ETL_ENOMEM;
+            set_result(first, len);
+            PhaseTimer pt("rank.top", s);
+            launch(k_top<S, DUAL, true>, 1, kTopThreads, top_smem(len, DUAL), s, succ, static_cast<R *>(recs), out->lb, nullptr,
+                   first, len, nullptr, len, d_head, head, expect_len, status);
+            note_launch();
+            return last_launch();
+        }
     }
 
     struct Level {
@@ -578,7 +583,7 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         launch(k_walk0_in_place<S, DUAL>, grid, P.block, 0, s, static_cast<R *>(recs), w, T, zero, words + 1, status);
         note_launch();
         st = last_launch();
-    } else {
+    } else if constexpr (kApart) {
         const int k = std::min(P.k0_log2, len > (int64_t(1) << 20) ? 4 : 3);
         Hash H;
         H.mask = uint32_t((uint64_t(1) << ceil_log2(uint64_t(len))) - 1);
@@ -602,6 +607,8 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
                H, static_cast<R *>(recs), out->lb, lcap, T, zero, cap, words + 1, status);
         note_launch();
         st = last_launch();
+    } else {
+        st = ETL_EINVAL;  // never: see kApart
     }
     if (st) return st;
 
