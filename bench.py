@@ -52,7 +52,9 @@ E2E_MIN_STEPS = 60  # steps of the end-to-end measurement (at least --steps)
 # algorithmic bytes per unit for each phase (what the method must read and write
 # once: int32 = 4 B); keys are (phase, part) where part is "tree" or "graph"
 ALGO = {
-    ("rank.walk0", "tree"): ("arc", 12),       # read succ 4, write (sublist, offsets) 8 (in place: 4-byte slots, 8)
+    ("rank.walk0_in_place", "tree"): ("arc", 8),  # 4-byte slots: exchange the successor for the record
+    ("rank.walk0_list", "graph"): ("arc", 8),  # read succ 4, write a 4-byte record
+    ("rank.walk0", "tree"): ("arc", 12),       # read succ 4, write an 8-byte record (tours of up to 2^21 nodes)
     ("rank.walk0", "graph"): ("arc", 12),
     ("rmq.level_min", "tree"): ("node", 8),    # read level l-1, write level l
     ("rmq.level_min", "graph"): ("pos", 8),
@@ -475,7 +477,7 @@ def random_access_ceiling(etl, dev, flush, n=1 << 25, reps=5):
         etl.profile_enable(True)
         etl.list_rank(succ, head)
         etl.profile_enable(False)
-        walk.append(etl.profile_read()["rank.walk0"][0] / 1e3)
+        walk.append(etl.profile_read()["rank.walk0_in_place"][0] / 1e3)
     t_walk = statistics.median(walk)
     etl.profile_reset()
     del order, succ, out
@@ -642,7 +644,7 @@ def committed_traffic(phase: str, n_trees: int, n_graphs: int):
     if any(tuned.get(k) != v for k, v in rec.get("launch_params", {}).items()):
         return None  # the capture was taken with other launch parameters
     c = rec["cases"]
-    keys = ("lca_grasp_inf", "lca_grasp_1024", "lca_grasp_1", "easy", "hard")  # one walk launch each per step
+    keys = ("lca_grasp_inf", "lca_grasp_1024", "lca_grasp_1")  # one launch each per step
     if any(k not in c for k in keys):
         return None
     return sum(c[k]["traffic_bytes"] for k in keys) / len(keys)

@@ -579,7 +579,7 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         int4 *T = alloc.template get<int4>(w.cap);
         if (!T) return ETL_ENOMEM;
         lv[nl++] = Level{T, nullptr, nullptr, w.start, w.cap, zero, words + 1};
-        PhaseTimer pt0("rank.walk0", s);
+        PhaseTimer pt0("rank.walk0_in_place", s);
         launch(k_walk0_in_place<S, DUAL>, grid, P.block, 0, s, static_cast<R *>(recs), w, T, zero, words + 1, status);
         note_launch();
         st = last_launch();
@@ -602,7 +602,7 @@ etl_status rank_impl(void *list, void *recs, int64_t len, const int32_t *d_head,
         int4 *T = alloc.template get<int4>(cap);
         if (!T) return ETL_ENOMEM;
         lv[nl++] = Level{T, nullptr, nullptr, int64_t(H.S0) + 1, cap, zero, words + 1};
-        PhaseTimer pt0("rank.walk0", s);
+        PhaseTimer pt0(DUAL ? "rank.walk0" : "rank.walk0_list", s);
         launch(k_walk0<S, DUAL>, grid_of(int64_t(H.S0) + 1, 2048 / P.block, P), P.block, 0, s, succ, len, d_head, head,
                H, static_cast<R *>(recs), out->lb, lcap, T, zero, cap, words + 1, status);
         note_launch();
