@@ -270,9 +270,10 @@ etl_status find_bridges(const int32_t *edges, int64_t m, int32_t n, uint8_t *is_
  * (paper_2103_15217_gb300/tune.py). Process-wide; set them between calls,
  * not while calls are being enqueued from another thread.
  *   ETL_TUNE_RANK_K0_LOG2   level-0 density of the list ranker, k in [1, 8]
- *                           (default 5): lists ranked in place (longer than
- *                           L2 holds) start one walk per 2^(k+1) elements at
- *                           most; shorter ones (bound by the latency of their
+ *                           (default 5): lists ranked in place (tours of
+ *                           more than 2^22 brackets, others of more than
+ *                           12,582,912 elements) start one walk per 2^(k+1)
+ *                           elements at most; shorter ones (bound by the latency of their
  *                           longest sublist) take one splitter in 8 elements
  *                           up to 2^20, one in 16 beyond, or one in 2^k where
  *                           that is denser

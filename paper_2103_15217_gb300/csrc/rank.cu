@@ -5,13 +5,14 @@
 //
 //  * Level 0 cuts the list into sublists, walks them and leaves a record
 //    (sublist id, local offset) per element. It has two forms:
-//    - k_walk0, for lists whose successors and records fit in L2: sublists
-//      start at splitters picked by a multiplicative hash of the element
-//      index, e is one iff (e * M mod 2^b) < S0; the hashed value is the
-//      sublist's id. A step is one dependent load, 0.25 us, and the walks are
+//    - k_walk0, for tours of up to 2^22 brackets and other lists whose
+//      successors and records fit in L2: sublists start at splitters picked
+//      by a multiplicative hash of the element index, e is one iff
+//      (e * M mod 2^b) < S0; the hashed value is the sublist's id. A step is one dependent load, 0.25 us, and the walks are
 //      bound by the longest sublist, about len / S0 * ln S0 steps.
-//    - k_walk0_in_place, for longer ones, which are bound by memory: element
-//      and record share one slot, and a step is ONE atomic exchange, which
+//    - k_walk0_in_place, for longer ones, which are bound by memory (tours by
+//      the rate of L2 first, of DRAM from some 2^25 brackets on): element and
+//      record share one slot, and a step is ONE atomic exchange, which
 //      stores the record and returns the successor. Reading the successor in
 //      one array and writing the record in another touches two sectors per
 //      element over three times the memory: 2^25 random elements take 1.65 ms
@@ -288,7 +289,8 @@ __global__ void k_walk0_in_place(typename S::T *__restrict__ slots, Walk0 W, int
 // Entry of a reduced list: x, y = the sublist's weights, z = the id of the next sublist (kEndT: none).
 // The hash covers the entries there are (the device knows how many); one in 2^k_log2 is a splitter, and
 // never more than `most`. One 16-byte load per step, 0.25 us; an entry's place (sublist, offsets) goes to
-// loc. (Replacing the entry by it would put a load and a store on one sector.)
+// loc. (Replacing the entry by it would put a load and a store on one sector.) A walk is as long as its
+// sublist: nothing cuts it short, and nothing has to, as the sums are 32 bits wide.
 __global__ void k_walk(const int4 *__restrict__ T, int64_t base, const int32_t *__restrict__ d_add, int64_t cap,
                        const int32_t *__restrict__ d_head, int k_log2, uint32_t most, int4 *__restrict__ loc,
                        int4 *__restrict__ up, int32_t *__restrict__ up_len, int32_t *__restrict__ next_head,
