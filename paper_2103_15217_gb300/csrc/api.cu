@@ -1,4 +1,7 @@
 // Shared host helpers: memory, tuning parameters, status names.
+#include <cuda.h>
+
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -24,6 +27,33 @@ int num_sms() {
         cached[dev] = v;
     }
     return cached[dev];
+}
+
+// The driver's functions are reached through the runtime (no link against libcuda); a driver without them has
+// no green contexts.
+int stream_sms(cudaStream_t s) {
+    using GetCtx = CUresult (*)(CUstream, CUgreenCtx *);
+    using GetResource = CUresult (*)(CUgreenCtx, CUdevResource *, CUdevResourceType);
+    static GetCtx get_ctx = nullptr;
+    static GetResource get_resource = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        auto entry = [](const char *name) -> void * {
+            void *f = nullptr;
+            cudaDriverEntryPointQueryResult q;
+            const bool ok = cudaGetDriverEntryPointByVersion(name, &f, CUDA_VERSION, cudaEnableDefault, &q) == cudaSuccess;
+            return ok && q == cudaDriverEntryPointSuccess ? f : nullptr;
+        };
+        get_ctx = reinterpret_cast<GetCtx>(entry("cuStreamGetGreenCtx"));
+        get_resource = reinterpret_cast<GetResource>(entry("cuGreenCtxGetDevResource"));
+        cudaGetLastError();
+    });
+    const int all = num_sms();
+    CUgreenCtx ctx = nullptr;
+    CUdevResource r;
+    if (!get_ctx || !get_resource || get_ctx(s, &ctx) != CUDA_SUCCESS || !ctx) return all;
+    if (get_resource(ctx, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS || r.sm.smCount < 1) return 1;
+    return std::min(all, int(r.sm.smCount));
 }
 
 namespace {

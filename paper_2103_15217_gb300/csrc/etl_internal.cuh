@@ -20,6 +20,11 @@ constexpr unsigned kFull = 0xffffffffu;
 // Number of SMs of the current device (cached per device).
 int num_sms();
 
+// Number of SMs the work of a stream can use: fewer than the device has if the stream belongs to a green
+// context. A cooperative grid must fit them: a larger one is refused at its launch, and replayed from a graph
+// it would wait for ever.
+int stream_sms(cudaStream_t s);
+
 // Caller-owned device memory. While an ArenaScope is active on the calling
 // thread, every device allocation the library makes (dev_alloc, and so
 // Workspace::get and the tables of an LCA handle) is carved from the arena

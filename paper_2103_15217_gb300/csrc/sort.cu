@@ -434,9 +434,9 @@ etl_status sort_heavy(const int32_t *par, int32_t n, const uint32_t *heavy, cons
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0) != cudaSuccess || per_sm < 1)
         return ETL_ECUDA;
-    // all that are resident at once, but no more than there are tiles
-    const int64_t tiles = ceil_div(n, kWarps * kWarp * R);
-    const int blocks = int(tiles < int64_t(num_sms()) * per_sm ? tiles : int64_t(num_sms()) * per_sm);
+    // all that are resident at once on the stream's SMs, but no more than there are tiles
+    const int64_t tiles = ceil_div(n, kWarps * kWarp * R), resident = int64_t(stream_sms(ws.stream())) * per_sm;
+    const int blocks = int(tiles < resident ? tiles : resident);
     int2 *buf0 = ws.get<int2>(n), *buf1 = ws.get<int2>(n);
     int32_t *ghist = ws.get<int32_t>(int64_t(kRadix) * (blocks + 1)), *totals = ghist + int64_t(kRadix) * blocks;
     if (!ws.ok()) return ETL_ENOMEM;
