@@ -123,8 +123,9 @@ __device__ __forceinline__ int64_t hook_chunk(int64_t c, int64_t nsuper, bool sp
 // finalizer, a bijection), or, where the component's label is to be its smallest vertex (BY_ID), by the id.
 // By ids a path whose vertices are numbered along it is hooked into one chain, and an edge that comes late
 // climbs it alone, 0.5 us for two steps. Whole calls, us, by ids and now: paths in order of 2^17 vertices 1170
-// to 2640 and 111, of 2^20 31700 and 254 (from their end 27700 and 257), a cycle of 2^14 4120 and 57. On the
-// easy graph of 2^22 vertices, whose labels are permuted, 1433 and 1442, on the hard one 1234 and 1196.
+// to 6690 and 89, of 2^20 31700 and 254 (from their end 27700 and 257), a cycle of 2^14 4120 and 58, a path of
+// 2^14, where no edge comes late, 48 and 58. On the easy graph of 2^22 vertices, whose labels are permuted, 1420
+// and 1428 (by ids the popular parents lie side by side), on the hard one 1222 and 1184.
 template <bool BY_ID>
 __device__ __forceinline__ uint32_t hook_key(int32_t v) {
     uint32_t h = uint32_t(v);
